@@ -96,7 +96,7 @@ int choose_shape(fstat_plan_s* p) {
   p->part_stride = n / 256 + 1;
   const int64_t tiles = ((int64_t)1 << l2) / p->sh.cols;
   if (tiles + 1 > p->part_stride) p->part_stride = tiles + 1;
-  p->z_stride = 2 * n;
+  p->z_stride = n;
   size_t o = 0;
   p->off_meta = o; o = align256(o + sizeof(TmplMeta) * ch);
   p->off_knots = o; o = align256(o + (size_t)p->rec_bytes * p->knot_stride * ch);
@@ -405,7 +405,7 @@ int fstat_compute(fstat_plan_t p, const float* x_h, const fstat_template* t, int
     if (e == cudaSuccess)
       e = timed(p, K_PERSIST, s, [&] {
         return launch_persist(p->pc, c, x, gaps, p->wcs, &p->twf, twoF, p->status,
-                              reinterpret_cast<float2*>(p->ws + p->off_z), p->z_stride, pcnt,
+                              p->ws + p->off_z, p->z_stride, pcnt,
                               reinterpret_cast<int*>(p->ws + p->off_sched),
                               reinterpret_cast<int*>(p->ws + p->off_tcnt), limit, stall, s);
       });

@@ -18,8 +18,8 @@ namespace fs {
 namespace {
 template <typename R, int L1, int SRC, int TAPS>
 cudaError_t run(const ColsArgs<R>& a, dim3 grid, cudaStream_t s) {
-  constexpr int C = cols_for<R>(L1);
-  constexpr int NT = threads_for<R>(L1, 2 * C);
+  constexpr int C = cols_for<points_a<R>()>(L1);
+  constexpr int NT = threads_for<R>(L1, C);
   constexpr size_t SM = cols_smem<R, L1, C>();
   auto kern = k_cols<R, L1, C, NT, SRC, TAPS>;
   // persistent grid: the blocks that fit on the device at once
@@ -44,6 +44,6 @@ cudaError_t FS_CAT(cols, FS_REAL, FS_L1)(const ColsArgs<FS_REAL>& a, int src, in
   if (taps8) return run<FS_REAL, FS_L1, SRC_SINC, 8>(a, grid, s);
   return run<FS_REAL, FS_L1, SRC_SINC, 0>(a, grid, s);
 }
-int FS_CAT(colsC, FS_REAL, FS_L1)() { return cols_for<FS_REAL>(FS_L1); }
+int FS_CAT(colsC, FS_REAL, FS_L1)() { return cols_for<points_a<FS_REAL>()>(FS_L1); }
 
 }  // namespace fs

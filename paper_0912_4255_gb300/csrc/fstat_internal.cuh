@@ -88,6 +88,12 @@ template <> struct Cx<float> { using T = float2; };
 template <> struct Cx<double> { using T = double2; };
 template <typename R> using cpx = typename Cx<R>::T;
 
+// One element of both series, w_a and w_b side by side: the two transforms
+// take the same indices and twiddles, so every thread carries both, one
+// 16-byte access (FP32) moves a value of each and a twiddle is fetched (or
+// formed) once for the two.
+template <typename R> struct alignas(16) Pair { cpx<R> a, b; };
+
 template <typename R> struct KnotOf;
 template <> struct KnotOf<float> { using T = KnotF; };
 template <> struct KnotOf<double> { using T = KnotD; };
@@ -783,14 +789,14 @@ struct Dft {
 // padded shared-memory index: one extra element every 16 avoids bank
 // conflicts of the stride-16 writes of the first radix-16 stage
 __device__ __forceinline__ int pidx(int e) { return e + (e >> 4); }
-// Sequence stride in shared memory.  Fills and epilogues interleave C
-// sequences across the lanes of a half-warp (16 lanes of 8-byte accesses);
-// a stride congruent to 16/C mod 16 puts them on distinct banks.
+// Sequence stride in shared memory, in pairs.  Fills and epilogues interleave
+// C sequences across the lanes of a quarter-warp (8 lanes of 16-byte
+// accesses); a stride congruent to 8/C mod 8 puts them on distinct banks.
 template <int LOGN, int C> struct FftGeom {
   static constexpr int N = 1 << LOGN;
   static constexpr int BASE = N + (N >> 4);
-  static constexpr int WANT = C >= 16 ? 1 : 16 / C;
-  static constexpr int STRIDE = BASE + ((WANT - (BASE & 15)) & 15);
+  static constexpr int WANT = C >= 8 ? 1 : 8 / C;
+  static constexpr int STRIDE = BASE + ((WANT - (BASE & 7)) & 7);
 };
 
 // Twiddles of the Stockham stages, held in shared memory.  The stage of
@@ -827,14 +833,39 @@ __device__ __forceinline__ void build_mid_tw(cpx<R>* __restrict__ dst, const cpx
     build_mid_tw<R, LOGN, NSL + RB, NSL_END, NT>(dst + stage_tw_count<NSL, RB>(), tw);
   }
 }
+// The last stage (radix 2^RB at NS = 2^NSL, LOGN = NSL + RB) keeps only the
+// powers W^k, W^{2k}, W^{4k}, ...: row p holds W_{2^LOGN}^{2^p k}, k < NS.  A
+// thread forms the others as products, once for both series: the rows in
+// full would take 30 KB of shared memory and 15 loads at radix 16.
+template <int NSL, int RB> constexpr int last_tw_count() { return RB << NSL; }
+template <typename R, int LOGN, int NSL, int RB, int NT>
+__device__ __forceinline__ void build_last_tw(cpx<R>* __restrict__ dst, const cpx<R>* __restrict__ tw) {
+  static_assert(LOGN == NSL + RB, "the last stage completes the transform");
+  for (int e = threadIdx.x; e < last_tw_count<NSL, RB>(); e += NT) {
+    const int p = e >> NSL, k = e & ((1 << NSL) - 1);
+    dst[e] = __ldg(tw + (k << p));
+  }
+}
+// t[q] = first * W^{q k}, q < 2^RB, from the rows of build_last_tw (lt points
+// at column k): one product each, at most RB deep.
+template <typename R, int NSL, int RB>
+__device__ __forceinline__ void last_twiddles(const cpx<R>* __restrict__ lt, cpx<R> first, cpx<R>* __restrict__ t) {
+  t[0] = first;
+#pragma unroll
+  for (int p = 0; p < RB; ++p) {
+    const cpx<R> w = lt[p << NSL];
+#pragma unroll
+    for (int q = 0; q < (1 << p); ++q) t[(1 << p) + q] = cmul(t[q], w);
+  }
+}
 
-// One Stockham stage of radix 2^RB over COUNT sequences of length 2^LOGN in
-// shared memory (sequence f at buf + f * STRIDE, padded); NS = 2^NSL is the
-// length of the sub-transforms already done; tws: this stage's twiddle table.
-// Every thread handles UPT units of 16 points; all reads happen before the
-// barrier, all writes after it.
+// One Stockham stage of radix 2^RB over COUNT pairs of sequences of length
+// 2^LOGN in shared memory (pair f at buf + f * STRIDE, padded); NS = 2^NSL is
+// the length of the sub-transforms already done; tws: this stage's twiddle
+// table.  Every thread handles UPT units of 16 points of both series; all
+// reads happen before the barrier, all writes after it.
 template <typename R, int LOGN, int RB, int NSL, int NT, int COUNT, int STRIDE>
-__device__ __forceinline__ void stockham_stage(cpx<R>* __restrict__ buf, const cpx<R>* __restrict__ tws) {
+__device__ __forceinline__ void stockham_stage(Pair<R>* __restrict__ buf, const cpx<R>* __restrict__ tws) {
   using C = cpx<R>;
   constexpr int N = 1 << LOGN;
   constexpr int RAD = 1 << RB;
@@ -843,25 +874,34 @@ __device__ __forceinline__ void stockham_stage(cpx<R>* __restrict__ buf, const c
   constexpr int UNITS = COUNT * UNITS_PER_SEQ;
   constexpr int UPT = (UNITS + NT - 1) / NT;
   constexpr int NS = 1 << NSL;
-  C v[UPT][16];
+  C va[UPT][16], vb[UPT][16];
 #pragma unroll
   for (int u = 0; u < UPT; ++u) {
     const int unit = threadIdx.x + u * NT;
     if (UNITS % NT == 0 || unit < UNITS) {
       const int f = unit / UNITS_PER_SEQ;
       const int w = unit - f * UNITS_PER_SEQ;
-      const C* src = buf + f * STRIDE;
+      const Pair<R>* src = buf + f * STRIDE;
 #pragma unroll
       for (int bb = 0; bb < BPU; ++bb) {
         const int j = w + bb * UNITS_PER_SEQ;     // lanes take consecutive butterflies
         const int k = j & (NS - 1);
 #pragma unroll
-        for (int r = 0; r < RAD; ++r) v[u][bb * RAD + r] = src[pidx(j + r * (N / RAD))];
-        if constexpr (NSL > 0) {
-#pragma unroll
-          for (int r = 1; r < RAD; ++r) v[u][bb * RAD + r] = cmul(v[u][bb * RAD + r], tws[((r - 1) << NSL) + k]);
+        for (int r = 0; r < RAD; ++r) {
+          const Pair<R> x = src[pidx(j + r * (N / RAD))];
+          C xa = x.a, xb = x.b;
+          if constexpr (NSL > 0) {
+            if (r > 0) {
+              const C t = tws[((r - 1) << NSL) + k];
+              xa = cmul(xa, t);
+              xb = cmul(xb, t);
+            }
+          }
+          va[u][bb * RAD + r] = xa;
+          vb[u][bb * RAD + r] = xb;
         }
-        Dft<C, RAD>::run(&v[u][bb * RAD]);
+        Dft<C, RAD>::run(&va[u][bb * RAD]);
+        Dft<C, RAD>::run(&vb[u][bb * RAD]);
       }
     }
   }
@@ -872,14 +912,14 @@ __device__ __forceinline__ void stockham_stage(cpx<R>* __restrict__ buf, const c
     if (UNITS % NT == 0 || unit < UNITS) {
       const int f = unit / UNITS_PER_SEQ;
       const int w = unit - f * UNITS_PER_SEQ;
-      C* dst = buf + f * STRIDE;
+      Pair<R>* dst = buf + f * STRIDE;
 #pragma unroll
       for (int bb = 0; bb < BPU; ++bb) {
         const int j = w + bb * UNITS_PER_SEQ;
         const int k = j & (NS - 1);
         const int base = ((j >> NSL) << (NSL + RB)) + k;
 #pragma unroll
-        for (int r = 0; r < RAD; ++r) dst[pidx(base + r * NS)] = v[u][bb * RAD + r];
+        for (int r = 0; r < RAD; ++r) dst[pidx(base + r * NS)] = Pair<R>{va[u][bb * RAD + r], vb[u][bb * RAD + r]};
       }
     }
   }
@@ -890,12 +930,28 @@ __device__ __forceinline__ void stockham_stage(cpx<R>* __restrict__ buf, const c
 // possible); the stages before and after are done by the caller.  tws: the
 // tables of these stages, one after the other (build_mid_tw).
 template <typename R, int LOGN, int NSL, int NSL_END, int NT, int COUNT, int STRIDE>
-__device__ __forceinline__ void fft_mid_stages(cpx<R>* buf, const cpx<R>* tws) {
+__device__ __forceinline__ void fft_mid_stages(Pair<R>* buf, const cpx<R>* tws) {
   if constexpr (NSL < NSL_END) {
     constexpr int RB = mid_rb<NSL, NSL_END>();
     stockham_stage<R, LOGN, RB, NSL, NT, COUNT, STRIDE>(buf, tws);
     fft_mid_stages<R, LOGN, NSL + RB, NSL_END, NT, COUNT, STRIDE>(buf, tws + stage_tw_count<NSL, RB>());
   }
+}
+
+// streaming access to one pair (both planes of an FP32 pair in 16 bytes)
+__device__ __forceinline__ Pair<float> ldcs(const Pair<float>* p) {
+  const float4 v = __ldcs(reinterpret_cast<const float4*>(p));
+  return Pair<float>{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ Pair<double> ldcs(const Pair<double>* p) {
+  return Pair<double>{__ldcs(&p->a), __ldcs(&p->b)};
+}
+__device__ __forceinline__ void stcs(Pair<float>* p, const Pair<float>& v) {
+  __stcs(reinterpret_cast<float4*>(p), make_float4(v.a.x, v.a.y, v.b.x, v.b.y));
+}
+__device__ __forceinline__ void stcs(Pair<double>* p, const Pair<double>& v) {
+  __stcs(&p->a, v.a);
+  __stcs(&p->b, v.b);
 }
 
 // exp(-2 pi i m / 2^L) from the two-level tables
@@ -980,9 +1036,9 @@ struct Chunk {
   double* partials;       // [nt][part_stride][3]
   int64_t part_stride;
   int* counters;          // [nt]
-  void* za;               // FFT intermediate [nt][2][n] complex (a plane, b plane)
-  int64_t z_stride;       // complex elements per template (2 n)
-  void* wa;               // unfused path: resampled series [nt][2][n], column-tiled
+  void* za;               // FFT intermediate [nt][n] pairs
+  int64_t z_stride;       // pairs per template (n)
+  void* wa;               // unfused path: resampled series [nt][n] pairs, column-tiled
   int nt;
 };
 
@@ -1041,7 +1097,7 @@ int cols_per_block(int precision, int l1);
 int persist_slots();
 size_t persist_smem();
 cudaError_t launch_persist(const PlanConst& pc, const Chunk& c, const float2* x, const int64_t* gaps,
-                           const double* wcs, const void* twf, float* out, int* status, float2* zslots,
+                           const double* wcs, const void* twf, float* out, int* status, void* zslots,
                            int64_t z_stride, int* counters, int* sched, int* cnt, int spin_limit,
                            int stall_template, cudaStream_t s);
 int rows_per_block(int precision, int l2);

@@ -241,7 +241,7 @@ extern "C" int fstat_compute_noalloc(const fstat_plan_desc* d, const float* x_h,
     c.part_stride = kNaParts;
     c.counters = reinterpret_cast<int*>(base + kOffCnt);
     c.za = base + kOffZ;
-    c.z_stride = 2 * d->n_fft;
+    c.z_stride = d->n_fft;
     c.wa = nullptr;
     c.nt = 1;
     // the block counters must start at zero for every template

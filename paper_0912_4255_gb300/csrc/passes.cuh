@@ -5,14 +5,16 @@
 //
 // N = N1 N2, k = k2 + N2 k1, p = p1 + N1 p2:
 //   X[p1 + N1 p2] = sum_k2 W_N2^{p2 k2} W_N^{p1 k2} sum_k1 x[k2 + N2 k1] W_N1^{p1 k1}.
-// Pass A (columns): a block owns C consecutive columns k2 of both series
-// (w_a, w_b), produces their samples (resampled on the fly, or loaded),
-// runs the N1-point FFTs over k1 in shared memory, multiplies by
-// W_N^{p1 k2} and stores into Z laid out as Z[p1 / RR][k2][p1 % RR].
+// Both series (w_a, w_b) travel together, a Pair per point, in memory, in
+// shared memory and in a thread's registers.
+// Pass A (columns): a block owns C consecutive columns k2, produces their
+// samples (resampled on the fly, or loaded), runs the N1-point FFTs over k1
+// in shared memory, multiplies by W_N^{p1 k2} and stores into Z laid out as
+// Z[p1 / RR][k2][p1 % RR].
 // Pass B (rows): a block owns the RR consecutive rows p1 of one row block,
-// which are one contiguous run of N2 * RR values per series; it runs the
-// N2-point FFTs over k2 and writes 2F for every (p1, p2) at the
-// ascending-frequency position q = p1 + N1 ((p2 + N2/2) mod N2).
+// which are one contiguous run of N2 * RR pairs; it runs the N2-point FFTs
+// over k2 and writes 2F for every (p1, p2) at the ascending-frequency
+// position q = p1 + N1 ((p2 + N2/2) mod N2).
 #pragma once
 
 #include "fstat_internal.cuh"
@@ -56,23 +58,36 @@ struct RowsArgs {
 
 // --------------------------------------------------------------- shapes
 
-// Points per block (both series): 16k complex values in FP32 (128 KB of
-// shared memory, one block of 1024 threads per SM; at N = 2^22 a first-pass
-// block's C = 2 columns and a second-pass block's R = 8 rows give Z runs of
-// R C values = 128 B and 2F runs of R values = 32 B), 4k in FP64 (two blocks
-// per SM); at most 16 columns (rows) per block.  P: the points of a block.
-template <typename R> constexpr int points_per_block() { return std::is_same<R, float>::value ? 16384 : 4096; }
-template <typename R, int P = points_per_block<R>()> constexpr int cols_for(int L1) {
+// Points per block (both series), at most 16 columns (rows) per block.
+// Pass A, FP32: 8k, so that the longest first pass (N1 = 2^12) is one column
+// pair of 68 KB, 256 threads of 16 points of each series, and two
+// independent blocks share an SM: one loads or stores while the other
+// computes.  Pass B, FP32: 16k (one block of 512 threads per SM), because
+// its 2F leaves in runs of R values and R = 8 rows at N = 2^22 fill a 32-byte
+// sector (runs of 4 measured 1.25 times the time).  FP64: 4k, bound by the
+// FP64 pipe at any size.
+template <typename R> constexpr int points_a() { return std::is_same<R, float>::value ? 8192 : 4096; }
+template <typename R> constexpr int points_b() { return std::is_same<R, float>::value ? 16384 : 4096; }
+template <int P> constexpr int cols_for(int L1) {
   const int c = (P / 2) >> L1;
   return c > 16 ? 16 : (c < 1 ? 1 : c);
 }
+// one thread per 16 points of both series
 template <typename R> constexpr int threads_for(int logn, int count) {
   const int units = (count << logn) / 16;
-  return units >= 1024 ? 1024 : (units < 32 ? 32 : units);
+  return units >= 512 ? 512 : (units < 32 ? 32 : units);
+}
+// Blocks per SM to compile for: 512 threads of 128 registers (FP64: 256 of
+// 255), as far as shared memory allows.
+template <typename R> constexpr int min_blocks(int nt, size_t smem) {
+  const int by_regs = (std::is_same<R, float>::value ? 512 : 256) / nt;
+  const int by_smem = (int)((220 * 1024) / smem);
+  const int b = by_regs < by_smem ? by_regs : by_smem;
+  return b < 1 ? 1 : b;
 }
 // Stage plan of pass A: shared-memory stages up to sub-transforms of 2^NSL_LAST,
-// then a last stage of radix 2^RBL in registers.  Its shared memory: both
-// series of C columns, the stage twiddle tables, and the two factors of the
+// then a last stage of radix 2^RBL in registers.  Its shared memory: C
+// column pairs, the stage twiddle tables, and the two factors of the
 // inter-pass twiddle W_N^{p1 k2} = W_N^{j k2} W_N^{q NS k2} (p1 = j + q NS)
 // for the block's C columns.
 template <int L1> struct PlanA {
@@ -81,49 +96,53 @@ template <int L1> struct PlanA {
   static constexpr int RADL = 1 << RBL;
   static constexpr int NS = (1 << L1) / RADL;
   static constexpr int MID_TW = mid_tw_count<0, NSL_LAST>();
-  static constexpr int LAST_TW = stage_tw_count<NSL_LAST, RBL>();
+  static constexpr int LAST_TW = last_tw_count<NSL_LAST, RBL>();
 };
 // Pass B: a first radix-16 stage from global memory, shared-memory stages,
-// a last stage of radix <= 8 in registers.
+// a last stage in registers: radix 16 at N2 = 2^8 and 2^12, which leaves one
+// (two) shared-memory exchanges instead of a further radix-2 one, else at
+// most 8.
 template <int L2> struct PlanB {
   static constexpr int RB0 = 4;
-  static constexpr int RBL = L2 - RB0 >= 3 ? 3 : L2 - RB0;
+  static constexpr int RBL = L2 == 8 || L2 == 12 ? 4 : (L2 - RB0 >= 3 ? 3 : L2 - RB0);
   static constexpr int NSL_LAST = L2 - RBL;
   static constexpr int RADL = 1 << RBL;
   static constexpr int NS = (1 << L2) / RADL;
   static constexpr int MID_TW = mid_tw_count<RB0, NSL_LAST>();
-  static constexpr int LAST_TW = stage_tw_count<NSL_LAST, RBL>();
+  static constexpr int LAST_TW = last_tw_count<NSL_LAST, RBL>();
 };
 template <typename R, int L1, int C> constexpr size_t cols_smem() {
   using P = PlanA<L1>;
-  return ((size_t)2 * C * FftGeom<L1, C>::STRIDE + P::MID_TW + P::LAST_TW + (size_t)C * (P::NS + P::RADL)) *
-         sizeof(cpx<R>);
+  return (size_t)C * FftGeom<L1, C>::STRIDE * sizeof(Pair<R>) +
+         (size_t)(P::MID_TW + P::LAST_TW + C * (P::NS + P::RADL)) * sizeof(cpx<R>);
 }
 template <typename R, int L2, int RR> constexpr size_t rows_smem() {
   using P = PlanB<L2>;
-  return ((size_t)2 * RR * FftGeom<L2, RR>::STRIDE + P::MID_TW + P::LAST_TW) * sizeof(cpx<R>);
+  return (size_t)RR * FftGeom<L2, RR>::STRIDE * sizeof(Pair<R>) + (size_t)(P::MID_TW + P::LAST_TW) * sizeof(cpx<R>);
 }
-// two blocks per SM when their shared memory allows it
-constexpr int blocks_for_smem(size_t bytes) { return bytes <= 110 * 1024 ? 2 : 1; }
 
 // --------------------------------------------------------------- pass A
 
 // Stage twiddle tables of pass A, the same for every tile of one shape
 // (all threads of the block; read after a barrier).
 template <typename R, int L1, int C, int NT>
-__device__ __forceinline__ void cols_tables(const Tw<R>& tw, cpx<R>* buf) {
+__device__ __forceinline__ void cols_tables(const Tw<R>& tw, Pair<R>* buf) {
   using PA = PlanA<L1>;
-  cpx<R>* tws = buf + 2 * C * FftGeom<L1, C>::STRIDE;
+  cpx<R>* tws = reinterpret_cast<cpx<R>*>(buf + C * FftGeom<L1, C>::STRIDE);
   build_mid_tw<R, L1, 0, PA::NSL_LAST, NT>(tws, tw.tl[L1]);
-  build_stage_tw<R, L1, PA::NSL_LAST, PA::RBL, NT>(tws + PA::MID_TW, tw.tl[L1]);
+  build_last_tw<R, L1, PA::NSL_LAST, PA::RBL, NT>(tws + PA::MID_TW, tw.tl[L1]);
 }
 
 // One column tile of pass A for template t (all threads of the block; the
-// stage tables from cols_tables).  za: this template's intermediate (a
-// plane; the b plane follows at +N).
+// stage tables from cols_tables).  za: this template's intermediate.
+//
+// Per point of a series (N1 = 2^12) the three radix-16 stages are about 50
+// FP32 instructions; carrying both series in one thread halves what is
+// around them: twiddle loads and products, addresses, and the load, store
+// and shared-memory instructions (16 bytes each instead of 8).
 template <typename R, int L1, int C, int NT, int SRC, int TAPS>
-__device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile, cpx<R>* __restrict__ buf,
-                                          double* red, cpx<R>* __restrict__ za, int RRr, int lr) {
+__device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile, Pair<R>* __restrict__ buf,
+                                          double* red, Pair<R>* __restrict__ za, int RRr, int lr) {
   using Cx = cpx<R>;
   using Knot = typename KnotOf<R>::T;
   constexpr int N1 = 1 << L1;
@@ -136,24 +155,16 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
   const int n_b = (int)m.n_b;
   const Knot* kn = reinterpret_cast<const Knot*>(a.c.knots) + (int64_t)t * a.c.knot_stride;
   R pA = 0, pB = 0, pC = 0;
-  const Cx* wa_in = nullptr;
-  const Cx* wb_in = nullptr;
-  if constexpr (SRC == SRC_LOAD) {
-    // the tiled resampler's order W[k2 / C][k1][k2 % C]: this tile's C * N1
-    // points of each series are contiguous, point i = c + C k1 at offset i
-    wa_in = reinterpret_cast<const Cx*>(a.c.wa) + (int64_t)t * a.c.z_stride + (int64_t)tile * (C * N1);
-    wb_in = wa_in + ((int64_t)1 << L);
-  }
   // twiddle tables (cols_tables); this tile's inter-pass factors are
   // written here and read after the barriers that end the fill
   using PA = PlanA<L1>;
   constexpr int NSL_LAST = PA::NSL_LAST;
   constexpr int RADL = PA::RADL;
   constexpr int NS = PA::NS;
-  cpx<R>* tws = buf + 2 * C * STRIDE;     // shared-memory stages
-  cpx<R>* tlast = tws + PA::MID_TW;       // last stage, [q - 1][j]
-  cpx<R>* ta = tlast + PA::LAST_TW;       // [c][j]: W_N^{j (c0 + c)}, j < NS
-  cpx<R>* tb = ta + C * NS;               // [c][q]: W_N^{q NS (c0 + c)}, q < RADL
+  Cx* tws = reinterpret_cast<Cx*>(buf + C * STRIDE);   // shared-memory stages
+  Cx* tlast = tws + PA::MID_TW;           // last stage, rows of powers
+  Cx* ta = tlast + PA::LAST_TW;           // [c][j]: W_N^{j (c0 + c)}, j < NS
+  Cx* tb = ta + C * NS;                   // [c][q]: W_N^{q NS (c0 + c)}, q < RADL
   for (int e = threadIdx.x; e < C * (NS + RADL); e += NT) {
     if (e < C * NS) {
       const int c = e / NS, j = e - c * NS;
@@ -165,28 +176,37 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
     }
   }
   if constexpr (SRC == SRC_LOAD) {
+    // the tiled resampler's order W[k2 / C][k1][k2 % C]: this tile's C * N1
+    // pairs are contiguous, pair i = c + C k1 at offset i
+    const Pair<R>* w_in = reinterpret_cast<const Pair<R>*>(a.c.wa) + (int64_t)t * a.c.z_stride +
+                          (int64_t)tile * (C * N1);
     // first radix-16 stage straight from the resampled series: unit
-    // (series, j, column) with the column fastest, so that the lanes of a
+    // (j, column) with the column fastest, so that the lanes of a
     // warp read consecutive values; outputs in the order of a first
     // Stockham stage (sub-transforms of length 16 at 16 j)
     constexpr int Q1 = N1 / 16;
 #pragma unroll 1
-    for (int u = threadIdx.x; u < 2 * C * Q1; u += NT) {
+    for (int u = threadIdx.x; u < C * Q1; u += NT) {
       const int c = u & (C - 1);
-      const int rest = u / C;
-      const int j = rest & (Q1 - 1);
-      const int sr = rest / Q1;
-      const Cx* src = (sr ? wb_in : wa_in) + c;
-      Cx v[16];
+      const int j = u / C;
+      const Pair<R>* src = w_in + c + j * C;
+      // points k = c0 + c + (j + r Q1) N2 < n_b: r below nr
+      const int step = Q1 * N2;                        // N / 16
+      const int left = n_b - (c0 + c + j * N2);
+      const int nr = left > 0 ? (left + step - 1) >> (L - 4) : 0;
+      Cx va[16], vb[16];
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
-        const int k1 = j + r * Q1;
-        v[r] = c0 + c + k1 * N2 < n_b ? __ldcs(src + k1 * C) : czero<Cx>();
+        Pair<R> v{czero<Cx>(), czero<Cx>()};
+        if (r < nr) v = ldcs(src + r * (Q1 * C));
+        va[r] = v.a;
+        vb[r] = v.b;
       }
-      Dft<Cx, 16>::run(v);
-      Cx* dst = buf + (sr * C + c) * STRIDE;
+      Dft<Cx, 16>::run(va);
+      Dft<Cx, 16>::run(vb);
+      Pair<R>* dst = buf + c * STRIDE + pidx(16 * j);
 #pragma unroll
-      for (int r = 0; r < 16; ++r) dst[pidx(16 * j + r)] = v[r];
+      for (int r = 0; r < 16; ++r) dst[r] = Pair<R>{va[r], vb[r]};
     }
   } else {
     GapCursor gc = make_cursor(m, a.gaps);
@@ -203,8 +223,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
           pA += aa * aa; pB += bb * bb; pC += aa * bb;
         }
       }
-      buf[c * STRIDE + pidx(k1)] = va;
-      buf[(C + c) * STRIDE + pidx(k1)] = vb;
+      buf[c * STRIDE + pidx(k1)] = Pair<R>{va, vb};
     }
   }
   if constexpr (SRC != SRC_LOAD) {
@@ -220,50 +239,44 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
   // all stages but the last in shared memory (the first one done above when
   // loading; it needs no twiddles, so the tables start at the same place)
   static_assert(stage_tw_count<0, 4>() == 0, "first stage without twiddles");
-  fft_mid_stages<R, L1, SRC == SRC_LOAD ? 4 : 0, NSL_LAST, NT, 2 * C, STRIDE>(buf, tws);
+  fft_mid_stages<R, L1, SRC == SRC_LOAD ? 4 : 0, NSL_LAST, NT, C, STRIDE>(buf, tws);
   // last stage: inputs from shared memory, outputs X[p1 = j + q NS] stay in
-  // registers, are multiplied by W_N^{p1 k2} and stored into Z.  Lanes run
-  // over j mod RR, then the column, then j / RR, so that a warp writes runs
-  // of RR * C consecutive values of Z.
-  constexpr int PER_S = C * NS;
-  Cx* zb = za + ((int64_t)1 << L);
+  // registers, are multiplied by W_N^{p1 k2} and stored into Z.  Of that
+  // twiddle the factor W_N^{j k2} is common to a butterfly's outputs, so it
+  // joins the stage twiddles of the inputs (t[q] = W_N^{j k2} W_N1^{q j}) and
+  // only W_N^{q NS k2} multiplies the outputs.  Lanes run over j mod RR, then
+  // the column, then j / RR, so that a warp writes runs of RR * C
+  // consecutive pairs of Z.
 #pragma unroll 1
-  for (int u = threadIdx.x; u < 2 * PER_S; u += NT) {
-    const int sr = u >= PER_S;
-    const int v = u - sr * PER_S;
-    const int jr = v & (RRr - 1);
-    const int rest = v >> lr;
+  for (int u = threadIdx.x; u < C * NS; u += NT) {
+    const int jr = u & (RRr - 1);
+    const int rest = u >> lr;
     const int c = rest & (C - 1);
     const int j = ((rest / C) << lr) + jr;
-    const int f = sr * C + c;
-    Cx x[RADL];
-#pragma unroll
-    for (int q = 0; q < RADL; ++q) x[q] = buf[f * STRIDE + pidx(j + q * NS)];
+    Cx xa[RADL], xb[RADL];
     {
-      // the stage twiddles W^(q j): the powers q = 1, 2, 4, 8 from the table,
-      // the others as products of at most three of them (shared-memory
-      // bandwidth, not arithmetic, limits this pass)
-      Cx wp[RADL];
-      wp[1] = tlast[j];
+      Cx tq[RADL];
+      last_twiddles<R, NSL_LAST, PA::RBL>(tlast + j, ta[c * NS + j], tq);
+      const Pair<R>* src = buf + c * STRIDE + pidx(j);
 #pragma unroll
-      for (int q = 2; q < RADL; ++q) {
-        if ((q & (q - 1)) == 0) wp[q] = tlast[(q - 1) * NS + j];
-        else { const int hb = (q & 8) ? 8 : ((q & 4) ? 4 : 2); wp[q] = cmul(wp[hb], wp[q - hb]); }
+      for (int q = 0; q < RADL; ++q) {
+        const Pair<R> v = src[q * (NS + NS / 16)];     // pidx(j + q NS): NS is a multiple of 16
+        xa[q] = cmul(v.a, tq[q]);
+        xb[q] = cmul(v.b, tq[q]);
       }
-#pragma unroll
-      for (int q = 1; q < RADL; ++q) x[q] = cmul(x[q], wp[q]);
     }
-    Dft<Cx, RADL>::run(x);
+    Dft<Cx, RADL>::run(xa);
+    Dft<Cx, RADL>::run(xb);
     const int k2 = c0 + c;
     // p1 = j + q NS lands at Z[p1 / R][k2][p1 % R]; NS is a multiple of R, so
     // consecutive q are N / RADL elements apart
-    Cx* zq = (sr ? zb : za) + ((((int64_t)(j >> lr) * N2 + k2) << lr) + (j & (RRr - 1)));
+    Pair<R>* zq = za + ((((int64_t)(j >> lr) * N2 + k2) << lr) + (j & (RRr - 1)));
     const int64_t zstep = ((int64_t)1 << L) / RADL;
-    const Cx wj = ta[c * NS + j];
 #pragma unroll
     for (int q = 0; q < RADL; ++q) {
-      const Cx w = q == 0 ? wj : cmul(wj, tb[c * RADL + q]);
-      zq[q * zstep] = cmul(x[q], w);
+      const Cx w = tb[c * RADL + q];
+      *zq = q == 0 ? Pair<R>{xa[q], xb[q]} : Pair<R>{cmul(xa[q], w), cmul(xb[q], w)};
+      zq += zstep;
     }
   }
 }
@@ -271,10 +284,10 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
 // Persistent over the (template, column tile) items of a chunk: the grid is
 // sized to the resident blocks, each builds the stage tables once.
 template <typename R, int L1, int C, int NT, int SRC, int TAPS>
-__global__ void __launch_bounds__(NT, (blocks_for_smem(cols_smem<R, L1, C>()))) k_cols(ColsArgs<R> a) {
+__global__ void __launch_bounds__(NT, (min_blocks<R>(NT, cols_smem<R, L1, C>()))) k_cols(ColsArgs<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[96];
-  cpx<R>* buf = reinterpret_cast<cpx<R>*>(smem_raw);
+  Pair<R>* buf = reinterpret_cast<Pair<R>*>(smem_raw);
   cols_tables<R, L1, C, NT>(a.tw, buf);
   const int nt = a.ti >= 0 ? 1 : a.c.nt;
   const int total = a.tiles_max * nt;
@@ -285,8 +298,7 @@ __global__ void __launch_bounds__(NT, (blocks_for_smem(cols_smem<R, L1, C>()))) 
     const int t = a.ti >= 0 ? a.ti : tq;
     const TmplMeta& m = a.c.meta[t];
     if constexpr (SRC == SRC_LOAD) {
-      // the rows below n_b of the next tile's resampled block, into L2 (one
-      // block per SM: nothing else hides the latency of the first stage)
+      // the rows below n_b of the next tile's resampled block, into L2
       const int wn = w + gridDim.x;
       if (threadIdx.x == 0 && wn < total) {
         const int tqn = wn / a.tiles_max;
@@ -297,18 +309,15 @@ __global__ void __launch_bounds__(NT, (blocks_for_smem(cols_smem<R, L1, C>()))) 
         if (mn.status == FSTAT_OK && tilen < (1 << (ln - L1)) / C) {
           const int64_t first = (int64_t)tilen * C;                        // c0 of that tile
           const int64_t rows = mn.n_b > first ? (mn.n_b - first + (1 << (ln - L1)) - 1) >> (ln - L1) : 0;
-          const unsigned bytes = (unsigned)((rows < (1 << L1) ? rows : (1 << L1)) * C * sizeof(cpx<R>));
-          if (bytes >= 16) {
-            const cpx<R>* pa = reinterpret_cast<const cpx<R>*>(a.c.wa) + (int64_t)tn * a.c.z_stride +
-                               first * (1 << L1);
-            prefetch_l2(pa, bytes & ~15u);
-            prefetch_l2(pa + ((int64_t)1 << ln), bytes & ~15u);
-          }
+          const unsigned bytes = (unsigned)((rows < (1 << L1) ? rows : (1 << L1)) * C * sizeof(Pair<R>));
+          if (bytes >= 16)
+            prefetch_l2(reinterpret_cast<const Pair<R>*>(a.c.wa) + (int64_t)tn * a.c.z_stride + first * (1 << L1),
+                        bytes);
         }
       }
     }
     if (tile >= (1 << (m.log2n - L1)) / C || m.status != FSTAT_OK) continue;
-    cpx<R>* za = reinterpret_cast<cpx<R>*>(a.c.za) + (int64_t)t * a.c.z_stride;
+    Pair<R>* za = reinterpret_cast<Pair<R>*>(a.c.za) + (int64_t)t * a.c.z_stride;
     cols_tile<R, L1, C, NT, SRC, TAPS>(a, t, tile, buf, red, za, a.rr, a.log2rr);
     __syncthreads();                      // the next tile reuses buf and its twiddle factors
   }
@@ -318,11 +327,11 @@ __global__ void __launch_bounds__(NT, (blocks_for_smem(cols_smem<R, L1, C>()))) 
 
 // Stage twiddle tables of pass B (all threads of the block; read after a barrier).
 template <typename R, int L2, int RR, int NT>
-__device__ __forceinline__ void rows_tables(const Tw<R>& tw, cpx<R>* buf) {
+__device__ __forceinline__ void rows_tables(const Tw<R>& tw, Pair<R>* buf) {
   using PB = PlanB<L2>;
-  cpx<R>* tws = buf + 2 * RR * FftGeom<L2, RR>::STRIDE;
+  cpx<R>* tws = reinterpret_cast<cpx<R>*>(buf + RR * FftGeom<L2, RR>::STRIDE);
   build_mid_tw<R, L2, PB::RB0, PB::NSL_LAST, NT>(tws, tw.tl[L2]);
-  build_stage_tw<R, L2, PB::NSL_LAST, PB::RBL, NT>(tws + PB::MID_TW, tw.tl[L2]);
+  build_last_tw<R, L2, PB::NSL_LAST, PB::RBL, NT>(tws + PB::MID_TW, tw.tl[L2]);
 }
 
 // One row block of pass B for template t (stage tables from rows_tables);
@@ -330,8 +339,8 @@ __device__ __forceinline__ void rows_tables(const Tw<R>& tw, cpx<R>* buf) {
 // BAND: the plan writes a partial output band (bins band_lo <= q < band_hi
 // only); without it every bin is stored, with no band test.
 template <typename R, int L2, int RR, int NT, bool BAND>
-__device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, cpx<R>* __restrict__ buf,
-                                          const cpx<R>* __restrict__ zbase) {
+__device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, Pair<R>* __restrict__ buf,
+                                          const Pair<R>* __restrict__ zbase) {
   using Cx = cpx<R>;
   constexpr int N2 = 1 << L2;
   constexpr int STRIDE = FftGeom<L2, RR>::STRIDE;
@@ -360,39 +369,39 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
     }
     return;
   }
-  // this block's rows are one contiguous run of N2 * RR values per series,
-  // element (k2, r) at k2 * RR + r.  First radix-16 stage straight from
-  // there: lanes run over r, then j, so the loads are contiguous.
-  const Cx* za = zbase + (int64_t)blk * N2 * RR;
-  const Cx* zb = za + ((int64_t)1 << L);
+  // this block's rows are one contiguous run of N2 * RR pairs, element
+  // (k2, r) at k2 * RR + r.  First radix-16 stage straight from there: lanes
+  // run over r, then j, so the loads are contiguous.
+  const Pair<R>* zr = zbase + (int64_t)blk * N2 * RR;
   using PB = PlanB<L2>;
-  Cx* tws = buf + 2 * RR * STRIDE;        // shared-memory stages (rows_tables)
-  Cx* tlast = tws + PB::MID_TW;           // last stage, [q - 1][j]
+  Cx* tws = reinterpret_cast<Cx*>(buf + RR * STRIDE);   // shared-memory stages (rows_tables)
+  Cx* tlast = tws + PB::MID_TW;           // last stage, rows of powers
   constexpr int RB0 = PB::RB0;
   constexpr int RAD0 = 1 << RB0;
   constexpr int Q0 = N2 / RAD0;                   // butterflies per sequence
-  constexpr int UNITS0 = 2 * RR * Q0;
 #pragma unroll 1
-  for (int u = threadIdx.x; u < UNITS0; u += NT) {
-    const int sr = u >= RR * Q0;
-    const int v = u - sr * RR * Q0;
-    const int r = v & (RR - 1);
-    const int j = v / RR;
-    const Cx* src = (sr ? zb : za) + r;
-    Cx x[RAD0];
+  for (int u = threadIdx.x; u < RR * Q0; u += NT) {
+    const int r = u & (RR - 1);
+    const int j = u / RR;
+    const Pair<R>* src = zr + u;
+    Cx xa[RAD0], xb[RAD0];
 #pragma unroll
-    for (int q = 0; q < RAD0; ++q) x[q] = __ldcs(src + (j + q * Q0) * RR);
-    Dft<Cx, RAD0>::run(x);
-    Cx* dst = buf + (sr * RR + r) * STRIDE;
+    for (int q = 0; q < RAD0; ++q) {
+      const Pair<R> v = ldcs(src + q * (Q0 * RR));
+      xa[q] = v.a;
+      xb[q] = v.b;
+    }
+    Dft<Cx, RAD0>::run(xa);
+    Dft<Cx, RAD0>::run(xb);
+    Pair<R>* dst = buf + r * STRIDE + pidx(j * RAD0);
 #pragma unroll
-    for (int q = 0; q < RAD0; ++q) dst[pidx(j * RAD0 + q)] = x[q];
+    for (int q = 0; q < RAD0; ++q) dst[q] = Pair<R>{xa[q], xb[q]};
   }
   __syncthreads();
-  // middle stages in shared memory; the last stage (radix <= 8) pairs the
-  // a and b series of the same butterfly so that 2F is formed in registers
-  constexpr int RBL = PB::RBL;
+  // middle stages in shared memory; in the last stage both series of a
+  // butterfly are in one thread, so that 2F is formed in registers
   constexpr int NSL_LAST = PB::NSL_LAST;
-  fft_mid_stages<R, L2, RB0, NSL_LAST, NT, 2 * RR, STRIDE>(buf, tws);
+  fft_mid_stages<R, L2, RB0, NSL_LAST, NT, RR, STRIDE>(buf, tws);
   R ca, cb, cc;
   if constexpr (std::is_same<R, float>::value) {
     ca = m.ca; cb = m.cb; cc = m.cc;
@@ -408,16 +417,15 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
     const int r = u & (RR - 1);
     const int j = u / RR;
     Cx fa[RADL], fb[RADL];
+    {
+      Cx tq[RADL];
+      last_twiddles<R, NSL_LAST, PB::RBL>(tlast + j, cmk<Cx, R>((R)1, (R)0), tq);
 #pragma unroll
-    for (int q = 0; q < RADL; ++q) {
-      fa[q] = buf[r * STRIDE + pidx(j + q * NS)];
-      fb[q] = buf[(RR + r) * STRIDE + pidx(j + q * NS)];
-    }
-#pragma unroll
-    for (int q = 1; q < RADL; ++q) {
-      const Cx w = tlast[(q - 1) * NS + j];
-      fa[q] = cmul(fa[q], w);
-      fb[q] = cmul(fb[q], w);
+      for (int q = 0; q < RADL; ++q) {
+        const Pair<R> v = buf[r * STRIDE + pidx(j + q * NS)];
+        fa[q] = q == 0 ? v.a : cmul(v.a, tq[q]);
+        fb[q] = q == 0 ? v.b : cmul(v.b, tq[q]);
+      }
     }
     Dft<Cx, RADL>::run(fa);
     Dft<Cx, RADL>::run(fb);
@@ -440,9 +448,9 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
 
 // Persistent over the (template, row block) items of a chunk.
 template <typename R, int L2, int RR, int NT, bool BAND>
-__global__ void __launch_bounds__(NT, (blocks_for_smem(rows_smem<R, L2, RR>()))) k_rows(RowsArgs<R> a) {
+__global__ void __launch_bounds__(NT, (min_blocks<R>(NT, rows_smem<R, L2, RR>()))) k_rows(RowsArgs<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<R>* buf = reinterpret_cast<cpx<R>*>(smem_raw);
+  Pair<R>* buf = reinterpret_cast<Pair<R>*>(smem_raw);
   rows_tables<R, L2, RR, NT>(a.tw, buf);
   __syncthreads();
   const int nt = a.ti >= 0 ? 1 : a.c.nt;
@@ -454,24 +462,21 @@ __global__ void __launch_bounds__(NT, (blocks_for_smem(rows_smem<R, L2, RR>())))
     const int t = a.ti >= 0 ? a.ti : tq;
     const TmplMeta& m = a.c.meta[t];
     {
-      // the next row block's two runs of the intermediate, into L2
+      // the next row block's run of the intermediate, into L2
       const int wn = w + gridDim.x;
       if (threadIdx.x == 0 && wn < total) {
         const int tqn = wn / a.blocks_max;
         const int tn = a.ti >= 0 ? a.ti : tqn;
         const int blkn = wn - tqn * a.blocks_max;
         const int ln = a.c.meta[tn].log2n;
-        if (blkn * RR < (1 << (ln - L2))) {
-          const cpx<R>* pz = reinterpret_cast<const cpx<R>*>(a.c.za) + (int64_t)tn * a.c.z_stride +
-                             (int64_t)blkn * ((1 << L2) * RR);
-          constexpr unsigned bytes = (unsigned)((1u << L2) * RR * sizeof(cpx<R>));
-          prefetch_l2(pz, bytes);
-          prefetch_l2(pz + ((int64_t)1 << ln), bytes);
-        }
+        if (blkn * RR < (1 << (ln - L2)))
+          prefetch_l2(reinterpret_cast<const Pair<R>*>(a.c.za) + (int64_t)tn * a.c.z_stride +
+                          (int64_t)blkn * ((1 << L2) * RR),
+                      (unsigned)((1u << L2) * RR * sizeof(Pair<R>)));
       }
     }
     if (blk * RR >= (1 << (m.log2n - L2))) continue;
-    const cpx<R>* za = reinterpret_cast<const cpx<R>*>(a.c.za) + (int64_t)t * a.c.z_stride;
+    const Pair<R>* za = reinterpret_cast<const Pair<R>*>(a.c.za) + (int64_t)t * a.c.z_stride;
     rows_tile<R, L2, RR, NT, BAND>(a, t, blk, buf, za);
     __syncthreads();                      // the next block reuses buf
   }

@@ -18,14 +18,14 @@ namespace fs {
 
 namespace {
 
-constexpr int kPT = 512;          // threads per block
+constexpr int kPT = 256;          // threads per block
 constexpr int kPP = 8192;         // points per work item (both series)
 constexpr int kSlots = 3;         // intermediate slots in flight
 
 struct PersistArgs {
   ColsArgs<float> ca;             // ca.c: per-template meta, knots, partials, counters
   RowsArgs<float> ra;
-  float2* zslots;                 // kSlots x z_stride complex values
+  Pair<float>* zslots;            // kSlots x z_stride pairs
   int64_t z_stride;
   const int* sched;               // item offset of each round, [n_t + 2]
   const int* cnt;                 // column tiles [0, n_t), row blocks [n_t, 2 n_t)
@@ -81,25 +81,25 @@ __device__ __forceinline__ int l1_of(int L) { return default_log2_n1(L); }
 // Each tile shape is its own (not inlined) function, so that its register
 // allocation does not have to cover the other shapes.
 template <int L1, int SRC, int TAPS>
-__device__ __noinline__ void cols_call(const ColsArgs<float>& a, int t, int tile, float2* buf, double* red,
-                                       float2* za, int rr, int lr) {
-  cols_tables<float, L1, cols_for<float, kPP>(L1), kPT>(a.tw, buf);
-  cols_tile<float, L1, cols_for<float, kPP>(L1), kPT, SRC, TAPS>(a, t, tile, buf, red, za, rr, lr);
+__device__ __noinline__ void cols_call(const ColsArgs<float>& a, int t, int tile, Pair<float>* buf, double* red,
+                                       Pair<float>* za, int rr, int lr) {
+  cols_tables<float, L1, cols_for<kPP>(L1), kPT>(a.tw, buf);
+  cols_tile<float, L1, cols_for<kPP>(L1), kPT, SRC, TAPS>(a, t, tile, buf, red, za, rr, lr);
 }
 template <int L2>
-__device__ __noinline__ void rows_call(const RowsArgs<float>& a, int t, int blk, float2* buf, const float2* za) {
-  rows_tables<float, L2, cols_for<float, kPP>(L2), kPT>(a.tw, buf);
+__device__ __noinline__ void rows_call(const RowsArgs<float>& a, int t, int blk, Pair<float>* buf, const Pair<float>* za) {
+  rows_tables<float, L2, cols_for<kPP>(L2), kPT>(a.tw, buf);
   __syncthreads();
-  rows_tile<float, L2, cols_for<float, kPP>(L2), kPT, true>(a, t, blk, buf, za);
+  rows_tile<float, L2, cols_for<kPP>(L2), kPT, true>(a, t, blk, buf, za);
 }
 
 template <int SRC, int TAPS>
-__device__ __forceinline__ void run_cols(const PersistArgs& p, int t, int tile, float2* buf, double* red) {
+__device__ __forceinline__ void run_cols(const PersistArgs& p, int t, int tile, Pair<float>* buf, double* red) {
   const int L = p.ca.c.meta[t].log2n;
   const int l1 = l1_of(L), l2 = L - l1;
-  const int rr = cols_for<float, kPP>(l2);
+  const int rr = cols_for<kPP>(l2);
   const int lr = 31 - __clz(rr);
-  float2* za = p.zslots + (int64_t)(t % kSlots) * p.z_stride;
+  Pair<float>* za = p.zslots + (int64_t)(t % kSlots) * p.z_stride;
   switch (l1) {
 #define FS_P_COLS(V) case V: cols_call<V, SRC, TAPS>(p.ca, t, tile, buf, red, za, rr, lr); break;
     FS_P_COLS(6) FS_P_COLS(7) FS_P_COLS(8) FS_P_COLS(9) FS_P_COLS(10) FS_P_COLS(11) FS_P_COLS(12)
@@ -108,10 +108,10 @@ __device__ __forceinline__ void run_cols(const PersistArgs& p, int t, int tile, 
   }
 }
 
-__device__ __forceinline__ void run_rows(const PersistArgs& p, int t, int blk, float2* buf) {
+__device__ __forceinline__ void run_rows(const PersistArgs& p, int t, int blk, Pair<float>* buf) {
   const int L = p.ra.c.meta[t].log2n;
   const int l2 = L - l1_of(L);
-  const float2* za = p.zslots + (int64_t)(t % kSlots) * p.z_stride;
+  const Pair<float>* za = p.zslots + (int64_t)(t % kSlots) * p.z_stride;
   switch (l2) {
 #define FS_P_ROWS(V) case V: rows_call<V>(p.ra, t, blk, buf, za); break;
     FS_P_ROWS(6) FS_P_ROWS(7) FS_P_ROWS(8) FS_P_ROWS(9) FS_P_ROWS(10) FS_P_ROWS(11) FS_P_ROWS(12)
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kPT, 2) k_persist(PersistArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[96];
   __shared__ int item_sh;
-  float2* buf = reinterpret_cast<float2*>(smem_raw);
+  Pair<float>* buf = reinterpret_cast<Pair<float>*>(smem_raw);
   const int n_t = p.n_t;
   const int total = p.sched[n_t + 1];
   for (;;) {
@@ -169,7 +169,7 @@ __global__ void k_schedule(const TmplMeta* __restrict__ meta, int n_t, int* cnt,
     const TmplMeta& m = meta[t];
     const int L = m.log2n;
     const int l1 = l1_of(L), l2 = L - l1;
-    const int C = cols_for<float, kPP>(l1), RR = cols_for<float, kPP>(l2);
+    const int C = cols_for<kPP>(l1), RR = cols_for<kPP>(l2);
     cnt[t] = m.status == FSTAT_OK ? (1 << l2) / C : 0;
     cnt[n_t + t] = (1 << l1) / RR;
   }
@@ -212,7 +212,7 @@ int persist_slots() { return kSlots; }
 // Largest dynamic shared memory of any tile shape of either pass (FP32).
 size_t persist_smem() {
   size_t m = 0;
-#define FS_P_SM(V) { const size_t a = cols_smem<float, V, cols_for<float, kPP>(V)>(), b = rows_smem<float, V, cols_for<float, kPP>(V)>(); \
+#define FS_P_SM(V) { const size_t a = cols_smem<float, V, cols_for<kPP>(V)>(), b = rows_smem<float, V, cols_for<kPP>(V)>(); \
                        if (a > m) m = a; if (b > m) m = b; }
   FS_P_SM(6) FS_P_SM(7) FS_P_SM(8) FS_P_SM(9) FS_P_SM(10) FS_P_SM(11) FS_P_SM(12)
 #undef FS_P_SM
@@ -221,7 +221,7 @@ size_t persist_smem() {
 
 // counters: [cols_done n_t][rows_done n_t][head][abort]; sched [n_t + 2]; cnt [2 n_t]
 cudaError_t launch_persist(const PlanConst& pc, const Chunk& c, const float2* x, const int64_t* gaps,
-                           const double* wcs, const void* twf, float* out, int* status, float2* zslots,
+                           const double* wcs, const void* twf, float* out, int* status, void* zslots,
                            int64_t z_stride, int* counters, int* sched, int* cnt, int spin_limit,
                            int stall_template, cudaStream_t s) {
   const int n_t = c.nt;
@@ -233,7 +233,7 @@ cudaError_t launch_persist(const PlanConst& pc, const Chunk& c, const float2* x,
   p.ca.tw = *reinterpret_cast<const Tw<float>*>(twf);
   p.ca.ti = -1; p.ca.tiles_max = 0; p.ca.status = status; p.ca.rr = 1; p.ca.log2rr = 0;
   p.ra.pc = pc; p.ra.c = c; p.ra.tw = p.ca.tw; p.ra.out = out; p.ra.ti = -1; p.ra.cols = 1; p.ra.log2cols = 0; p.ra.blocks_max = 0; p.ra.band = 1;
-  p.zslots = zslots;
+  p.zslots = static_cast<Pair<float>*>(zslots);
   p.z_stride = z_stride;
   p.sched = sched;
   p.cnt = cnt;

@@ -117,7 +117,7 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ x
   constexpr int LP = tile_log2<R>();
   constexpr int P = 1 << LP;
   __shared__ double red[96];
-  __shared__ Cx sa[P + 32], sb[P + 32];
+  __shared__ Pair<R> sw[P + 32];
   const int t = blockIdx.y;
   const TmplMeta& m = c.meta[t];
   if (m.status != FSTAT_OK) return;
@@ -129,8 +129,7 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ x
   const int TR = P >> ltc;
   const Knot* kn = reinterpret_cast<const Knot*>(c.knots) + (int64_t)t * c.knot_stride;
   double* part = c.partials + (int64_t)t * c.part_stride * 3;
-  Cx* wa = reinterpret_cast<Cx*>(c.wa) + (int64_t)t * c.z_stride;
-  Cx* wb = wa + ((int64_t)1 << L);
+  Pair<R>* w_out = reinterpret_cast<Pair<R>*>(c.wa) + (int64_t)t * c.z_stride;
   const int lrun = (LP - ltc) + lc;            // log2 (TR * C)
   const int64_t gstride = (int64_t)1 << (L - l2 + lc);   // N1 * C
   GapCursor gc = make_cursor(m, gaps);
@@ -153,8 +152,7 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ x
           pa += (float)(aa * aa); pb += (float)(bb * bb); pcc += (float)(aa * bb);
         }
       }
-      sa[row * (TC + 1) + col] = va;
-      sb[row * (TC + 1) + col] = vb;
+      sw[row * (TC + 1) + col] = Pair<R>{va, vb};
     }
     double sA, sB, sC;
     block_sum3(pa, pb, pcc, sA, sB, sC, red);   // also orders the tile writes before the reads below
@@ -164,10 +162,9 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ x
       const int g = e >> lrun, w = e & ((1 << lrun) - 1);
       const int row = w >> lc, col = (g << lc) + (w & ((1 << lc) - 1));
       const int64_t o = ((int64_t)(c0 >> lc) + g) * gstride + ((int64_t)r0 << lc) + w;
-      __stcs(wa + o, sa[row * (TC + 1) + col]);
-      __stcs(wb + o, sb[row * (TC + 1) + col]);
+      stcs(w_out + o, sw[row * (TC + 1) + col]);
     }
-    __syncthreads();                            // before the next tile overwrites sa, sb
+    __syncthreads();                            // before the next tile overwrites sw
   }
 }
 
@@ -195,7 +192,7 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ x
 // on, their taps all lying above this run's).
 __device__ __noinline__ void run_slow(const PlanConst& pc, const KnotF* __restrict__ kn, int k0, int n_b,
                                       const float2* __restrict__ x, const GapCursor& gc,
-                                      const double* __restrict__ wcs, float2* da, float2* db, float& pa, float& pb,
+                                      const double* __restrict__ wcs, Pair<float>* dw, float& pa, float& pb,
                                       float& pcc) {
 #pragma unroll 1
   for (int i = 0; i < 8; ++i) {
@@ -207,8 +204,7 @@ __device__ __noinline__ void run_slow(const PlanConst& pc, const KnotF* __restri
         pa += aa * aa; pb += bb * bb; pcc += aa * bb;
       }
     }
-    da[i] = va;
-    db[i] = vb;
+    dw[i] = Pair<float>{va, vb};
   }
 }
 
@@ -216,7 +212,7 @@ constexpr int kRunTC = 256;
 constexpr int kRunTR = kResThreads / 32;
 // padded shared-memory rows: the eight-value strides of the compute phase
 // and the column groups of the store phase both fall on distinct banks
-constexpr int kRunStride = kRunTC + kRunTC / 8 + 2;
+constexpr int kRunStride = kRunTC + kRunTC / 8 + 1;
 __device__ __forceinline__ int run_idx(int row, int col) { return row * kRunStride + col + (col >> 3); }
 
 __global__ void __launch_bounds__(kResThreads, 3)
@@ -224,7 +220,7 @@ k_resample_r8(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ 
               const int64_t* __restrict__ gaps, const double* __restrict__ wcs) {
   constexpr int LP = tile_log2<float>();
   static_assert((1 << LP) == kRunTC * kRunTR, "a tile is 8 rows of 256 points");
-  __shared__ float2 sa[kRunTR * kRunStride], sb[kRunTR * kRunStride];
+  __shared__ Pair<float> sw[kRunTR * kRunStride];
   const int t = blockIdx.y;
   const TmplMeta& m = c.meta[t];
   if (m.status != FSTAT_OK) return;
@@ -233,8 +229,7 @@ k_resample_r8(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ 
   const int nlive = live_tiles(m.n_b, l2, lc, LP);
   const KnotF* kn = reinterpret_cast<const KnotF*>(c.knots) + (int64_t)t * c.knot_stride;
   double* part = c.partials + (int64_t)t * c.part_stride * 3;
-  float2* wa = reinterpret_cast<float2*>(c.wa) + (int64_t)t * c.z_stride;
-  float2* wb = wa + ((int64_t)1 << L);
+  Pair<float>* w_out = reinterpret_cast<Pair<float>*>(c.wa) + (int64_t)t * c.z_stride;
   const int lrun = (LP - 8) + lc;                        // log2 (TR * C)
   const int64_t gstride = (int64_t)1 << (L - l2 + lc);   // N1 * C
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -259,11 +254,10 @@ k_resample_r8(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ 
     const int krow = c0 + ((r0 + warp) << l2);            // first point of this warp's row
     const int k0 = krow + 8 * lane;
     float pa = 0.f, pb = 0.f, pcc = 0.f;
-    float2* da = sa + run_idx(warp, 8 * lane);
-    float2* db = sb + run_idx(warp, 8 * lane);
+    Pair<float>* dw = sw + run_idx(warp, 8 * lane);
     if (krow >= n_b) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) { da[i] = make_float2(0.f, 0.f); db[i] = make_float2(0.f, 0.f); }
+      for (int i = 0; i < 8; ++i) dw[i] = Pair<float>{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     } else {
       const bool live = k0 < n_b;
       const int sk = k0 & hmask;                         // the run stays in one knot interval
@@ -337,13 +331,12 @@ k_resample_r8(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ 
             int dummy;
             const float2 e = expm2pi(ph - round_nearest(ph, &dummy));
             const float2 y = cmul(z, e);
-            da[h + i] = make_float2(a * y.x, a * y.y);
-            db[h + i] = make_float2(bb * y.x, bb * y.y);
+            dw[h + i] = Pair<float>{make_float2(a * y.x, a * y.y), make_float2(bb * y.x, bb * y.y)};
             pa = fmaf(a, a, pa); pb = fmaf(bb, bb, pb); pcc = fmaf(a, bb, pcc);
           }
         }
       } else {
-        run_slow(pc, kn, k0, n_b, x, gc, wcs, da, db, pa, pb, pcc);
+        run_slow(pc, kn, k0, n_b, x, gc, wcs, dw, pa, pb, pcc);
       }
     }
     // A, B, C of this warp's row of the tile (sums in FP32 across the warp;
@@ -364,10 +357,9 @@ k_resample_r8(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ 
       const int g = e >> lrun, w = e & ((1 << lrun) - 1);
       const int row = w >> lc, col = (g << lc) + (w & ((1 << lc) - 1));
       const int64_t o = ((int64_t)(c0 >> lc) + g) * gstride + ((int64_t)r0 << lc) + w;
-      __stcs(wa + o, sa[run_idx(row, col)]);
-      __stcs(wb + o, sb[run_idx(row, col)]);
+      stcs(w_out + o, sw[run_idx(row, col)]);
     }
-    __syncthreads();                            // before the next tile overwrites sa, sb and the runs
+    __syncthreads();                            // before the next tile overwrites sw
   }
 }
 

@@ -17,8 +17,8 @@ namespace fs {
 cudaError_t FS_CAT(rows, FS_REAL, FS_L2)(const RowsArgs<FS_REAL>& a, dim3 grid, cudaStream_t s) {
   using R = FS_REAL;
   constexpr int L2 = FS_L2;
-  constexpr int RR = cols_for<R>(L2);
-  constexpr int NT = threads_for<R>(L2, 2 * RR);
+  constexpr int RR = cols_for<points_b<R>()>(L2);
+  constexpr int NT = threads_for<R>(L2, RR);
   constexpr size_t SM = rows_smem<R, L2, RR>();
   auto kern = a.band ? k_rows<R, L2, RR, NT, true> : k_rows<R, L2, RR, NT, false>;
   // persistent grid: the blocks that fit on the device at once
@@ -31,6 +31,6 @@ cudaError_t FS_CAT(rows, FS_REAL, FS_L2)(const RowsArgs<FS_REAL>& a, dim3 grid, 
   kern<<<total < (unsigned)resident ? total : (unsigned)resident, NT, SM, s>>>(a);
   return cudaGetLastError();
 }
-int FS_CAT(rowsR, FS_REAL, FS_L2)() { return cols_for<FS_REAL>(FS_L2); }
+int FS_CAT(rowsR, FS_REAL, FS_L2)() { return cols_for<points_b<FS_REAL>()>(FS_L2); }
 
 }  // namespace fs
