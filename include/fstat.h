@@ -73,7 +73,8 @@ enum {
 };
 /* execution mode (fstat_tuning.mode; a new plan starts in FSTAT_MODE_SPLIT) */
 enum {
-  FSTAT_MODE_FUSED      = 0, /* resample+weight fused into the first FFT pass, batched grids */
+  FSTAT_MODE_FUSED      = 0, /* FSTAT_MODE_SPLIT in one buffer: the first pass transforms the
+                                resampled columns in place (half the workspace)             */
   FSTAT_MODE_PLAIN      = 1, /* FSTAT_MODE_SPLIT one template per launch                      */
   FSTAT_MODE_PERSISTENT = 2, /* one persistent launch over all (template, tile) work items  */
   FSTAT_MODE_SPLIT      = 3  /* resample+weight over contiguous runs into HBM, in the first

@@ -414,18 +414,15 @@ int fstat_compute(fstat_plan_t p, const float* x_h, const fstat_template* t, int
   for (int64_t t0 = 0; t0 < n_t; t0 += p->chunk) {
     const int nt = (int)(n_t - t0 < p->chunk ? n_t - t0 : p->chunk);
     Chunk c = chunk_at(p, t + t0, nt);
-    cudaError_t e = cudaMemsetAsync(c.counters, 0, sizeof(int) * nt, s);
-    if (e == cudaSuccess)
-      e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, gaps, n_gaps_total, p->status, t0, s); });
-    if (e != cudaSuccess) return FSTAT_ECUDA;
-    const int fused = p->tune.mode == FSTAT_MODE_FUSED;
-    if (!fused) {
-      e = timed(p, K_RESAMPLE, s, [&] { return launch_resample_t(p->pc, c, p->sh, x, gaps, p->wcs, s); });
-      if (e == cudaSuccess) e = timed(p, K_SUMS, s, [&] { return launch_sums_t(p->pc, c, p->sh, p->status, s); });
-    }
-    if (e == cudaSuccess)
-      e = timed(p, K_COLS, s, [&] { return launch_cols_w(p->pc, c, p->sh, fused, -1, x, gaps, p->wcs, &p->twf, &p->twd, p->status, s); });
-    if (e == cudaSuccess) e = timed(p, K_ROWS, s, [&] { return launch_rows_w(p->pc, c, p->sh, -1, &p->twf, &p->twd, twoF, s); });
+    // fused mode: the resampled series lies where the intermediate goes, and
+    // pass A transforms each column in place
+    const int inplace = p->tune.mode == FSTAT_MODE_FUSED;
+    if (inplace) c.wa = c.za;
+    cudaError_t e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, gaps, n_gaps_total, p->status, t0, s); });
+    if (e == cudaSuccess) e = timed(p, K_RESAMPLE, s, [&] { return launch_resample_t(p->pc, c, p->sh, x, gaps, p->wcs, s); });
+    if (e == cudaSuccess) e = timed(p, K_SUMS, s, [&] { return launch_sums_t(p->pc, c, p->sh, p->status, s); });
+    if (e == cudaSuccess) e = timed(p, K_COLS, s, [&] { return launch_cols_w(p->pc, c, p->sh, inplace, &p->twf, &p->twd, p->status, s); });
+    if (e == cudaSuccess) e = timed(p, K_ROWS, s, [&] { return launch_rows_w(p->pc, c, p->sh, inplace, &p->twf, &p->twd, twoF, s); });
     if (e != cudaSuccess) return FSTAT_ECUDA;
   }
   return FSTAT_OK;

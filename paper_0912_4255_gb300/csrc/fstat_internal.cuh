@@ -365,6 +365,10 @@ struct GapCursor {
     g = a;
     load();
   }
+  // the first gap that ends after j (j ascending)
+  __device__ __forceinline__ void advance(int j) {
+    while (ce <= j) { ++g; load(); }
+  }
   // true iff every sample of [j0, j1] is valid; advances the cursor to j0
   __device__ __forceinline__ bool window_valid(int j0, int j1) {
     if (j0 < lo || j1 >= hi) return false;
@@ -551,6 +555,15 @@ __device__ __forceinline__ bool sinc8_f32(const float2* __restrict__ x, GapCurso
   return true;
 }
 
+// Phase P + ((p3 s + p2) s + p1) s of a knot interval, mod 1: the linear
+// term reaches many cycles at the end of an interval, so its whole cycles come
+// off exactly before the terms are added.
+__device__ __forceinline__ float knot_phase(float P, float p1, float p2, float p3, float s) {
+  int n;
+  const float whole = round_nearest(p1 * s, &n);
+  return P + fmaf((p3 * s + p2) * s, s, fmaf(p1, s, -whole));
+}
+
 // Per-sample time map and weights (steps 2-5) at grid point k < N_b of a
 // template: returns the mask and writes wa = m a y, wb = m b y with
 // y = z(T^k) exp(-2 pi i P(k)), and the beam values a, b.
@@ -572,7 +585,7 @@ __device__ __forceinline__ bool sample_weights(
     const float4 r0 = __ldg(q), r1 = __ldg(q + 1), r2 = __ldg(q + 2), r3 = __ldg(q + 3), r4 = __ldg(q + 4);
     ibase = __float_as_int(r0.x) + sk;
     dev = r0.y + ((r1.x * s + r0.w) * s + r0.z) * s;
-    ph = r1.y + ((r2.x * s + r1.w) * s + r1.z) * s;
+    ph = knot_phase(r1.y, r1.z, r1.w, r2.x, s);
     a = r2.y + ((r3.x * s + r2.w) * s + r2.z) * s;
     b = r3.y + ((r4.x * s + r3.w) * s + r3.z) * s;
   } else {
@@ -1084,10 +1097,9 @@ cudaError_t launch_resample_w(const PlanConst& pc, const Chunk& c, int ti, int l
 cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& sh, const float2* x,
                               const int64_t* gaps, const double* wcs, cudaStream_t s);
 cudaError_t launch_sums_t(const PlanConst& pc, const Chunk& c, const Shape& sh, int* status, cudaStream_t s);
-cudaError_t launch_cols_w(const PlanConst& pc, const Chunk& c, const Shape& sh, int fused, int ti,
-                          const float2* x, const int64_t* gaps, const double* wcs, const void* twf,
+cudaError_t launch_cols_w(const PlanConst& pc, const Chunk& c, const Shape& sh, int inplace, const void* twf,
                           const void* twd, int* status, cudaStream_t s);
-cudaError_t launch_rows_w(const PlanConst& pc, const Chunk& c, const Shape& sh, int ti, const void* twf,
+cudaError_t launch_rows_w(const PlanConst& pc, const Chunk& c, const Shape& sh, int inplace, const void* twf,
                           const void* twd, float* out, cudaStream_t s);
 cudaError_t launch_grad_pass(const PlanConst& pc, const Chunk& c, const float2* x, const int64_t* gaps,
                              const double* wcs, const double* df, double* work, double* twoF,

@@ -242,13 +242,13 @@ extern "C" int fstat_compute_noalloc(const fstat_plan_desc* d, const float* x_h,
     c.counters = reinterpret_cast<int*>(base + kOffCnt);
     c.za = base + kOffZ;
     c.z_stride = d->n_fft;
-    c.wa = nullptr;
+    c.wa = c.za;              // the resampled series, transformed in place by pass A
     c.nt = 1;
-    // the block counters must start at zero for every template
-    cudaError_t e = cudaMemsetAsync(c.counters, 0, 2 * sizeof(int), s);
-    if (e == cudaSuccess) e = launch_timemap(pc, c, L, FSTAT_MODE_FUSED, gaps, n_gaps_total, status, t, s);
-    if (e == cudaSuccess) e = launch_cols_w(pc, c, sh, 1, -1, x, gaps, wcs, &twf, &twd, status, s);
-    if (e == cudaSuccess) e = launch_rows_w(pc, c, sh, -1, &twf, &twd, twoF, s);
+    cudaError_t e = launch_timemap(pc, c, L, FSTAT_MODE_FUSED, gaps, n_gaps_total, status, t, s);
+    if (e == cudaSuccess) e = launch_resample_t(pc, c, sh, x, gaps, wcs, s);
+    if (e == cudaSuccess) e = launch_sums_t(pc, c, sh, status, s);
+    if (e == cudaSuccess) e = launch_cols_w(pc, c, sh, 1, &twf, &twd, status, s);
+    if (e == cudaSuccess) e = launch_rows_w(pc, c, sh, 1, &twf, &twd, twoF, s);
     if (e != cudaSuccess) return FSTAT_ECUDA;
   }
   return FSTAT_OK;

@@ -1,7 +1,7 @@
 // The two passes of the four-step FFT that evaluates Eqs. 19-20 for every
-// bin.  Steps 2-5 of Sec. III.A.2 are either fused into the first pass (fused
-// and persistent modes) or done by the tiled resampler, whose output the
-// first pass loads (split mode); Eq. 6 is fused into the second pass.
+// bin.  Steps 2-5 of Sec. III.A.2 are done by the tiled resampler, whose
+// output the first pass loads, or in the first pass (persistent mode); Eq. 6
+// is fused into the second pass.
 //
 // N = N1 N2, k = k2 + N2 k1, p = p1 + N1 p2:
 //   X[p1 + N1 p2] = sum_k2 W_N2^{p2 k2} W_N^{p1 k2} sum_k1 x[k2 + N2 k1] W_N1^{p1 k1}.
@@ -21,7 +21,11 @@
 
 namespace fs {
 
-enum { SRC_LOAD = 0, SRC_NN = 1, SRC_SINC = 2 };
+// Where pass A's samples come from: the tiled resampler's series (SRC_LOAD),
+// the same with the result written over it (SRC_INPLACE), or the resampling
+// of each point in the pass itself (persistent mode).
+enum { SRC_LOAD = 0, SRC_NN = 1, SRC_SINC = 2, SRC_INPLACE = 3 };
+__host__ __device__ constexpr bool loads(int src) { return src == SRC_LOAD || src == SRC_INPLACE; }
 
 // Bulk prefetch of [p, p + bytes) into L2 (p 16-byte aligned, bytes a
 // multiple of 16): issued by one thread, completes in the background.
@@ -37,8 +41,7 @@ struct ColsArgs {
   const int64_t* gaps;
   const double* wcs;
   Tw<R> tw;
-  int ti;        // template within the chunk, or -1 for blockIdx.y
-  int tiles_max; // grid.x
+  int tiles_max; // column tiles of one template
   int* status;
   int rr, log2rr; // rows per block of the second pass (layout of Z)
 };
@@ -49,7 +52,6 @@ struct RowsArgs {
   Chunk c;
   Tw<R> tw;
   float* out;
-  int ti;
   int cols;      // C of pass A
   int log2cols;
   int blocks_max; // row blocks of one template
@@ -175,7 +177,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
       tb[e2] = twiddle<R>(a.tw, L, (uint32_t)(q * NS) * (uint32_t)(c0 + c));
     }
   }
-  if constexpr (SRC == SRC_LOAD) {
+  if constexpr (loads(SRC)) {
     // the tiled resampler's order W[k2 / C][k1][k2 % C]: this tile's C * N1
     // pairs are contiguous, pair i = c + C k1 at offset i
     const Pair<R>* w_in = reinterpret_cast<const Pair<R>*>(a.c.wa) + (int64_t)t * a.c.z_stride +
@@ -226,7 +228,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
       buf[c * STRIDE + pidx(k1)] = Pair<R>{va, vb};
     }
   }
-  if constexpr (SRC != SRC_LOAD) {
+  if constexpr (!loads(SRC)) {
     double sA, sB, sC;
     block_sum3((float)pA, (float)pB, (float)pC, sA, sB, sC, red);
     double* part = a.c.partials + (int64_t)t * a.c.part_stride * 3;
@@ -239,7 +241,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
   // all stages but the last in shared memory (the first one done above when
   // loading; it needs no twiddles, so the tables start at the same place)
   static_assert(stage_tw_count<0, 4>() == 0, "first stage without twiddles");
-  fft_mid_stages<R, L1, SRC == SRC_LOAD ? 4 : 0, NSL_LAST, NT, C, STRIDE>(buf, tws);
+  fft_mid_stages<R, L1, loads(SRC) ? 4 : 0, NSL_LAST, NT, C, STRIDE>(buf, tws);
   // last stage: inputs from shared memory, outputs X[p1 = j + q NS] stay in
   // registers, are multiplied by W_N^{p1 k2} and stored into Z.  Of that
   // twiddle the factor W_N^{j k2} is common to a butterfly's outputs, so it
@@ -270,8 +272,16 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
     const int k2 = c0 + c;
     // p1 = j + q NS lands at Z[p1 / R][k2][p1 % R]; NS is a multiple of R, so
     // consecutive q are N / RADL elements apart
-    Pair<R>* zq = za + ((((int64_t)(j >> lr) * N2 + k2) << lr) + (j & (RRr - 1)));
-    const int64_t zstep = ((int64_t)1 << L) / RADL;
+    Pair<R>* zq;
+    int64_t zstep;
+    if constexpr (SRC == SRC_INPLACE) {
+      // over the tile's own columns, which were read whole above: [k2 / C][p1][k2 % C]
+      zq = za + (int64_t)tile * (C * N1) + j * C + c;
+      zstep = NS * C;
+    } else {
+      zq = za + ((((int64_t)(j >> lr) * N2 + k2) << lr) + (j & (RRr - 1)));
+      zstep = ((int64_t)1 << L) / RADL;
+    }
 #pragma unroll
     for (int q = 0; q < RADL; ++q) {
       const Cx w = tb[c * RADL + q];
@@ -289,21 +299,18 @@ __global__ void __launch_bounds__(NT, (min_blocks<R>(NT, cols_smem<R, L1, C>()))
   __shared__ double red[96];
   Pair<R>* buf = reinterpret_cast<Pair<R>*>(smem_raw);
   cols_tables<R, L1, C, NT>(a.tw, buf);
-  const int nt = a.ti >= 0 ? 1 : a.c.nt;
-  const int total = a.tiles_max * nt;
+  const int total = a.tiles_max * a.c.nt;
 #pragma unroll 1
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    const int tq = w / a.tiles_max;
-    const int tile = w - tq * a.tiles_max;
-    const int t = a.ti >= 0 ? a.ti : tq;
+    const int t = w / a.tiles_max;
+    const int tile = w - t * a.tiles_max;
     const TmplMeta& m = a.c.meta[t];
-    if constexpr (SRC == SRC_LOAD) {
+    if constexpr (loads(SRC)) {
       // the rows below n_b of the next tile's resampled block, into L2
       const int wn = w + gridDim.x;
       if (threadIdx.x == 0 && wn < total) {
-        const int tqn = wn / a.tiles_max;
-        const int tn = a.ti >= 0 ? a.ti : tqn;
-        const int tilen = wn - tqn * a.tiles_max;
+        const int tn = wn / a.tiles_max;
+        const int tilen = wn - tn * a.tiles_max;
         const TmplMeta& mn = a.c.meta[tn];
         const int ln = mn.log2n;
         if (mn.status == FSTAT_OK && tilen < (1 << (ln - L1)) / C) {
@@ -336,9 +343,11 @@ __device__ __forceinline__ void rows_tables(const Tw<R>& tw, Pair<R>* buf) {
 
 // One row block of pass B for template t (stage tables from rows_tables);
 // za: the template's intermediate.
+// INPLACE: the intermediate lies in pass A's column order [k2 / C][p1][k2 % C]
+// instead of row blocks.
 // BAND: the plan writes a partial output band (bins band_lo <= q < band_hi
 // only); without it every bin is stored, with no band test.
-template <typename R, int L2, int RR, int NT, bool BAND>
+template <typename R, int L2, int RR, int NT, bool BAND, bool INPLACE>
 __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, Pair<R>* __restrict__ buf,
                                           const Pair<R>* __restrict__ zbase) {
   using Cx = cpx<R>;
@@ -387,7 +396,14 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
     Cx xa[RAD0], xb[RAD0];
 #pragma unroll
     for (int q = 0; q < RAD0; ++q) {
-      const Pair<R> v = ldcs(src + q * (Q0 * RR));
+      Pair<R> v;
+      if constexpr (INPLACE) {
+        const int k2 = j + q * Q0;
+        v = ldcs(zbase + ((int64_t)(k2 >> a.log2cols) << (L - L2 + a.log2cols)) + ((r0 + r) << a.log2cols) +
+                 (k2 & (a.cols - 1)));
+      } else {
+        v = ldcs(src + q * (Q0 * RR));
+      }
       xa[q] = v.a;
       xb[q] = v.b;
     }
@@ -447,27 +463,24 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
 }
 
 // Persistent over the (template, row block) items of a chunk.
-template <typename R, int L2, int RR, int NT, bool BAND>
+template <typename R, int L2, int RR, int NT, bool BAND, bool INPLACE>
 __global__ void __launch_bounds__(NT, (min_blocks<R>(NT, rows_smem<R, L2, RR>()))) k_rows(RowsArgs<R> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Pair<R>* buf = reinterpret_cast<Pair<R>*>(smem_raw);
   rows_tables<R, L2, RR, NT>(a.tw, buf);
   __syncthreads();
-  const int nt = a.ti >= 0 ? 1 : a.c.nt;
-  const int total = a.blocks_max * nt;
+  const int total = a.blocks_max * a.c.nt;
 #pragma unroll 1
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
-    const int tq = w / a.blocks_max;
-    const int blk = w - tq * a.blocks_max;
-    const int t = a.ti >= 0 ? a.ti : tq;
+    const int t = w / a.blocks_max;
+    const int blk = w - t * a.blocks_max;
     const TmplMeta& m = a.c.meta[t];
-    {
+    if constexpr (!INPLACE) {
       // the next row block's run of the intermediate, into L2
       const int wn = w + gridDim.x;
       if (threadIdx.x == 0 && wn < total) {
-        const int tqn = wn / a.blocks_max;
-        const int tn = a.ti >= 0 ? a.ti : tqn;
-        const int blkn = wn - tqn * a.blocks_max;
+        const int tn = wn / a.blocks_max;
+        const int blkn = wn - tn * a.blocks_max;
         const int ln = a.c.meta[tn].log2n;
         if (blkn * RR < (1 << (ln - L2)))
           prefetch_l2(reinterpret_cast<const Pair<R>*>(a.c.za) + (int64_t)tn * a.c.z_stride +
@@ -477,7 +490,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<R>(NT, rows_smem<R, L2, RR>())
     }
     if (blk * RR >= (1 << (m.log2n - L2))) continue;
     const Pair<R>* za = reinterpret_cast<const Pair<R>*>(a.c.za) + (int64_t)t * a.c.z_stride;
-    rows_tile<R, L2, RR, NT, BAND>(a, t, blk, buf, za);
+    rows_tile<R, L2, RR, NT, BAND, INPLACE>(a, t, blk, buf, za);
     __syncthreads();                      // the next block reuses buf
   }
 }

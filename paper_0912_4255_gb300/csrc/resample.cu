@@ -4,6 +4,7 @@
 // fstat_resample (parity/debug output) and by the unfused single-template
 // path, whose first FFT pass then loads these series from memory.
 #include "passes.cuh"
+#include "sinc_run.cuh"
 
 namespace fs {
 
@@ -74,77 +75,105 @@ cudaError_t dispatch(const PlanConst& pc, const Chunk& c, int ti, int log2n, con
   return cudaGetLastError();
 }
 
-// Tiled form for the unfused path.  A tile is TR rows x TC consecutive
-// columns of the N1 x N2 grid (grid point k = k2 + N2 k1), so that a warp
-// handles 32 consecutive grid points: one knot record for all lanes, taps
-// from one contiguous run of x.  The tile goes through shared memory and is
-// stored in the order in which the first FFT pass reads its columns,
-// W[k2 / C][k1][k2 % C], as runs of TR * C values.  Tiles are numbered by
-// row tile, then column tile, so that their first point c0 + r0 N2 grows
-// with the number: the tiles holding points below n_b are a prefix, and the
-// first pass reads every point at k >= n_b as zero without loading it.  Each
-// tile leaves its partial sums of A, B, C; k_sums_t reduces them.
-template <typename R> constexpr int tile_log2() { return std::is_same<R, float>::value ? 11 : 10; }
-constexpr int kTilesPerBlock = 4;
+// Tiled form for the unfused path, one warp per tile of 8 rows x 32
+// consecutive columns of the N1 x N2 grid (grid point k = k2 + N2 k1).  The
+// tile goes through the warp's own shared memory and leaves in the order in
+// which the first FFT pass reads its columns, W[k2 / C][k1][k2 % C], as runs
+// of 8 C pairs (128 bytes at C = 1): no warp waits for another one.  Tiles are
+// numbered by row tile, then column tile; those of the row tiles with a point
+// below n_b are done, and the first pass reads every point at k >= n_b as
+// zero without loading it.  A warp takes per_warp consecutive tiles and
+// leaves one partial sum of A, B, C; k_sums_t reduces them.
+constexpr int kTileRows = 8, kTileCols = 32;
+constexpr int kTilePts = kTileRows * kTileCols;
+constexpr int kTileWarps = 4;                       // warps per block
+constexpr int kTileThreads = 32 * kTileWarps;
+constexpr int kMaxPerWarp = 8;
 
-// log2 of the tile width TC: at most 256 and N2, and small enough that a
-// tile keeps TR >= 16 / C rows, so that its stores form runs of at least 16
-// values (TR * C) per column group.
-__host__ __device__ __forceinline__ int tile_log2_cols(int l2, int lc, int lp) {
-  int ltc = l2 < 8 ? l2 : 8;
-  if (ltc > lp - 4 + lc) ltc = lp - 4 + lc;
-  return ltc;
+// tiles of the row tiles with a point below n_b
+__host__ __device__ __forceinline__ int live_tiles(int64_t n_b, int l2) {
+  return n_b <= 0 ? 0 : (int)(((n_b - 1) >> (l2 + 3)) + 1) << (l2 - 5);
 }
 
-// number of tiles with a point below n_b
-__host__ __device__ __forceinline__ int live_tiles(int64_t n_b, int l2, int lc, int lp) {
-  if (n_b <= 0) return 0;
-  const int ltc = tile_log2_cols(l2, lc, lp);
-  const int64_t span = (int64_t)1 << (lp - ltc + l2);    // points of one row tile, TR N2
-  const int ncol = 1 << (l2 - ltc);
-  const int64_t rt = (n_b - 1) / span;
-  const int64_t rem = n_b - rt * span;
-  const int64_t ct = (rem + (1 << ltc) - 1) >> ltc;
-  return (int)(rt * ncol + (ct < ncol ? ct : ncol));
+// Position of (row, col) in a warp's tile: rows of 32 pairs, the low three
+// bits of the column xored with a key of the row and the column's group of
+// eight.  Writes (8 lanes: two rows x four groups, one column each) and reads
+// (8 lanes: eight rows of one column) then fall on distinct 16-byte banks.
+__device__ __forceinline__ int tile_key(int row, int grp) { return grp ^ ((row >> 1) | ((row & 1) << 2)); }
+__device__ __forceinline__ int tile_pos(int row, int col) {
+  return row * kTileCols + (col & 24) + ((col & 7) ^ tile_key(row, col >> 3));
 }
 
+// The warp's tile from shared memory into W (first column c0, first row r0).
+template <typename R>
+__device__ __forceinline__ void store_tile(Pair<R>* __restrict__ w_out, const Pair<R>* __restrict__ so, int c0, int r0,
+                                           int lc, int64_t gstride, int lane) {
+  if (lc == 0) {
+    // one column pair per first-pass block: eight lanes a column
+    const int row = lane & 7, cl = lane >> 3;
+    const Pair<R>* sr = so + row * kTileCols;
+    Pair<R>* o = w_out + (int64_t)(c0 + cl) * gstride + r0 + row;
+#pragma unroll
+    for (int it = 0; it < kTilePts / 32; ++it) {
+      const int grp = it >> 1;                      // column 4 it + cl
+      stcs(o, sr[8 * grp + ((4 * (it & 1) + cl) ^ tile_key(row, grp))]);
+      o += 4 * gstride;
+    }
+    return;
+  }
+#pragma unroll
+  for (int it = 0; it < kTilePts / 32; ++it) {
+    const int e = it * 32 + lane;
+    const int g = e >> (3 + lc), w = e & ((8 << lc) - 1);
+    const int row = w >> lc, col = (g << lc) + (w & ((1 << lc) - 1));
+    stcs(w_out + ((int64_t)(c0 >> lc) + g) * gstride + ((int64_t)r0 << lc) + w, so[tile_pos(row, col)]);
+  }
+}
+
+// The warp's partial sum of A, B, C (a barrier over the block's warps would
+// hold them until the slowest is done).
+__device__ __forceinline__ void warp_partial(float pa, float pb, float pcc, double* __restrict__ part) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    pa += __shfl_down_sync(0xffffffffu, pa, o);
+    pb += __shfl_down_sync(0xffffffffu, pb, o);
+    pcc += __shfl_down_sync(0xffffffffu, pcc, o);
+  }
+  if ((threadIdx.x & 31) == 0) { part[0] = pa; part[1] = pb; part[2] = pcc; }
+}
+
+// Other tap counts, FP64 (and knot intervals of fewer than 32 points): one point per lane and row (32
+// consecutive points of a row at a time: one knot record for all lanes, taps
+// from one contiguous run of x).
 template <typename R, int INTERP, int TAPS>
-__global__ void __launch_bounds__(kResThreads)
-k_resample_t(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ x,
+__global__ void __launch_bounds__(kTileThreads)
+k_resample_t(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* __restrict__ x,
              const int64_t* __restrict__ gaps, const double* __restrict__ wcs) {
   using Cx = cpx<R>;
   using Knot = typename KnotOf<R>::T;
-  constexpr int LP = tile_log2<R>();
-  constexpr int P = 1 << LP;
-  __shared__ double red[96];
-  __shared__ Pair<R> sw[P + 32];
+  __shared__ Pair<R> tiles[kTileWarps][kTilePts];
   const int t = blockIdx.y;
   const TmplMeta& m = c.meta[t];
   if (m.status != FSTAT_OK) return;
-  const int L = m.log2n;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_b = (int)m.n_b;
-  const int nlive = live_tiles(m.n_b, l2, lc, LP);
-  const int ltc = tile_log2_cols(l2, lc, LP);  // log2 TC
-  const int TC = 1 << ltc;
-  const int TR = P >> ltc;
+  const int nlive = live_tiles(m.n_b, l2);
+  const int wid = (int)blockIdx.x * kTileWarps + warp;
+  const int b0 = wid * per_warp;
+  if (b0 >= nlive) return;
   const Knot* kn = reinterpret_cast<const Knot*>(c.knots) + (int64_t)t * c.knot_stride;
-  double* part = c.partials + (int64_t)t * c.part_stride * 3;
   Pair<R>* w_out = reinterpret_cast<Pair<R>*>(c.wa) + (int64_t)t * c.z_stride;
-  const int lrun = (LP - ltc) + lc;            // log2 (TR * C)
-  const int64_t gstride = (int64_t)1 << (L - l2 + lc);   // N1 * C
-  GapCursor gc = make_cursor(m, gaps);
+  const int64_t gstride = (int64_t)1 << (m.log2n - l2 + lc);   // N1 * C
+  Pair<R>* so = tiles[warp];
+  float pa = 0.f, pb = 0.f, pcc = 0.f;
 #pragma unroll 1
-  for (int tt = 0; tt < kTilesPerBlock; ++tt) {
-    const int b = (int)blockIdx.x * kTilesPerBlock + tt;
-    if (b >= nlive) break;
-    const int c0 = (b & ((1 << (l2 - ltc)) - 1)) << ltc;
-    const int r0 = (b >> (l2 - ltc)) * TR;
-    if (tt > 0) gc = make_cursor(m, gaps);    // the points of a new tile start lower
-    float pa = 0.f, pb = 0.f, pcc = 0.f;
+  for (int b = b0; b < b0 + per_warp && b < nlive; ++b) {
+    const int c0 = (b & ((1 << (l2 - 5)) - 1)) << 5;
+    const int r0 = (b >> (l2 - 5)) * kTileRows;
+    GapCursor gc = make_cursor(m, gaps);      // the points of a new tile start lower
 #pragma unroll 1
-    for (int e = threadIdx.x; e < P; e += kResThreads) {
-      const int col = e & (TC - 1), row = e >> ltc;
-      const int k = c0 + col + ((r0 + row) << l2);
+    for (int row = 0; row < kTileRows; ++row) {
+      const int k = c0 + lane + ((r0 + row) << l2);
       Cx va = czero<Cx>(), vb = czero<Cx>();
       if (k < n_b) {
         R aa, bb;
@@ -152,242 +181,334 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ x
           pa += (float)(aa * aa); pb += (float)(bb * bb); pcc += (float)(aa * bb);
         }
       }
-      sw[row * (TC + 1) + col] = Pair<R>{va, vb};
+      so[tile_pos(row, lane)] = Pair<R>{va, vb};
     }
-    double sA, sB, sC;
-    block_sum3(pa, pb, pcc, sA, sB, sC, red);   // also orders the tile writes before the reads below
-    if (threadIdx.x == 0) { part[3 * b] = sA; part[3 * b + 1] = sB; part[3 * b + 2] = sC; }
-#pragma unroll 4
-    for (int e = threadIdx.x; e < P; e += kResThreads) {
-      const int g = e >> lrun, w = e & ((1 << lrun) - 1);
-      const int row = w >> lc, col = (g << lc) + (w & ((1 << lc) - 1));
-      const int64_t o = ((int64_t)(c0 >> lc) + g) * gstride + ((int64_t)r0 << lc) + w;
-      stcs(w_out + o, sw[row * (TC + 1) + col]);
-    }
-    __syncthreads();                            // before the next tile overwrites sw
+    __syncwarp();
+    store_tile<R>(w_out, so, c0, r0, lc, gstride, lane);
+    __syncwarp();                             // before the next tile overwrites so
   }
+  warp_partial(pa, pb, pcc, c.partials + ((int64_t)t * c.part_stride + wid) * 3);
 }
 
-// Tiled form in runs of eight points (FP32, 8-tap windowed sinc, tiles of 8
-// rows x 256 consecutive columns, N2 >= 256): warp w of a block owns row
-// r0 + w of the tile, lane l the eight consecutive grid points
-// k0 = c0 + 8 l + (r0 + w) N2 .. k0 + 7.  The eight points lie in one knot
-// interval, and since the data index u advances by 1 + O(1e-4) samples per
-// grid point (dt_m/dt is bounded by the orbital and diurnal speeds, Eq.
-// 4pt2), floor(u) - k is the same for all of them except at rare slips.
-// Then their taps are the one run x[n0 - 3 .. n0 + 11] (n0 = floor(u) at
-// k0), loaded once, and the gap list is consulted once per run.  A run with
-// a slip, one that meets a gap or the span's edge, or one that reaches
-// n_b, takes the per-point path (sample_weights).  The per-point arithmetic
-// is that of sample_weights and sinc8_f32, so the series equals the one of
-// the per-point kernels bit for bit.  Each thread's runs only move forward
-// from tile to tile, so its gap cursor is kept across the tiles.  Every
-// warp leaves its own partial sums of A, B, C (one row of a tile), which
-// saves the block reduction's barriers; k_sums_t adds them.
-// The per-point path of a run that cannot take the shared tap run (a slip,
-// a gap or span edge, n_b): rare, kept out of line.  The windows of
-// consecutive points overlap, so a cursor that one point's last taps moved
-// past a gap would misjudge the next point's first taps: every point starts
-// from the cursor as it stands before the run (which only later runs move
-// on, their taps all lying above this run's).
-__device__ __noinline__ void run_slow(const PlanConst& pc, const KnotF* __restrict__ kn, int k0, int n_b,
-                                      const float2* __restrict__ x, const GapCursor& gc,
-                                      const double* __restrict__ wcs, Pair<float>* dw, float& pa, float& pb,
-                                      float& pcc) {
-#pragma unroll 1
-  for (int i = 0; i < 8; ++i) {
-    float2 va = make_float2(0.f, 0.f), vb = make_float2(0.f, 0.f);
-    if (k0 + i < n_b) {
-      float aa, bb;
-      GapCursor gi = gc;
-      if (sample_weights<float, FSTAT_SINC, 8>(pc, kn, k0 + i, x, gi, wcs, va, vb, aa, bb)) {
-        pa += aa * aa; pb += bb * bb; pcc += aa * bb;
-      }
+// One point of a run that cannot take the shared tap run (a slip, a gap or
+// span edge, n_b): rare, kept out of line.  The windows of consecutive points
+// overlap, so a cursor that one point's last taps moved past a gap would
+// misjudge the next point's first taps: every point starts from the cursor
+// as the run found it (gap index g).
+template <int INTERP>
+__device__ __noinline__ void slow_point(const PlanConst& pc, const KnotF* __restrict__ kn, int k, int n_b,
+                                        const float2* __restrict__ x, GapCursor gc, int g,
+                                        const double* __restrict__ wcs, Pair<float>* dst, float& pa, float& pb,
+                                        float& pcc) {
+  float2 va = make_float2(0.f, 0.f), vb = make_float2(0.f, 0.f);
+  if (k < n_b) {
+    float aa, bb;
+    gc.g = g;
+    gc.load();
+    if (sample_weights<float, INTERP, 8>(pc, kn, k, x, gc, wcs, va, vb, aa, bb)) {
+      pa += aa * aa; pb += bb * bb; pcc += aa * bb;
     }
-    dw[i] = Pair<float>{va, vb};
   }
+  *dst = Pair<float>{va, vb};
 }
 
-constexpr int kRunTC = 256;
-constexpr int kRunTR = kResThreads / 32;
-// padded shared-memory rows: the eight-value strides of the compute phase
-// and the column groups of the store phase both fall on distinct banks
-constexpr int kRunStride = kRunTC + kRunTC / 8 + 1;
-__device__ __forceinline__ int run_idx(int row, int col) { return row * kRunStride + col + (col >> 3); }
+// FP32, 8-tap windowed sinc or nearest neighbour, in runs of eight points: a lane owns eight
+// consecutive grid points of a row, four lanes a row of the tile.  The eight
+// points lie in one knot interval, and since u advances by 1 + O(1e-4)
+// samples per grid point floor(u) - k is the same for all of them except at
+// rare slips, so that their taps are the one run x[n0 - 3 .. n0 + 11],
+// n0 = floor(u) at k0, and the gap list is consulted once.  The knot's cubics
+// (u, phase, a, b) are taken to second order about the run's centre, the tap
+// weights come from one expansion (sinc_run.cuh), and the phase factor is the
+// centre's times a rotation, whose sine and cosine serve the two points at
+// equal distances from the centre.  A run with a slip, one that meets a gap
+// or the span's edge, one that reaches n_b, and one whose u moves too far for
+// the expansion are done point by point; a run inside one gap is zero.
+// With the Lanczos window a slip of at most e = kRunNarrow needs no care: the
+// tap that it drops and the one that it adds sit where the kernel is e^2 / 16.
+//
+// The samples of a row (48 from the one before its first tap) are copied as
+// 16-byte pieces into the warp's shared memory, a tile ahead (cp.async): read
+// straight from memory, the lanes' 64-byte stride cost 16 wavefronts a load.  Instruction issue
+// bounds the kernel (60 % of the cycles at 16 warps per SM, 128 registers; 96
+// registers spill and measured 1.07 times the time).  64 templates of 1,728,000
+// samples: 531 us, 1016 us when a block formed the weights of an 8 x 256 tile
+// point by point (240 instructions a point, now about 120); nearest neighbour,
+// 128 templates of 86,400: 62 us, 98 us with one point per lane.
+constexpr int kRowSamples = 44;
+constexpr int kRowUnits = kRowSamples / 2;        // 16-byte pieces of two samples
+constexpr float kRunRotation = 0.125f;            // cycles: sincospi_small holds for |2 cycles| <= 1/4
 
-__global__ void __launch_bounds__(kResThreads, 3)
-k_resample_r8(PlanConst pc, Chunk c, int l2, int lc, const float2* __restrict__ x,
-              const int64_t* __restrict__ gaps, const double* __restrict__ wcs) {
-  constexpr int LP = tile_log2<float>();
-  static_assert((1 << LP) == kRunTC * kRunTR, "a tile is 8 rows of 256 points");
-  __shared__ Pair<float> sw[kRunTR * kRunStride];
+__device__ __forceinline__ void copy_async16(void* dst, const void* src, bool inside) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(inside ? 16 : 0) : "memory");
+}
+
+enum { RUN_NEAREST = 0, RUN_LANCZOS = 1, RUN_RECT = 2 };
+
+template <int KIND, bool QUAD>
+__global__ void __launch_bounds__(kTileThreads, 4)
+k_resample_run(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* __restrict__ x,
+               const int64_t* __restrict__ gaps, const double* __restrict__ wcs) {
+  __shared__ __align__(128) Pair<float> tiles[kTileWarps][kTilePts];
+  __shared__ float4 rows[kTileWarps][2][kTileRows * kRowUnits];
+  __shared__ float4 recs[kTileWarps][kTileRows][5];
   const int t = blockIdx.y;
   const TmplMeta& m = c.meta[t];
   if (m.status != FSTAT_OK) return;
-  const int L = m.log2n;
-  const int n_b = (int)m.n_b;
-  const int nlive = live_tiles(m.n_b, l2, lc, LP);
-  const KnotF* kn = reinterpret_cast<const KnotF*>(c.knots) + (int64_t)t * c.knot_stride;
-  double* part = c.partials + (int64_t)t * c.part_stride * 3;
-  Pair<float>* w_out = reinterpret_cast<Pair<float>*>(c.wa) + (int64_t)t * c.z_stride;
-  const int lrun = (LP - 8) + lc;                        // log2 (TR * C)
-  const int64_t gstride = (int64_t)1 << (L - l2 + lc);   // N1 * C
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool lanczos = pc.window == FSTAT_WIN_LANCZOS;
+  const int n_b = (int)m.n_b;
+  const int nlive = live_tiles(m.n_b, l2);
+  const int wid = (int)blockIdx.x * kTileWarps + warp;
+  const int b0 = wid * per_warp;
+  if (b0 >= nlive) return;
+  const int b1 = b0 + per_warp < nlive ? b0 + per_warp : nlive;
+  const KnotF* kn = reinterpret_cast<const KnotF*>(c.knots) + (int64_t)t * c.knot_stride;
+  Pair<float>* w_out = reinterpret_cast<Pair<float>*>(c.wa) + (int64_t)t * c.z_stride;
+  const int64_t gstride = (int64_t)1 << (m.log2n - l2 + lc);   // N1 * C
+  const int row = lane >> 2, grp = lane & 3;
+  Pair<float>* so = tiles[warp];
+  const int key = tile_key(row, grp);
+  Pair<float>* dw = so + row * kTileCols + 8 * grp;
+  const unsigned out0 = (unsigned)__cvta_generic_to_shared(dw) + 16u * key;   // point i goes to out0 ^ 16 i
+  // x may start in the middle of a 16-byte piece: samples j with j + odd even
+  // start a piece, and samples outside [odd, x_end) lie in no whole piece
+  const int odd = (int)(((uintptr_t)x >> 3) & 1);
+  const int x_end = (((int)pc.n_data + odd) & ~1) - odd;
   const int hmask = (1 << pc.log2h) - 1;
-  const float sc_win = lanczos ? (float)(4.0 / (3.14159265358979323846 * 3.14159265358979323846))
-                               : (float)(1.0 / 3.14159265358979323846);
-  GapCursor gc = make_cursor(m, gaps);
-  {
-    // start the cursor near the block's first sample: the base index of the
-    // knot interval of its first point, less a margin for the taps
-    const int b = (int)blockIdx.x * kTilesPerBlock;
-    const int kf = ((b & ((1 << (l2 - 8)) - 1)) << 8) + (((b >> (l2 - 8)) * kRunTR) << l2);
-    if (kf < n_b) gc.seek(__float_as_int(__ldg(reinterpret_cast<const float*>(kn + (kf >> pc.log2h)))) - 64);
-  }
-#pragma unroll 1
-  for (int tt = 0; tt < kTilesPerBlock; ++tt) {
-    const int b = (int)blockIdx.x * kTilesPerBlock + tt;
-    if (b >= nlive) break;
-    const int c0 = (b & ((1 << (l2 - 8)) - 1)) << 8;
-    const int r0 = (b >> (l2 - 8)) * kRunTR;
-    const int krow = c0 + ((r0 + warp) << l2);            // first point of this warp's row
-    const int k0 = krow + 8 * lane;
-    float pa = 0.f, pb = 0.f, pcc = 0.f;
-    Pair<float>* dw = sw + run_idx(warp, 8 * lane);
-    if (krow >= n_b) {
+
+  // the lane's run in tile b: its first point
+  auto first_point = [&](int b) {
+    const int c0 = (b & ((1 << (l2 - 5)) - 1)) << 5;
+    const int r0 = (b >> (l2 - 5)) * kTileRows;
+    return c0 + 8 * grp + ((r0 + row) << l2);
+  };
+  // The knot records of the tile's eight rows, kept in shared memory: rows are
+  // N2 points apart and intervals h, both powers of two, so all rows enter
+  // their next interval at the same column.
+  float4(*rec)[5] = recs[warp];
+  auto load_records = [&](int k) {
+    const int kc = k < n_b ? k : n_b - 1;          // a record that exists
+    const float4* q = reinterpret_cast<const float4*>(kn + (kc >> pc.log2h));
+    __syncwarp();                                  // the last readers are done
+    rec[row][grp] = __ldg(q + grp);
+    if (grp == 0) rec[row][4] = __ldg(q + 4);
+    __syncwarp();
+  };
+  // floor(u) at the run's first point; f = the fraction at its centre
+  // (u = I + sk + i + dev(s + tau), s = sk + 3.5, tau = i - 3.5)
+  auto centre = [&](int k, float& s, float& f) {
+    const float4 q0 = rec[row][0];
+    const float u3 = rec[row][1].x;
+    const int sk = k & hmask;                      // a run stays in one knot interval
+    s = small_int_to_float(sk) + 3.5f;
+    const float dev = fmaf(fmaf(fmaf(u3, s, q0.w), s, q0.z), s, q0.y);
+    int fl;
+    float flf = round_nearest(dev, &fl);
+    if (flf > dev) { flf -= 1.0f; --fl; }
+    f = dev - flf;
+    return __float_as_int(q0.x) + sk + fl;
+  };
+  // starts the copy of the row's samples into buffer u; returns the index of
+  // the first one
+  auto stage = [&](int n0, int u) {
+    const int first = __shfl_sync(0xffffffffu, n0, lane & 28) - 4;
+    const int base = ((first + odd) & ~1) - odd;
+    float4* dst = rows[warp][u] + row * kRowUnits + grp;
+    const float2* src = x + base + 2 * grp;
+    if (__all_sync(0xffffffffu, base >= odd && base + kRowSamples <= x_end)) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) dw[i] = Pair<float>{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      for (int i = 0; i < (kRowUnits + 3) / 4; ++i)
+        if (4 * i + 4 <= kRowUnits || grp < kRowUnits % 4) copy_async16(dst + 4 * i, src + 8 * i, true);
     } else {
-      const bool live = k0 < n_b;
-      const int sk = k0 & hmask;                         // the run stays in one knot interval
-      const float4* q = reinterpret_cast<const float4*>(kn + (k0 >> pc.log2h));
-      const float4 q0 = __ldg(q), q1 = __ldg(q + 1), q2 = __ldg(q + 2), q3 = __ldg(q + 3), q4 = __ldg(q + 4);
-      const float s0 = small_int_to_float(sk);
-      // u = I + sk + i + dev_i; floor(dev_i) must not change along the run
-      int fl0 = 0;
-      float flf0 = 0.f;
-      bool even = true;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float s = s0 + (float)i;
-        const float dv = q0.y + ((q1.x * s + q0.w) * s + q0.z) * s;
-        int fi;
-        float ff = round_nearest(dv, &fi);
-        if (ff > dv) { ff -= 1.0f; --fi; }
-        if (i == 0) { fl0 = fi; flf0 = ff; }
-        else even = even && fi == fl0;
-      }
-      const int n0 = __float_as_int(q0.x) + sk + fl0;      // floor(u) at k0
-      const bool fast = live && even && k0 + 7 < n_b && gc.window_valid(n0 - 3, n0 + 11);
-      if (fast) {
-        // two halves of four points, each from its run of eleven samples
 #pragma unroll 1
-        for (int h = 0; h < 8; h += 4) {
-          float2 v[11];
+      for (int i = 0; grp + 4 * i < kRowUnits; ++i) {
+        const int jx = base + 2 * (grp + 4 * i);
+        const bool inside = jx >= odd && jx < x_end;
+        copy_async16(dst + 4 * i, inside ? src + 8 * i : x + odd, inside);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    return base;
+  };
+
+  GapCursor gc = make_cursor(m, gaps);
+  float pa = 0.f, pb = 0.f, pcc = 0.f;
+  int k0 = first_point(b0);
+  load_records(k0);
+  float s, f;
+  int n0 = centre(k0, s, f);
+  int base = stage(n0, 0);
+  if (gc.n > 0) gc.seek(n0 - 64);                    // this warp's points only move forward
+#pragma unroll 1
+  for (int b = b0; b < b1; ++b) {
+    const float4 q0 = rec[row][0], q1 = rec[row][1], q2 = rec[row][2], q3 = rec[row][3], q4 = rec[row][4];
+    const float d1 = q0.z + s * (2.0f * q0.w + 3.0f * q1.x * s), d2 = q0.w + 3.0f * q1.x * s;
+    const float p1 = q1.z + s * (2.0f * q1.w + 3.0f * q2.x * s), p2 = q1.w + 3.0f * q2.x * s;
+    const float pc0 = knot_phase(q1.y, q1.z, q1.w, q2.x, s);
+    const float a0 = q2.y + ((q3.x * s + q2.w) * s + q2.z) * s;
+    const float a1 = q2.z + s * (2.0f * q2.w + 3.0f * q3.x * s), a2 = q2.w + 3.0f * q3.x * s;
+    const float b0f = q3.y + ((q4.x * s + q3.w) * s + q3.z) * s;
+    const float b1f = q3.z + s * (2.0f * q3.w + 3.0f * q4.x * s), b2 = q3.w + 3.0f * q4.x * s;
+    const float spread = 3.5f * fabsf(d1) + 12.25f * fabsf(d2);
+    const int off = n0 - 3 - base;                   // the run's first tap
+    // the first gap that ends above the run (a slip may lower a tap by one)
+    gc.advance(n0 - 5);
+    const bool live = k0 < n_b;
+    const bool smooth = spread <= (QUAD ? kRunSpread : kRunNarrow);
+    // the nearest sample of every point in one gap: all masked
+    const bool masked = smooth && gc.cs < n0 && n0 + 9 < gc.ce;
+    // the data samples that the run's points may take: [j0, j1]
+    const int j0 = KIND == RUN_NEAREST ? n0 - 1 : n0 - 3, j1 = KIND == RUN_NEAREST ? n0 + 9 : n0 + 11;
+    const bool fast = live && smooth && k0 + 7 < n_b && j0 >= base && base + kRowSamples > j0 + 15 && j0 >= odd &&
+                      j1 < x_end && j0 >= gc.lo && j1 < gc.hi && j1 < gc.cs &&
+                      (KIND == RUN_NEAREST || (KIND == RUN_LANCZOS && !QUAD) ||
+                       (f >= spread + 1e-6f && f + spread < 1.0f - 1e-6f));
+    // the next tile's samples are on their way while this one is computed
+    const int k0n = first_point(b + 1 < b1 ? b + 1 : b);
+    if ((((k0n ^ k0) >> pc.log2h) | ((k0n ^ k0) >> l2)) != 0) load_records(k0n);
+    float sn_, fn_;
+    const int n0n = centre(k0n, sn_, fn_);
+    const int basen = stage(n0n, (b + 1 - b0) & 1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();
+    if (fast) {
+      // rotations of the points 3 - h and 4 + h (tau = -+(h + 1/2)) to the
+      // phase removed: the centre's factor times exp(-2 pi i (tau p1 + tau^2 p2));
+      // the linear part is one sine and cosine for both, the square a first-order turn
+      int di;
+      const float2 ec = expm2pi(pc0 - round_nearest(pc0, &di));
+      float2 rm[4], rp[4];
+      if (3.5f * fabsf(p1) <= kRunRotation && 12.25f * fabsf(p2) <= 1e-5f) {
 #pragma unroll
-          for (int j = 0; j < 11; ++j) v[j] = __ldg(x + n0 - 3 + h + j);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float s = s0 + (float)(h + i);
-            const float f = (q0.y + ((q1.x * s + q0.w) * s + q0.z) * s) - flf0;
-            const int qoff = f >= 0.5f ? 1 : 0;
-            const float dn = qoff ? f - 1.0f : f;
-            float sh, ch;
-            sincospi_small(0.25f * dn, &sh, &ch);
-            const float s2 = 2.0f * sh * ch, c2 = fmaf(ch, ch, -sh * sh);
-            const float sdn = 2.0f * s2 * c2;
-            const float sf = qoff ? -sdn : sdn;
-            const float r2 = 0.70710678118654752f;
-            const float p = (sh + ch) * r2, mm = (ch - sh) * r2;
-            const float w0 = qoff ? -sh : mm, w1 = qoff ? mm : ch, w2 = qoff ? ch : p, w3 = qoff ? p : sh;
-            float2 acc = make_float2(0.f, 0.f);
-            if (lanczos) {
-              const float g[8] = {-w0, w1, -w2, w3, w0, -w1, w2, -w3};
-#pragma unroll
-              for (int tp = 0; tp < 8; ++tp) {
-                const float xi = f + (float)(3 - tp);
-                const float w = g[tp] * rcp_approx(xi * xi);
-                acc.x = fmaf(w, v[i + tp].x, acc.x);
-                acc.y = fmaf(w, v[i + tp].y, acc.y);
-              }
-            } else {
-#pragma unroll
-              for (int tp = 0; tp < 8; ++tp) {
-                const float w = rcp_approx(f + (float)(3 - tp));
-                const float ws = ((3 - tp) & 1) ? -w : w;
-                acc.x = fmaf(ws, v[i + tp].x, acc.x);
-                acc.y = fmaf(ws, v[i + tp].y, acc.y);
-              }
-            }
-            // u on a sample (to the precision of u): the interpolant is that sample
-            const float2 vnn = qoff ? v[i + 4] : v[i + 3];
-            const float sc = sf * sc_win;
-            const bool on = fabsf(dn) < 1e-7f;
-            const float2 z = make_float2(on ? vnn.x : acc.x * sc, on ? vnn.y : acc.y * sc);
-            const float ph = q1.y + ((q2.x * s + q1.w) * s + q1.z) * s;
-            const float a = q2.y + ((q3.x * s + q2.w) * s + q2.z) * s;
-            const float bb = q3.y + ((q4.x * s + q3.w) * s + q3.z) * s;
-            int dummy;
-            const float2 e = expm2pi(ph - round_nearest(ph, &dummy));
-            const float2 y = cmul(z, e);
-            dw[h + i] = Pair<float>{make_float2(a * y.x, a * y.y), make_float2(bb * y.x, bb * y.y)};
-            pa = fmaf(a, a, pa); pb = fmaf(bb, bb, pb); pcc = fmaf(a, bb, pcc);
-          }
+        for (int h = 0; h < 4; ++h) {
+          const float tau = (float)h + 0.5f;
+          float sn, cs;
+          sincospi_small(2.0f * tau * p1, &sn, &cs);
+          const float eps = (6.28318531f * tau * tau) * p2;
+          const float ex = fmaf(eps, ec.y, ec.x), ey = fmaf(-eps, ec.x, ec.y);
+          const float xc = ex * cs, yc = ey * cs;
+          rp[h] = make_float2(fmaf(ey, sn, xc), fmaf(-ex, sn, yc));
+          rm[h] = make_float2(fmaf(-ey, sn, xc), fmaf(ex, sn, yc));
         }
       } else {
-        run_slow(pc, kn, k0, n_b, x, gc, wcs, dw, pa, pb, pcc);
-      }
-    }
-    // A, B, C of this warp's row of the tile (sums in FP32 across the warp;
-    // k_sums_t adds the per-warp partials in FP64 in a fixed order)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      pa += __shfl_down_sync(0xffffffffu, pa, o);
-      pb += __shfl_down_sync(0xffffffffu, pb, o);
-      pcc += __shfl_down_sync(0xffffffffu, pcc, o);
+        for (int h = 0; h < 4; ++h) {
+          const float tau = (float)h + 0.5f;
+          const float gp = tau * fmaf(tau, p2, p1), gm = tau * fmaf(tau, p2, -p1);
+          rp[h] = cmul(ec, expm2pi(gp - round_nearest(gp, &di)));
+          rm[h] = cmul(ec, expm2pi(gm - round_nearest(gm, &di)));
+        }
+      }
+      [[maybe_unused]] float w0[8], w1[8], w2[8];
+      [[maybe_unused]] float2 v[16];
+      const float4* xr = rows[warp][(b - b0) & 1] + row * kRowUnits;
+      if constexpr (KIND != RUN_NEAREST) {
+        run_weights<KIND == RUN_LANCZOS>(f - 0.5f, w0, w1, w2);
+        if constexpr (!QUAD) {
+          // d^2 w2 by its mean over |d| <= spread: what is left, (d^2 -
+          // spread^2 / 2) w2, is below 1.7e-7 (1.1e-7 at the Earth's)
+          const float hs = 0.5f * spread * spread;
+#pragma unroll
+          for (int tp = 0; tp < 8; ++tp) w0[tp] = fmaf(hs, w2[tp], w0[tp]);
+        }
+        const float4* xo = xr + (off >> 1);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float4 p = xo[j];
+          v[2 * j] = make_float2(p.x, p.y);
+          v[2 * j + 1] = make_float2(p.z, p.w);
+        }
+        if (off & 1) {
+#pragma unroll
+          for (int j = 0; j < 15; ++j) v[j] = v[j + 1];
+        }
+      }
+      const int sk = k0 & hmask;
+      [[maybe_unused]] const int ibase = __float_as_int(q0.x) + sk - base;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int h = i < 4 ? 3 - i : i - 4;
+        const float tau = (float)i - 3.5f, tau2 = tau * tau;
+        float2 z;
+        if constexpr (KIND == RUN_NEAREST) {
+          // the nearest sample is decided point by point: floor(dev + 1/2)
+          const float si = small_int_to_float(sk + i);
+          const float dv = q0.y + ((q1.x * si + q0.w) * si + q0.z) * si;
+          int ji;
+          if (round_nearest(dv + 0.5f, &ji) > dv + 0.5f) --ji;
+          z = reinterpret_cast<const float2*>(xr)[ibase + i + ji];
+        } else {
+          const float d = fmaf(tau, d1, tau2 * d2);
+          z = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int tp = 0; tp < 8; ++tp) {
+            float w;
+            if constexpr (QUAD) w = fmaf(d, fmaf(d, w2[tp], w1[tp]), w0[tp]);
+            else w = fmaf(d, w1[tp], w0[tp]);
+            z.x = fmaf(w, v[i + tp].x, z.x);
+            z.y = fmaf(w, v[i + tp].y, z.y);
+          }
+        }
+        const float2 y = cmul(z, i < 4 ? rm[h] : rp[h]);
+        const float a = fmaf(tau, a1, fmaf(tau2, a2, a0));
+        const float bb = fmaf(tau, b1f, fmaf(tau2, b2, b0f));
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(out0 ^ (16u * i)), "f"(a * y.x), "f"(a * y.y),
+                     "f"(bb * y.x), "f"(bb * y.y) : "memory");
+      }
+      // sums over the run of a^2, b^2, a b: sum tau^2 = 42, sum tau^4 = 388.5
+      pa += fmaf(8.0f * a0, a0, fmaf(42.0f, fmaf(a1, a1, 2.0f * a0 * a2), 388.5f * a2 * a2));
+      pb += fmaf(8.0f * b0f, b0f, fmaf(42.0f, fmaf(b1f, b1f, 2.0f * b0f * b2), 388.5f * b2 * b2));
+      pcc += fmaf(8.0f * a0, b0f, fmaf(42.0f, fmaf(a1, b1f, fmaf(a0, b2, a2 * b0f)), 388.5f * a2 * b2));
+    } else if (!live || masked) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) dw[i] = Pair<float>{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
     }
-    if (lane == 0) {
-      double* pw = part + 3 * ((int64_t)b * kRunTR + warp);
-      pw[0] = pa; pw[1] = pb; pw[2] = pcc;
+    // the other runs, four at a time, eight lanes a run (by its own lane, point
+    // after point, one such run held its warp for 10 us)
+    unsigned slow = __ballot_sync(0xffffffffu, live && !fast && !masked);
+    while (slow) {
+      int src = -1;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (lane >> 3 == r) src = __ffs(slow) - 1;
+        slow &= slow - 1;
+      }
+      const int sl = src < 0 ? 0 : src, i = lane & 7;
+      const int ks = __shfl_sync(0xffffffffu, k0, sl), gs = __shfl_sync(0xffffffffu, gc.g, sl);
+      if (src >= 0)
+        slow_point<KIND == RUN_NEAREST ? FSTAT_NEAREST : FSTAT_SINC>(
+            pc, kn, ks + i, n_b, x, gc, gs, wcs, so + tile_pos(sl >> 2, 8 * (sl & 3) + i), pa, pb, pcc);
+      __syncwarp();
     }
-    __syncthreads();                            // the tile is complete in shared memory
-#pragma unroll 4
-    for (int e = threadIdx.x; e < (1 << LP); e += kResThreads) {
-      const int g = e >> lrun, w = e & ((1 << lrun) - 1);
-      const int row = w >> lc, col = (g << lc) + (w & ((1 << lc) - 1));
-      const int64_t o = ((int64_t)(c0 >> lc) + g) * gstride + ((int64_t)r0 << lc) + w;
-      stcs(w_out + o, sw[run_idx(row, col)]);
-    }
-    __syncthreads();                            // before the next tile overwrites sw
+    __syncwarp();
+    store_tile<float>(w_out, so, (b & ((1 << (l2 - 5)) - 1)) << 5, (b >> (l2 - 5)) * kTileRows, lc, gstride, lane);
+    __syncwarp();                             // before the next tile overwrites so and the rows
+    k0 = k0n; n0 = n0n; base = basen; s = sn_; f = fn_;
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  warp_partial(pa, pb, pcc, c.partials + ((int64_t)t * c.part_stride + wid) * 3);
 }
 
-// The tiled resampler that runs in eights applies (it writes one partial of
-// A, B, C per warp and tile).
-bool use_runs(const PlanConst& pc, const Shape& sh, int lc) {
-  return pc.precision != FSTAT_PREC_FP64 && pc.interp == FSTAT_SINC && pc.taps == 8 &&
-         tile_log2_cols(sh.l2, lc, tile_log2<float>()) == 8;
-}
-
-// One block per template: A, B, C from the partials of its tiles, summed in
+// One block per template: A, B, C from the partials of its warps, summed in
 // FP64 in a fixed order (deterministic).  covered: tiles the resampling grid
 // reached; a template with more tiles below n_b (not expected: the grid is
 // sized from a bound on n_b) is reported as FSTAT_ERANGE.
 constexpr int kSumThreads = 256;
 __global__ void __launch_bounds__(kSumThreads)
-k_sums_t(Chunk c, int l2, int lc, int lp, int covered, int per_tile, double sigma2, int* status) {
+k_sums_t(Chunk c, int l2, int covered, int per_warp, double sigma2, int* status) {
   __shared__ double sh[3][kSumThreads];
   TmplMeta* m = c.meta + blockIdx.x;
   if (m->status != FSTAT_OK) return;
-  const int nlive = live_tiles(m->n_b, l2, lc, lp);
+  const int nlive = live_tiles(m->n_b, l2);
   if (nlive > covered) {
     if (threadIdx.x == 0) { m->status = FSTAT_ERANGE; set_status(status, FSTAT_ERANGE); }
     return;
   }
   const double* part = c.partials + (int64_t)blockIdx.x * c.part_stride * 3;
+  const int nparts = (nlive + per_warp - 1) / per_warp;
   double A = 0, B = 0, Cc = 0;
-  for (int i = threadIdx.x; i < nlive * per_tile; i += kSumThreads) {
+  for (int i = threadIdx.x; i < nparts; i += kSumThreads) {
     A += part[3 * i]; B += part[3 * i + 1]; Cc += part[3 * i + 2];
   }
   sh[0][threadIdx.x] = A; sh[1][threadIdx.x] = B; sh[2][threadIdx.x] = Cc;
@@ -419,10 +540,23 @@ int log2_cols(const Shape& sh) {
   return lc;
 }
 
-template <typename R>
-int resample_blocks(const PlanConst& pc, const Shape& sh) {
-  const int covered = live_tiles(nb_bound(pc, (int64_t)1 << sh.log2n), sh.l2, log2_cols(sh), tile_log2<R>());
-  return (covered + kTilesPerBlock - 1) / kTilesPerBlock;
+// Tiles the grid covers per template, and the tiles each warp takes, by the
+// rounds of the 16 warps x 152 SMs that hold the kernel at once: up to four
+// rounds, as many as make it one round (a warp overlaps its next tile's loads
+// with the present one, and a second round would start over: one template of
+// 1,728,000 samples 32.5 -> 30.5 us); above, enough for six rounds, so that
+// the last one is short, and at most 8.
+struct TileGrid { int covered, per_warp, blocks; };
+TileGrid tile_grid(const PlanConst& pc, const Shape& sh, int nt) {
+  TileGrid g;
+  g.covered = live_tiles(nb_bound(pc, (int64_t)1 << sh.log2n), sh.l2);
+  const int64_t warps = 16 * 152;
+  const int64_t rounds = ((int64_t)g.covered * nt + warps - 1) / warps;
+  g.per_warp = (int)(rounds <= 4 ? rounds : rounds / 6 < 2 ? 2 : rounds / 6 > kMaxPerWarp ? kMaxPerWarp : rounds / 6);
+  if (g.per_warp < 1) g.per_warp = 1;
+  const int per_block = g.per_warp * kTileWarps;
+  g.blocks = (g.covered + per_block - 1) / per_block;
+  return g;
 }
 
 }  // namespace
@@ -430,38 +564,41 @@ int resample_blocks(const PlanConst& pc, const Shape& sh) {
 cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& sh, const float2* x,
                               const int64_t* gaps, const double* wcs, cudaStream_t s) {
   const int lc = log2_cols(sh);
+  const TileGrid tg = tile_grid(pc, sh, c.nt);
+  if (tg.blocks == 0) return cudaSuccess;
+  const dim3 grid((unsigned)tg.blocks, (unsigned)c.nt);
+  auto go = [&](auto kern) { kern<<<grid, kTileThreads, 0, s>>>(pc, c, sh.l2, lc, tg.per_warp, x, gaps, wcs); };
   if (pc.precision == FSTAT_PREC_FP64) {
-    dim3 grid((unsigned)resample_blocks<double>(pc, sh), (unsigned)c.nt);
-    if (grid.x == 0) return cudaSuccess;
-    if (pc.interp == FSTAT_NEAREST)
-      k_resample_t<double, FSTAT_NEAREST, 8><<<grid, kResThreads, 0, s>>>(pc, c, sh.l2, lc, x, gaps, wcs);
-    else if (pc.taps == 8)
-      k_resample_t<double, FSTAT_SINC, 8><<<grid, kResThreads, 0, s>>>(pc, c, sh.l2, lc, x, gaps, wcs);
-    else
-      k_resample_t<double, FSTAT_SINC, 0><<<grid, kResThreads, 0, s>>>(pc, c, sh.l2, lc, x, gaps, wcs);
-    return cudaGetLastError();
+    if (pc.interp == FSTAT_NEAREST) go(k_resample_t<double, FSTAT_NEAREST, 8>);
+    else if (pc.taps == 8) go(k_resample_t<double, FSTAT_SINC, 8>);
+    else go(k_resample_t<double, FSTAT_SINC, 0>);
+  } else if (pc.interp == FSTAT_SINC && pc.taps != 8) {
+    go(k_resample_t<float, FSTAT_SINC, 0>);
+  } else if (pc.log2h < 5) {
+    // knot intervals shorter than a tile's 32 columns
+    if (pc.interp == FSTAT_NEAREST) go(k_resample_t<float, FSTAT_NEAREST, 8>);
+    else go(k_resample_t<float, FSTAT_SINC, 8>);
+  } else {
+    // u - k moves by at most beta (1 + beta) a grid point: the linear form of
+    // the weights up to kRunNarrow over 3.5 points (the Earth's: 3.7e-4)
+    const double beta = pc.wo * pc.auc + pc.ws * pc.rc;
+    const bool quad = 3.5 * beta * (1.0 + 2.0 * beta) > 0.98 * kRunNarrow;
+    if (pc.interp == FSTAT_NEAREST) {
+      go(k_resample_run<RUN_NEAREST, true>);
+    } else if (pc.window == FSTAT_WIN_LANCZOS) {
+      if (quad) go(k_resample_run<RUN_LANCZOS, true>);
+      else go(k_resample_run<RUN_LANCZOS, false>);
+    } else {
+      if (quad) go(k_resample_run<RUN_RECT, true>);
+      else go(k_resample_run<RUN_RECT, false>);
+    }
   }
-  dim3 grid((unsigned)resample_blocks<float>(pc, sh), (unsigned)c.nt);
-  if (grid.x == 0) return cudaSuccess;
-  if (use_runs(pc, sh, lc)) {
-    k_resample_r8<<<grid, kResThreads, 0, s>>>(pc, c, sh.l2, lc, x, gaps, wcs);
-    return cudaGetLastError();
-  }
-  if (pc.interp == FSTAT_NEAREST)
-    k_resample_t<float, FSTAT_NEAREST, 8><<<grid, kResThreads, 0, s>>>(pc, c, sh.l2, lc, x, gaps, wcs);
-  else if (pc.taps == 8)
-    k_resample_t<float, FSTAT_SINC, 8><<<grid, kResThreads, 0, s>>>(pc, c, sh.l2, lc, x, gaps, wcs);
-  else
-    k_resample_t<float, FSTAT_SINC, 0><<<grid, kResThreads, 0, s>>>(pc, c, sh.l2, lc, x, gaps, wcs);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sums_t(const PlanConst& pc, const Chunk& c, const Shape& sh, int* status, cudaStream_t s) {
-  const bool d = pc.precision == FSTAT_PREC_FP64;
-  const int lp = d ? tile_log2<double>() : tile_log2<float>();
-  const int covered = (d ? resample_blocks<double>(pc, sh) : resample_blocks<float>(pc, sh)) * kTilesPerBlock;
-  const int per_tile = use_runs(pc, sh, log2_cols(sh)) ? kRunTR : 1;
-  k_sums_t<<<c.nt, kSumThreads, 0, s>>>(c, sh.l2, log2_cols(sh), lp, covered, per_tile, pc.sigma2, status);
+  const TileGrid tg = tile_grid(pc, sh, c.nt);
+  k_sums_t<<<c.nt, kSumThreads, 0, s>>>(c, sh.l2, tg.covered, tg.per_warp, pc.sigma2, status);
   return cudaGetLastError();
 }
 

@@ -14,17 +14,18 @@
 
 namespace fs {
 
-cudaError_t FS_CAT(rows, FS_REAL, FS_L2)(const RowsArgs<FS_REAL>& a, dim3 grid, cudaStream_t s) {
+cudaError_t FS_CAT(rows, FS_REAL, FS_L2)(const RowsArgs<FS_REAL>& a, int inplace, dim3 grid, cudaStream_t s) {
   using R = FS_REAL;
   constexpr int L2 = FS_L2;
   constexpr int RR = cols_for<points_b<R>()>(L2);
   constexpr int NT = threads_for<R>(L2, RR);
   constexpr size_t SM = rows_smem<R, L2, RR>();
-  auto kern = a.band ? k_rows<R, L2, RR, NT, true> : k_rows<R, L2, RR, NT, false>;
+  auto kern = inplace ? (a.band ? k_rows<R, L2, RR, NT, true, true> : k_rows<R, L2, RR, NT, false, true>)
+                      : (a.band ? k_rows<R, L2, RR, NT, true, false> : k_rows<R, L2, RR, NT, false, false>);
   // persistent grid: the blocks that fit on the device at once
-  static DeviceOnce once[2];
+  static DeviceOnce once[4];
   int resident = 0;
-  const cudaError_t e = kernel_setup(once[a.band ? 1 : 0], kern, NT, SM, &resident);
+  const cudaError_t e = kernel_setup(once[(a.band ? 1 : 0) + (inplace ? 2 : 0)], kern, NT, SM, &resident);
   if (e != cudaSuccess) return e;
   if (resident < 1) resident = 1;
   const unsigned total = grid.x * grid.y;
