@@ -239,11 +239,6 @@ constexpr int kRowSamples = 44;
 constexpr int kRowUnits = kRowSamples / 2;        // 16-byte pieces of two samples
 constexpr float kRunRotation = 0.125f;            // cycles: sincospi_small holds for |2 cycles| <= 1/4
 
-__device__ __forceinline__ void copy_async16(void* dst, const void* src, bool inside) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(inside ? 16 : 0) : "memory");
-}
-
 enum { RUN_NEAREST = 0, RUN_LANCZOS = 1, RUN_RECT = 2 };
 
 template <int KIND, bool QUAD>
@@ -579,10 +574,7 @@ cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& 
     if (pc.interp == FSTAT_NEAREST) go(k_resample_t<float, FSTAT_NEAREST, 8>);
     else go(k_resample_t<float, FSTAT_SINC, 8>);
   } else {
-    // u - k moves by at most beta (1 + beta) a grid point: the linear form of
-    // the weights up to kRunNarrow over 3.5 points (the Earth's: 3.7e-4)
-    const double beta = pc.wo * pc.auc + pc.ws * pc.rc;
-    const bool quad = 3.5 * beta * (1.0 + 2.0 * beta) > 0.98 * kRunNarrow;
+    const bool quad = runs_need_square(pc);
     if (pc.interp == FSTAT_NEAREST) {
       go(k_resample_run<RUN_NEAREST, true>);
     } else if (pc.window == FSTAT_WIN_LANCZOS) {

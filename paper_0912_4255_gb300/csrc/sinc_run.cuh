@@ -17,6 +17,8 @@
 // instructions and 8 reciprocals for weights formed point by point.
 #pragma once
 
+#include "fstat_internal.cuh"
+
 namespace fs {
 
 constexpr float kRunSpread = 1.5e-3f;
@@ -142,6 +144,20 @@ __device__ __forceinline__ void run_weights_d(float g, float (&w0)[8], float (&w
     w1[7 - p] = -w1[7 - p];
     FS_EVEN_ODD(sinc_d2<LANCZOS>, 5, p, g, t, w2[p], w2[7 - p]);
   }
+}
+
+// u - k moves by at most beta (1 + beta) samples a grid point: whether that
+// leaves the linear form of the weights (kRunNarrow over 3.5 points; the
+// Earth's motion gives 3.7e-4).
+inline bool runs_need_square(const PlanConst& pc) {
+  const double beta = pc.wo * pc.auc + pc.ws * pc.rc;
+  return 3.5 * beta * (1.0 + 2.0 * beta) > 0.98 * kRunNarrow;
+}
+
+// 16 bytes into shared memory, behind the thread's back; zeros if !inside.
+__device__ __forceinline__ void copy_async16(void* dst, const void* src, bool inside) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(inside ? 16 : 0) : "memory");
 }
 
 }  // namespace fs
