@@ -16,7 +16,7 @@ using namespace fs;
 namespace {
 constexpr int kKinds = 8;
 enum { K_TIMEMAP = 0, K_RESAMPLE = 1, K_COLS = 2, K_ROWS = 3, K_GRADF = 4, K_GRADB = 5, K_PERSIST = 6,
-       K_SUMS = 7 };
+       K_SUMS = 7 };    // K_SUMS: no kernel of its own any more (pass A does it)
 }
 
 struct fstat_plan_s {
@@ -420,7 +420,6 @@ int fstat_compute(fstat_plan_t p, const float* x_h, const fstat_template* t, int
     if (inplace) c.wa = c.za;
     cudaError_t e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, gaps, n_gaps_total, p->status, t0, s); });
     if (e == cudaSuccess) e = timed(p, K_RESAMPLE, s, [&] { return launch_resample_t(p->pc, c, p->sh, x, gaps, p->wcs, s); });
-    if (e == cudaSuccess) e = timed(p, K_SUMS, s, [&] { return launch_sums_t(p->pc, c, p->sh, p->status, s); });
     if (e == cudaSuccess) e = timed(p, K_COLS, s, [&] { return launch_cols_w(p->pc, c, p->sh, inplace, &p->twf, &p->twd, p->status, s); });
     if (e == cudaSuccess) e = timed(p, K_ROWS, s, [&] { return launch_rows_w(p->pc, c, p->sh, inplace, &p->twf, &p->twd, twoF, s); });
     if (e != cudaSuccess) return FSTAT_ECUDA;

@@ -70,6 +70,7 @@ static cudaError_t do_cols(const PlanConst& pc, const Chunk& c, const Shape& sh,
   a.tw = *reinterpret_cast<const Tw<R>*>(tw);
   const int tiles = (1 << sh.l2) / sh.cols;
   a.tiles_max = tiles;
+  a.covered = resample_covered(pc, sh);
   const dim3 grid((unsigned)tiles, (unsigned)c.nt);
   return cols_any<R>(a, sh.l1, inplace, grid, s);
 }

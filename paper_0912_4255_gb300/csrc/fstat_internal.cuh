@@ -40,6 +40,7 @@ struct PlanConst {
   double wo, ws;                                  // orbital and sidereal rates (rad/s)
   double th0;                                     // sidereal angle of the meridian at t = 0
   double inv_dt;                                  // 1 / dt
+  double beta;                                    // bound of |dt_m/dt|: orbital and diurnal speed over c
   // output band: 2F is written for bins band_lo <= q < band_hi only, at
   // out_off + q - band_lo
   int64_t band_lo, band_hi;
@@ -50,6 +51,9 @@ struct PlanConst {
 struct TmplMeta {
   double tb0;        // t_b of grid point 0
   double A, B, C;    // masked antenna sums (Eq. 9 as sums)
+  // the same while the tiled resampler adds them up, in units of 2^-32: whole
+  // numbers, so that the order of the warps' additions does not matter
+  unsigned long long acc[3];
   int64_t n_b;       // resampled length N_b
   int64_t out_off;   // output offset in floats
   int64_t span_lo, span_hi, gap_off, n_gaps;
@@ -193,12 +197,10 @@ struct Sky {
   R e0, e1, e2, e3, e4, f1, f2, f3, f4;
 };
 
+// sa, ca, sd, cd: sines and cosines of alpha and delta
 template <typename R>
-__device__ __forceinline__ Sky<R> make_sky(const PlanConst& pc, R alpha, R delta) {
+__device__ __forceinline__ Sky<R> make_sky(const PlanConst& pc, R alpha, R sa, R ca, R sd, R cd) {
   Sky<R> s;
-  R sa, ca, sd, cd;
-  if constexpr (std::is_same<R, float>::value) { sincosf(alpha, &sa, &ca); sincosf(delta, &sd, &cd); }
-  else { sincos(alpha, &sa, &ca); sincos(delta, &sd, &cd); }
   s.nx = cd * ca; s.ny = cd * sa; s.nz = sd;
   const R auc = (R)pc.auc;
   s.ox = auc * s.nx;                         // coefficient of cos(phi)
@@ -225,6 +227,14 @@ __device__ __forceinline__ Sky<R> make_sky(const PlanConst& pc, R alpha, R delta
 template <typename R>
 __device__ __forceinline__ void rsincos(R x, R* s, R* c) {
   if constexpr (std::is_same<R, float>::value) sincosf(x, s, c); else sincos(x, s, c);
+}
+
+template <typename R>
+__device__ __forceinline__ Sky<R> make_sky(const PlanConst& pc, R alpha, R delta) {
+  R sa, ca, sd, cd;
+  rsincos<R>(alpha, &sa, &ca);
+  rsincos<R>(delta, &sd, &cd);
+  return make_sky<R>(pc, alpha, sa, ca, sd, cd);
 }
 
 // t_m(t) and dt_m/dt; sH, cH: sin and cos of the hour angle theta(t) - alpha.
@@ -283,7 +293,20 @@ template <typename R>
 __device__ __forceinline__ void advance(R a, R d, R* s, R* c) {
   if (fabs(d) <= (R)0.1) {
     R sd, cd;
-    sincos_small<R>(d, &sd, &cd);
+    if (fabs(d) <= (R)1e-3) {
+      // the same series to x^5 and x^6: the terms left out are below 1e-24
+      const R x2 = d * d;
+      sd = d * (1 - x2 * (R)(1.0 / 6) * (1 - x2 * (R)(1.0 / 20)));
+      cd = 1 - x2 * (R)0.5 * (1 - x2 * (R)(1.0 / 12) * (1 - x2 * (R)(1.0 / 30)));
+    } else if (fabs(d) <= (R)2e-2) {
+      // to x^9 and x^8: below 1e-20
+      const R x2 = d * d;
+      sd = d * (1 - x2 * (R)(1.0 / 6) * (1 - x2 * (R)(1.0 / 20) * (1 - x2 * (R)(1.0 / 42) * (1 - x2 * (R)(1.0 / 72)))));
+      cd = 1 - x2 * (R)0.5 * (1 - x2 * (R)(1.0 / 12) * (1 - x2 * (R)(1.0 / 30) * (1 - x2 * (R)(1.0 / 56) *
+           (1 - x2 * (R)(1.0 / 90)))));
+    } else {
+      sincos_small<R>(d, &sd, &cd);
+    }
     const R s0 = *s, c0 = *c;
     *s = s0 * cd + c0 * sd;
     *c = c0 * cd - s0 * sd;
@@ -1059,6 +1082,12 @@ struct Shape {
   int log2n, l1, l2, cols, rows;
 };
 
+// The resampler's tiles (8 rows x 32 columns) of the row tiles with a point
+// below n_b.
+__host__ __device__ __forceinline__ int live_tiles(int64_t n_b, int l2) {
+  return n_b <= 0 ? 0 : (int)(((n_b - 1) >> (l2 + 3)) + 1) << (l2 - 5);
+}
+
 // Default factorisation N = N1 N2 of the four-step FFT: the longest first
 // pass (N1 <= 2^12, N2 >= 2^6), so that a second-pass block holds as many
 // rows as its shared memory allows and its 2F stores form longer runs.
@@ -1096,7 +1125,7 @@ cudaError_t launch_resample_w(const PlanConst& pc, const Chunk& c, int ti, int l
                               cudaStream_t s);
 cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& sh, const float2* x,
                               const int64_t* gaps, const double* wcs, cudaStream_t s);
-cudaError_t launch_sums_t(const PlanConst& pc, const Chunk& c, const Shape& sh, int* status, cudaStream_t s);
+int resample_covered(const PlanConst& pc, const Shape& sh);
 cudaError_t launch_cols_w(const PlanConst& pc, const Chunk& c, const Shape& sh, int inplace, const void* twf,
                           const void* twd, int* status, cudaStream_t s);
 cudaError_t launch_rows_w(const PlanConst& pc, const Chunk& c, const Shape& sh, int inplace, const void* twf,
@@ -1124,6 +1153,7 @@ inline void derive_constants(PlanConst& pc) {
   pc.wo = kTwoPi / pc.year; pc.ws = kTwoPi / pc.sid;
   pc.th0 = pc.sid0 + pc.lon;
   pc.inv_dt = 1.0 / pc.dt;
+  pc.beta = pc.wo * pc.auc + pc.ws * pc.rc;
 }
 
 // Host-side validation of a plan descriptor: FSTAT_OK or the error code

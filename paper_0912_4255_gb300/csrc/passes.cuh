@@ -42,6 +42,7 @@ struct ColsArgs {
   const double* wcs;
   Tw<R> tw;
   int tiles_max; // column tiles of one template
+  int covered;   // tiles per template that the resampling grid covered
   int* status;
   int rr, log2rr; // rows per block of the second pass (layout of Z)
 };
@@ -291,6 +292,24 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
   }
 }
 
+// A, B, C of template t and the coefficients of 2F from the resampler's sums
+// (one thread of the block that has the template's first column tile; the
+// second pass, which needs them, starts after this one).  A template with
+// more tiles below n_b than the resampling grid covered (not expected: the
+// grid is sized from a bound on n_b) is reported as FSTAT_ERANGE.
+template <typename R>
+__device__ __forceinline__ void finish_sums(const ColsArgs<R>& a, int t, int l2) {
+  TmplMeta* m = a.c.meta + t;
+  if (live_tiles(m->n_b, l2) > a.covered) {
+    m->status = FSTAT_ERANGE;
+    set_status(a.status, FSTAT_ERANGE);
+    return;
+  }
+  constexpr double u = 1.0 / 4294967296.0;
+  set_sums(m, u * (double)(long long)m->acc[0], u * (double)(long long)m->acc[1], u * (double)(long long)m->acc[2],
+           a.pc.sigma2, nullptr, a.status);
+}
+
 // Persistent over the (template, column tile) items of a chunk: the grid is
 // sized to the resident blocks, each builds the stage tables once.
 template <typename R, int L1, int C, int NT, int SRC, int TAPS>
@@ -326,6 +345,9 @@ __global__ void __launch_bounds__(NT, (min_blocks<R>(NT, cols_smem<R, L1, C>()))
     if (tile >= (1 << (m.log2n - L1)) / C || m.status != FSTAT_OK) continue;
     Pair<R>* za = reinterpret_cast<Pair<R>*>(a.c.za) + (int64_t)t * a.c.z_stride;
     cols_tile<R, L1, C, NT, SRC, TAPS>(a, t, tile, buf, red, za, a.rr, a.log2rr);
+    if constexpr (loads(SRC)) {
+      if (tile == 0 && threadIdx.x == 0) finish_sums<R>(a, t, m.log2n - L1);
+    }
     __syncthreads();                      // the next tile reuses buf and its twiddle factors
   }
 }

@@ -83,17 +83,12 @@ cudaError_t dispatch(const PlanConst& pc, const Chunk& c, int ti, int log2n, con
 // numbered by row tile, then column tile; those of the row tiles with a point
 // below n_b are done, and the first pass reads every point at k >= n_b as
 // zero without loading it.  A warp takes per_warp consecutive tiles and
-// leaves one partial sum of A, B, C; k_sums_t reduces them.
+// adds its part of A, B, C to the template's.
 constexpr int kTileRows = 8, kTileCols = 32;
 constexpr int kTilePts = kTileRows * kTileCols;
 constexpr int kTileWarps = 4;                       // warps per block
 constexpr int kTileThreads = 32 * kTileWarps;
 constexpr int kMaxPerWarp = 8;
-
-// tiles of the row tiles with a point below n_b
-__host__ __device__ __forceinline__ int live_tiles(int64_t n_b, int l2) {
-  return n_b <= 0 ? 0 : (int)(((n_b - 1) >> (l2 + 3)) + 1) << (l2 - 5);
-}
 
 // Position of (row, col) in a warp's tile: rows of 32 pairs, the low three
 // bits of the column xored with a key of the row and the column's group of
@@ -130,16 +125,23 @@ __device__ __forceinline__ void store_tile(Pair<R>* __restrict__ w_out, const Pa
   }
 }
 
-// The warp's partial sum of A, B, C (a barrier over the block's warps would
-// hold them until the slowest is done).
-__device__ __forceinline__ void warp_partial(float pa, float pb, float pcc, double* __restrict__ part) {
+// Adds the warp's sums of a^2, b^2, a b to the template's (|a|, |b| <= 2: the
+// whole numbers stay below 2^59 for 2^24 points).  One atomic addition per
+// warp and sum: partial sums in memory and a kernel to reduce them took 10 us
+// of every call, a barrier over the block's warps held them until the slowest
+// was done.
+__device__ __forceinline__ void add_sums(float pa, float pb, float pcc, TmplMeta* m) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    pa += __shfl_down_sync(0xffffffffu, pa, o);
-    pb += __shfl_down_sync(0xffffffffu, pb, o);
-    pcc += __shfl_down_sync(0xffffffffu, pcc, o);
+    pa += __shfl_xor_sync(0xffffffffu, pa, o);
+    pb += __shfl_xor_sync(0xffffffffu, pb, o);
+    pcc += __shfl_xor_sync(0xffffffffu, pcc, o);
   }
-  if ((threadIdx.x & 31) == 0) { part[0] = pa; part[1] = pb; part[2] = pcc; }
+  const int lane = threadIdx.x & 31;
+  if (lane < 3) {
+    const float v = lane == 0 ? pa : (lane == 1 ? pb : pcc);
+    atomicAdd(&m->acc[lane], (unsigned long long)__double2ll_rn((double)v * 4294967296.0));
+  }
 }
 
 // Other tap counts, FP64 (and knot intervals of fewer than 32 points): one point per lane and row (32
@@ -187,7 +189,7 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* 
     store_tile<R>(w_out, so, c0, r0, lc, gstride, lane);
     __syncwarp();                             // before the next tile overwrites so
   }
-  warp_partial(pa, pb, pcc, c.partials + ((int64_t)t * c.part_stride + wid) * 3);
+  add_sums(pa, pb, pcc, c.meta + t);
 }
 
 // One point of a run that cannot take the shared tap run (a slip, a gap or
@@ -482,48 +484,14 @@ k_resample_run(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2
     k0 = k0n; n0 = n0n; base = basen; s = sn_; f = fn_;
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  warp_partial(pa, pb, pcc, c.partials + ((int64_t)t * c.part_stride + wid) * 3);
-}
-
-// One block per template: A, B, C from the partials of its warps, summed in
-// FP64 in a fixed order (deterministic).  covered: tiles the resampling grid
-// reached; a template with more tiles below n_b (not expected: the grid is
-// sized from a bound on n_b) is reported as FSTAT_ERANGE.
-constexpr int kSumThreads = 256;
-__global__ void __launch_bounds__(kSumThreads)
-k_sums_t(Chunk c, int l2, int covered, int per_warp, double sigma2, int* status) {
-  __shared__ double sh[3][kSumThreads];
-  TmplMeta* m = c.meta + blockIdx.x;
-  if (m->status != FSTAT_OK) return;
-  const int nlive = live_tiles(m->n_b, l2);
-  if (nlive > covered) {
-    if (threadIdx.x == 0) { m->status = FSTAT_ERANGE; set_status(status, FSTAT_ERANGE); }
-    return;
-  }
-  const double* part = c.partials + (int64_t)blockIdx.x * c.part_stride * 3;
-  const int nparts = (nlive + per_warp - 1) / per_warp;
-  double A = 0, B = 0, Cc = 0;
-  for (int i = threadIdx.x; i < nparts; i += kSumThreads) {
-    A += part[3 * i]; B += part[3 * i + 1]; Cc += part[3 * i + 2];
-  }
-  sh[0][threadIdx.x] = A; sh[1][threadIdx.x] = B; sh[2][threadIdx.x] = Cc;
-  __syncthreads();
-  for (int h = kSumThreads / 2; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) {
-      sh[0][threadIdx.x] += sh[0][threadIdx.x + h];
-      sh[1][threadIdx.x] += sh[1][threadIdx.x + h];
-      sh[2][threadIdx.x] += sh[2][threadIdx.x + h];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) set_sums(m, sh[0][0], sh[1][0], sh[2][0], sigma2, nullptr, status);
+  add_sums(pa, pb, pcc, c.meta + t);
 }
 
 // Upper bound on n_b for every template of the plan: t_b = t + t_m(t) and
 // |dt_m/dt| <= (2 pi / year) au / c + (2 pi / sidereal day) R / c, so a span
 // of n_data samples maps to at most (n_data - 1)(1 + beta) + 1 grid points.
 int64_t nb_bound(const PlanConst& pc, int64_t n_fft) {
-  const double beta = pc.wo * pc.auc + pc.ws * pc.rc;
+  const double beta = pc.beta;
   const double b = (double)(pc.n_data - 1) * (1.0 + 1.01 * beta + 1e-12) + 3.0;
   const int64_t nb = (int64_t)b;
   return nb < n_fft ? nb : n_fft;
@@ -541,16 +509,16 @@ int log2_cols(const Shape& sh) {
 // with the present one, and a second round would start over: one template of
 // 1,728,000 samples 32.5 -> 30.5 us); above, enough for six rounds, so that
 // the last one is short, and at most 8.
-struct TileGrid { int covered, per_warp, blocks; };
+struct TileGrid { int per_warp, blocks; };
 TileGrid tile_grid(const PlanConst& pc, const Shape& sh, int nt) {
   TileGrid g;
-  g.covered = live_tiles(nb_bound(pc, (int64_t)1 << sh.log2n), sh.l2);
+  const int covered = resample_covered(pc, sh);
   const int64_t warps = 16 * 152;
-  const int64_t rounds = ((int64_t)g.covered * nt + warps - 1) / warps;
+  const int64_t rounds = ((int64_t)covered * nt + warps - 1) / warps;
   g.per_warp = (int)(rounds <= 4 ? rounds : rounds / 6 < 2 ? 2 : rounds / 6 > kMaxPerWarp ? kMaxPerWarp : rounds / 6);
   if (g.per_warp < 1) g.per_warp = 1;
   const int per_block = g.per_warp * kTileWarps;
-  g.blocks = (g.covered + per_block - 1) / per_block;
+  g.blocks = (covered + per_block - 1) / per_block;
   return g;
 }
 
@@ -588,10 +556,9 @@ cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& 
   return cudaGetLastError();
 }
 
-cudaError_t launch_sums_t(const PlanConst& pc, const Chunk& c, const Shape& sh, int* status, cudaStream_t s) {
-  const TileGrid tg = tile_grid(pc, sh, c.nt);
-  k_sums_t<<<c.nt, kSumThreads, 0, s>>>(c, sh.l2, tg.covered, tg.per_warp, pc.sigma2, status);
-  return cudaGetLastError();
+// Tiles per template that the resampling grid covers.
+int resample_covered(const PlanConst& pc, const Shape& sh) {
+  return live_tiles(nb_bound(pc, (int64_t)1 << sh.log2n), sh.l2);
 }
 
 // out_double: 0 -> complex64 output, 1 -> complex128 output (FP64 internal buffers)

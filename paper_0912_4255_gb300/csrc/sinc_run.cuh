@@ -150,7 +150,7 @@ __device__ __forceinline__ void run_weights_d(float g, float (&w0)[8], float (&w
 // leaves the linear form of the weights (kRunNarrow over 3.5 points; the
 // Earth's motion gives 3.7e-4).
 inline bool runs_need_square(const PlanConst& pc) {
-  const double beta = pc.wo * pc.auc + pc.ws * pc.rc;
+  const double beta = pc.beta;
   return 3.5 * beta * (1.0 + 2.0 * beta) > 0.98 * kRunNarrow;
 }
 
