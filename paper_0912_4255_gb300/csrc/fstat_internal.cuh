@@ -578,6 +578,72 @@ __device__ __forceinline__ bool sinc8_f32(const float2* __restrict__ x, GapCurso
   return true;
 }
 
+// sin and cos of pi x for |x| <= 1/4 by their Taylor series (terms to x^17 and
+// x^16; truncation below 4e-20), double precision.  The FP64 pipe is what the
+// double-precision resampler waits for, so its elementary functions are kept
+// to what their arguments need.
+__device__ __forceinline__ void sincospi_small(double x, double* s, double* c) {
+  const double t = 3.14159265358979323846 * x;
+  const double u = t * t;
+  *s = t * fma(u, fma(u, fma(u, fma(u, fma(u, fma(u, fma(u, fma(u, 1.0 / 355687428096000.0, -1.0 / 1307674368000.0),
+           1.0 / 6227020800.0), -1.0 / 39916800.0), 1.0 / 362880.0), -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0), 1.0);
+  *c = fma(u, fma(u, fma(u, fma(u, fma(u, fma(u, fma(u, fma(u, 1.0 / 20922789888000.0, -1.0 / 87178291200.0),
+           1.0 / 479001600.0), -1.0 / 3628800.0), 1.0 / 40320.0), -1.0 / 720.0), 1.0 / 24.0), -0.5), 1.0);
+}
+
+// exp(-2 pi i r) for |r| <= 1/2, as the single-precision form.
+__device__ __forceinline__ double2 expm2pi(double r) {
+  const double q = rint(4.0 * r);
+  double sn, cs;
+  sincospi_small(2.0 * fma(-0.25, q, r), &sn, &cs);
+  const int qi = (int)q & 3;
+  double re = cs, im = -sn;
+  if (qi & 1) { const double t = re; re = im; im = -t; }   // times -i
+  if (qi & 2) { re = -re; im = -im; }                      // times -1
+  return make_double2(re, im);
+}
+
+// The weights of the 8-tap windowed sinc in double precision at the fraction
+// f (x_i = f + 3 - i, dn = f or f - 1 the offset from the nearest sample, not
+// 0).  The products x_i x_{7-i} = f (f - 1) - (0, 2, 6, 12) share one
+// reciprocal, and 1 / x_i = x_{7-i} / (x_i x_{7-i}); sin(pi x_i) and
+// sin(pi x_i / 4) come from sin, cos(pi dn / 4): about 75 FP64 operations
+// where eight divisions and two sincospi took over 200.
+__device__ __forceinline__ void sinc8_weights(double f, double dn, int qoff, bool lanczos, double (&w)[8]) {
+  double sh, ch;
+  sincospi_small(0.25 * dn, &sh, &ch);
+  const double s2 = 2.0 * sh * ch, c2 = fma(ch, ch, -sh * sh);
+  const double sdn = 2.0 * s2 * c2;
+  const double sf = qoff ? -sdn : sdn;                     // sin(pi f)
+  const double q = f * (qoff ? dn : f - 1.0);              // f (f - 1): both factors exact
+  const double q1 = q - 2.0, q2 = q - 6.0, q3 = q - 12.0;
+  const double p01 = q * q1, p23 = q2 * q3;
+  const double r = __drcp_rn(p01 * p23);
+  const double r01 = r * p23, r23 = r * p01;
+  const double ip[4] = {r23 * q2, r23 * q3, r01 * q, r01 * q1};   // 1 / (x_i x_{7-i}), i = 0 .. 3
+  double ix[8];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const double xa = i == 3 && qoff == 0 ? dn : f + (double)(3 - i);
+    const double xb = i == 3 && qoff ? dn : f + (double)(i - 4);
+    ix[i] = xb * ip[i];
+    ix[7 - i] = xa * ip[i];
+  }
+  if (lanczos) {
+    const double r2 = 0.70710678118654752440;
+    const double p = (sh + ch) * r2, m = (ch - sh) * r2;
+    const double k = sf * (4.0 / (3.14159265358979323846 * 3.14159265358979323846));
+    // (-1)^(3-i) sin(pi x_i / 4) for i = 0 .. 3; taps 4 .. 7 take the negatives
+    const double g[4] = {-k * (qoff ? -sh : m), k * (qoff ? m : ch), -k * (qoff ? ch : p), k * (qoff ? p : sh)};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = (i < 4 ? g[i & 3] : -g[i & 3]) * (ix[i] * ix[i]);
+  } else {
+    const double k = sf * (1.0 / 3.14159265358979323846);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = (((3 - i) & 1) ? -k : k) * ix[i];
+  }
+}
+
 // Phase P + ((p3 s + p2) s + p1) s of a knot interval, mod 1: the linear
 // term reaches many cycles at the end of an interval, so its whole cycles come
 // off exactly before the terms are added.
@@ -635,6 +701,39 @@ __device__ __forceinline__ bool sample_weights(
       wa = czero<C>(); wb = czero<C>(); return false;
     }
     z = zz;
+  } else if constexpr (std::is_same<R, double>::value && INTERP == FSTAT_SINC && TAPS == 8) {
+    const int qoff = dev >= 0.5 ? 1 : 0;
+    const double dn = qoff ? dev - 1.0 : dev;   // dev = u - floor(u)
+    const int jlo = ibase - 3, jnn = ibase + qoff;
+    if (dn == 0.0) {
+      // u on a sample: the interpolant is that sample
+      if (!gc.valid(jnn)) { wa = czero<C>(); wb = czero<C>(); return false; }
+      z = ldx<R>(x, jnn);
+    } else {
+      const bool full = gc.window_valid(jlo, jlo + 7);
+      float2 v[8];
+      if (full) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = __ldg(x + jlo + i);
+      }
+      double w[8];
+      sinc8_weights(dev, dn, qoff, pc.window == FSTAT_WIN_LANCZOS, w);
+      double2 acc = make_double2(0.0, 0.0);
+      bool msk = full;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float2 t = v[i];
+        if (!full) {
+          const bool ok = gc.valid(jlo + i);
+          if (jlo + i == jnn) msk = ok;
+          t = ok ? __ldg(x + jlo + i) : make_float2(0.f, 0.f);
+        }
+        acc.x = fma(w[i], (double)t.x, acc.x);
+        acc.y = fma(w[i], (double)t.y, acc.y);
+      }
+      if (!msk) { wa = czero<C>(); wb = czero<C>(); return false; }
+      z = acc;
+    }
   } else {
   int jnn_off;                        // jnn - ibase = floor(dev + 1/2)
   R jnn_f;
@@ -774,10 +873,7 @@ __device__ __forceinline__ bool sample_weights(
     const float r = ph - round_nearest(ph, &dummy);
     e = expm2pi(r);
   } else {
-    const R r = ph - rint(ph);
-    R sp, cp;
-    sincospi(2.0 * r, &sp, &cp);
-    e = cmk<C, R>(cp, -sp);
+    e = expm2pi(ph - rint(ph));
   }
   const C y = cmul(z, e);
   wa = cmk<C, R>(a * y.x, a * y.y);
