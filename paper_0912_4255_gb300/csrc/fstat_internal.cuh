@@ -918,52 +918,43 @@ struct Dft {
   }
 };
 
-// padded shared-memory index: one extra element every 16 avoids bank
-// conflicts of the stride-16 writes of the first radix-16 stage
-__device__ __forceinline__ int pidx(int e) { return e + (e >> 4); }
+// A transform of N = 16 RM RL points in shared memory, in place.  With
+//   k = lo + RL (mid + RM hi)   and   p = p0 + 16 (q1 + RM q2)
+// its stages run over hi (radix 16), mid (radix RM, if any) and lo (radix RL),
+// and a butterfly's outputs take the places of its inputs, [p0][q1][lo]: only
+// one barrier lies between two stages, where writing a stage in transform
+// order needs a second one between its reads and its writes.  The low bits of a place are
+// xored with its first digit, so that the accesses of a quarter-warp (8
+// lanes of 16 bytes), which run over lo in the first two stages and over p0
+// in the last, fall on distinct banks without padding.
+// With COUNT >= 8 interleaved sequences the lanes run over these, on distinct
+// banks by their stride, and the key is left out.
+template <int LOGN, int RBL, int COUNT> struct FftPlan {
+  static constexpr int RBM = LOGN - 4 - RBL;
+  static constexpr int RM = 1 << RBM, RL = 1 << RBL;
+  static constexpr int SUB = RM * RL;               // points of one hi digit: N / 16
+  static constexpr int KEYS = COUNT >= 8 ? 0 : (SUB < 8 ? SUB - 1 : 7);
+  static __device__ __forceinline__ int key(int hi) { return hi & KEYS; }
+  // place of (hi, j), j = mid RL + lo
+  static __device__ __forceinline__ int place(int hi, int j) { return hi * SUB + (j ^ key(hi)); }
+};
 // Sequence stride in shared memory, in pairs.  Fills and epilogues interleave
-// C sequences across the lanes of a quarter-warp (8 lanes of 16-byte
-// accesses); a stride congruent to 8/C mod 8 puts them on distinct banks.
+// C sequences across the lanes of a quarter-warp; a stride congruent to 8/C
+// mod 8 puts them on distinct banks.
 template <int LOGN, int C> struct FftGeom {
   static constexpr int N = 1 << LOGN;
-  static constexpr int BASE = N + (N >> 4);
   static constexpr int WANT = C >= 8 ? 1 : 8 / C;
-  static constexpr int STRIDE = BASE + ((WANT - (BASE & 7)) & 7);
+  static constexpr int STRIDE = N + (WANT & 7);
 };
 
-// Twiddles of the Stockham stages, held in shared memory.  The stage of
-// radix 2^RB after sub-transforms of length NS = 2^NSL multiplies input r of
-// butterfly k (k < NS) by W_{NS 2^RB}^{r k}; its table is laid out [r - 1][k]
-// (r = 1 .. 2^RB - 1), so that lanes with consecutive k read consecutive
-// entries.  The first stage (NS = 1) needs none.
-template <int NSL, int RB> constexpr int stage_tw_count() { return NSL > 0 ? ((1 << RB) - 1) << NSL : 0; }
-// radix of the stage after sub-transforms 2^NSL when the stages run to 2^NSL_END
-template <int NSL, int NSL_END> constexpr int mid_rb() { return NSL_END - NSL >= 4 ? 4 : NSL_END - NSL; }
-template <int NSL, int NSL_END> constexpr int mid_tw_count() {
-  if constexpr (NSL < NSL_END) {
-    constexpr int RB = mid_rb<NSL, NSL_END>();
-    return stage_tw_count<NSL, RB>() + mid_tw_count<NSL + RB, NSL_END>();
-  } else {
-    return 0;
-  }
-}
-
-// Fill the table of one stage from the length-2^LOGN table tw (all threads).
-template <typename R, int LOGN, int NSL, int RB, int NT>
-__device__ __forceinline__ void build_stage_tw(cpx<R>* __restrict__ dst, const cpx<R>* __restrict__ tw) {
-  constexpr int CNT = stage_tw_count<NSL, RB>();
-  for (int e = threadIdx.x; e < CNT; e += NT) {
-    const int r = (e >> NSL) + 1, k = e & ((1 << NSL) - 1);
-    dst[e] = __ldg(tw + ((r * k) << (LOGN - NSL - RB)));
-  }
-}
-template <typename R, int LOGN, int NSL, int NSL_END, int NT>
+// Twiddles of the middle stage, held in shared memory: input mid = r of the
+// butterfly (p0, lo) takes W_{16 RM}^{r p0}, table [r - 1][p0], r = 1 .. RM - 1.
+constexpr int mid_tw_count(int rbm) { return ((1 << rbm) - 1) << 4; }
+// Filled from the length-2^LOGN table tw (all threads).
+template <typename R, int LOGN, int RBM, int NT>
 __device__ __forceinline__ void build_mid_tw(cpx<R>* __restrict__ dst, const cpx<R>* __restrict__ tw) {
-  if constexpr (NSL < NSL_END) {
-    constexpr int RB = mid_rb<NSL, NSL_END>();
-    build_stage_tw<R, LOGN, NSL, RB, NT>(dst, tw);
-    build_mid_tw<R, LOGN, NSL + RB, NSL_END, NT>(dst + stage_tw_count<NSL, RB>(), tw);
-  }
+  for (int e = threadIdx.x; e < mid_tw_count(RBM); e += NT)
+    dst[e] = __ldg(tw + ((((e >> 4) + 1) * (e & 15)) << (LOGN - 4 - RBM)));
 }
 // The last stage (radix 2^RB at NS = 2^NSL, LOGN = NSL + RB) keeps only the
 // powers W^k, W^{2k}, W^{4k}, ...: row p holds W_{2^LOGN}^{2^p k}, k < NS.  A
@@ -991,82 +982,62 @@ __device__ __forceinline__ void last_twiddles(const cpx<R>* __restrict__ lt, cpx
   }
 }
 
-// One Stockham stage of radix 2^RB over COUNT pairs of sequences of length
-// 2^LOGN in shared memory (pair f at buf + f * STRIDE, padded); NS = 2^NSL is
-// the length of the sub-transforms already done; tws: this stage's twiddle
-// table.  Every thread handles UPT units of 16 points of both series; all
-// reads happen before the barrier, all writes after it.
-template <typename R, int LOGN, int RB, int NSL, int NT, int COUNT, int STRIDE>
-__device__ __forceinline__ void stockham_stage(Pair<R>* __restrict__ buf, const cpx<R>* __restrict__ tws) {
+// The first stage in shared memory (persistent mode; elsewhere its inputs come
+// from global memory) over COUNT interleaved sequences f at buf + f * STRIDE.
+template <typename R, int LOGN, int RBL, int NT, int COUNT, int STRIDE>
+__device__ __forceinline__ void first_stage(Pair<R>* __restrict__ buf) {
   using C = cpx<R>;
-  constexpr int N = 1 << LOGN;
-  constexpr int RAD = 1 << RB;
-  constexpr int BPU = 16 / RAD;                   // butterflies per 16-point unit
-  constexpr int UNITS_PER_SEQ = N / 16;
-  constexpr int UNITS = COUNT * UNITS_PER_SEQ;
-  constexpr int UPT = (UNITS + NT - 1) / NT;
-  constexpr int NS = 1 << NSL;
-  C va[UPT][16], vb[UPT][16];
+  using P = FftPlan<LOGN, RBL, COUNT>;
+#pragma unroll 1
+  for (int u = threadIdx.x; u < COUNT * P::SUB; u += NT) {
+    Pair<R>* x = buf + (u % COUNT) * STRIDE;
+    const int j = u / COUNT;
+    C va[16], vb[16];
 #pragma unroll
-  for (int u = 0; u < UPT; ++u) {
-    const int unit = threadIdx.x + u * NT;
-    if (UNITS % NT == 0 || unit < UNITS) {
-      const int f = unit / UNITS_PER_SEQ;
-      const int w = unit - f * UNITS_PER_SEQ;
-      const Pair<R>* src = buf + f * STRIDE;
+    for (int r = 0; r < 16; ++r) { const Pair<R> v = x[P::place(r, j)]; va[r] = v.a; vb[r] = v.b; }
+    Dft<C, 16>::run(va);
+    Dft<C, 16>::run(vb);
 #pragma unroll
-      for (int bb = 0; bb < BPU; ++bb) {
-        const int j = w + bb * UNITS_PER_SEQ;     // lanes take consecutive butterflies
-        const int k = j & (NS - 1);
-#pragma unroll
-        for (int r = 0; r < RAD; ++r) {
-          const Pair<R> x = src[pidx(j + r * (N / RAD))];
-          C xa = x.a, xb = x.b;
-          if constexpr (NSL > 0) {
-            if (r > 0) {
-              const C t = tws[((r - 1) << NSL) + k];
-              xa = cmul(xa, t);
-              xb = cmul(xb, t);
-            }
-          }
-          va[u][bb * RAD + r] = xa;
-          vb[u][bb * RAD + r] = xb;
-        }
-        Dft<C, RAD>::run(&va[u][bb * RAD]);
-        Dft<C, RAD>::run(&vb[u][bb * RAD]);
-      }
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int u = 0; u < UPT; ++u) {
-    const int unit = threadIdx.x + u * NT;
-    if (UNITS % NT == 0 || unit < UNITS) {
-      const int f = unit / UNITS_PER_SEQ;
-      const int w = unit - f * UNITS_PER_SEQ;
-      Pair<R>* dst = buf + f * STRIDE;
-#pragma unroll
-      for (int bb = 0; bb < BPU; ++bb) {
-        const int j = w + bb * UNITS_PER_SEQ;
-        const int k = j & (NS - 1);
-        const int base = ((j >> NSL) << (NSL + RB)) + k;
-#pragma unroll
-        for (int r = 0; r < RAD; ++r) dst[pidx(base + r * NS)] = Pair<R>{va[u][bb * RAD + r], vb[u][bb * RAD + r]};
-      }
-    }
+    for (int r = 0; r < 16; ++r) x[P::place(r, j)] = Pair<R>{va[r], vb[r]};
   }
   __syncthreads();
 }
 
-// Stages from sub-transform length 2^NSL up to 2^NSL_END (radix 16 while
-// possible); the stages before and after are done by the caller.  tws: the
-// tables of these stages, one after the other (build_mid_tw).
-template <typename R, int LOGN, int NSL, int NSL_END, int NT, int COUNT, int STRIDE>
-__device__ __forceinline__ void fft_mid_stages(Pair<R>* buf, const cpx<R>* tws) {
-  if constexpr (NSL < NSL_END) {
-    constexpr int RB = mid_rb<NSL, NSL_END>();
-    stockham_stage<R, LOGN, RB, NSL, NT, COUNT, STRIDE>(buf, tws);
-    fft_mid_stages<R, LOGN, NSL + RB, NSL_END, NT, COUNT, STRIDE>(buf, tws + stage_tw_count<NSL, RB>());
+// The middle stage: butterflies (p0, lo) over mid, twiddles tws
+// (build_mid_tw); lanes run over the sequences, then lo, then p0.
+template <typename R, int LOGN, int RBL, int NT, int COUNT, int STRIDE>
+__device__ __forceinline__ void mid_stage(Pair<R>* __restrict__ buf, const cpx<R>* __restrict__ tws) {
+  using C = cpx<R>;
+  using P = FftPlan<LOGN, RBL, COUNT>;
+  if constexpr (P::RBM > 0) {
+    constexpr int UNITS = COUNT * 16 * P::RL;
+#pragma unroll
+    for (int u0 = 0; u0 < UNITS; u0 += NT) {
+      const int u = u0 + threadIdx.x;
+      if (UNITS % NT == 0 || u < UNITS) {
+        const int b = u / COUNT;
+        const int lo = b & (P::RL - 1), p0 = b >> RBL;
+        Pair<R>* x = buf + (u % COUNT) * STRIDE + p0 * P::SUB;
+        const int o = lo ^ P::key(p0);
+        C va[P::RM], vb[P::RM];
+#pragma unroll
+        for (int r = 0; r < P::RM; ++r) {
+          const Pair<R> v = x[o + r * P::RL];
+          va[r] = v.a;
+          vb[r] = v.b;
+          if (r > 0) {
+            const C w = tws[((r - 1) << 4) + p0];
+            va[r] = cmul(va[r], w);
+            vb[r] = cmul(vb[r], w);
+          }
+        }
+        Dft<C, P::RM>::run(va);
+        Dft<C, P::RM>::run(vb);
+#pragma unroll
+        for (int r = 0; r < P::RM; ++r) x[o + r * P::RL] = Pair<R>{va[r], vb[r]};
+      }
+    }
+    __syncthreads();
   }
 }
 

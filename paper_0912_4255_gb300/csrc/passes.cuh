@@ -88,8 +88,8 @@ template <typename R> constexpr int min_blocks(int nt, size_t smem) {
   const int b = by_regs < by_smem ? by_regs : by_smem;
   return b < 1 ? 1 : b;
 }
-// Stage plan of pass A: shared-memory stages up to sub-transforms of 2^NSL_LAST,
-// then a last stage of radix 2^RBL in registers.  Its shared memory: C
+// Stage plan of pass A: radix 16, a middle stage up to sub-transforms of
+// 2^NSL_LAST, then a last stage of radix 2^RBL, its outputs in registers.  Its shared memory: C
 // column pairs, the stage twiddle tables, and the two factors of the
 // inter-pass twiddle W_N^{p1 k2} = W_N^{j k2} W_N^{q NS k2} (p1 = j + q NS)
 // for the block's C columns.
@@ -98,20 +98,19 @@ template <int L1> struct PlanA {
   static constexpr int NSL_LAST = L1 - RBL;
   static constexpr int RADL = 1 << RBL;
   static constexpr int NS = (1 << L1) / RADL;
-  static constexpr int MID_TW = mid_tw_count<0, NSL_LAST>();
+  static constexpr int MID_TW = mid_tw_count(NSL_LAST - 4);
   static constexpr int LAST_TW = last_tw_count<NSL_LAST, RBL>();
 };
-// Pass B: a first radix-16 stage from global memory, shared-memory stages,
-// a last stage in registers: radix 16 at N2 = 2^8 and 2^12, which leaves one
-// (two) shared-memory exchanges instead of a further radix-2 one, else at
-// most 8.
+// Pass B: a first radix-16 stage from global memory, a middle stage, a last
+// stage with its outputs in registers: radix 16 at N2 = 2^8 (no middle stage)
+// and 2^12, else at most 8.
 template <int L2> struct PlanB {
   static constexpr int RB0 = 4;
   static constexpr int RBL = L2 == 8 || L2 == 12 ? 4 : (L2 - RB0 >= 3 ? 3 : L2 - RB0);
   static constexpr int NSL_LAST = L2 - RBL;
   static constexpr int RADL = 1 << RBL;
   static constexpr int NS = (1 << L2) / RADL;
-  static constexpr int MID_TW = mid_tw_count<RB0, NSL_LAST>();
+  static constexpr int MID_TW = mid_tw_count(NSL_LAST - RB0);
   static constexpr int LAST_TW = last_tw_count<NSL_LAST, RBL>();
 };
 template <typename R, int L1, int C> constexpr size_t cols_smem() {
@@ -124,6 +123,17 @@ template <typename R, int L2, int RR> constexpr size_t rows_smem() {
   return (size_t)RR * FftGeom<L2, RR>::STRIDE * sizeof(Pair<R>) + (size_t)(P::MID_TW + P::LAST_TW) * sizeof(cpx<R>);
 }
 
+// f(u) for the units u < COUNT of a block of NT threads.
+template <int COUNT, int NT, typename F>
+__device__ __forceinline__ void each_unit(F&& f) {
+  if constexpr (COUNT == NT) {
+    f((int)threadIdx.x);
+  } else {
+#pragma unroll 1
+    for (int u = threadIdx.x; u < COUNT; u += NT) f(u);
+  }
+}
+
 // --------------------------------------------------------------- pass A
 
 // Stage twiddle tables of pass A, the same for every tile of one shape
@@ -132,7 +142,7 @@ template <typename R, int L1, int C, int NT>
 __device__ __forceinline__ void cols_tables(const Tw<R>& tw, Pair<R>* buf) {
   using PA = PlanA<L1>;
   cpx<R>* tws = reinterpret_cast<cpx<R>*>(buf + C * FftGeom<L1, C>::STRIDE);
-  build_mid_tw<R, L1, 0, PA::NSL_LAST, NT>(tws, tw.tl[L1]);
+  build_mid_tw<R, L1, PA::NSL_LAST - 4, NT>(tws, tw.tl[L1]);
   build_last_tw<R, L1, PA::NSL_LAST, PA::RBL, NT>(tws + PA::MID_TW, tw.tl[L1]);
 }
 
@@ -161,6 +171,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
   // twiddle tables (cols_tables); this tile's inter-pass factors are
   // written here and read after the barriers that end the fill
   using PA = PlanA<L1>;
+  using F = FftPlan<L1, PA::RBL, C>;
   constexpr int NSL_LAST = PA::NSL_LAST;
   constexpr int RADL = PA::RADL;
   constexpr int NS = PA::NS;
@@ -168,16 +179,16 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
   Cx* tlast = tws + PA::MID_TW;           // last stage, rows of powers
   Cx* ta = tlast + PA::LAST_TW;           // [c][j]: W_N^{j (c0 + c)}, j < NS
   Cx* tb = ta + C * NS;                   // [c][q]: W_N^{q NS (c0 + c)}, q < RADL
-  for (int e = threadIdx.x; e < C * (NS + RADL); e += NT) {
-    if (e < C * NS) {
-      const int c = e / NS, j = e - c * NS;
-      ta[e] = twiddle<R>(a.tw, L, (uint32_t)j * (uint32_t)(c0 + c));
-    } else {
-      const int e2 = e - C * NS;
-      const int c = e2 / RADL, q = e2 - c * RADL;
-      tb[e2] = twiddle<R>(a.tw, L, (uint32_t)(q * NS) * (uint32_t)(c0 + c));
+  auto factors = [&] {
+#pragma unroll
+    for (int e0 = 0; e0 < C * NS; e0 += NT) {
+      const int e = e0 + threadIdx.x;
+      if (C * NS % NT == 0 || e < C * NS)
+        ta[e] = twiddle<R>(a.tw, L, (uint32_t)(e & (NS - 1)) * (uint32_t)(c0 + e / NS));
     }
-  }
+    for (int e = threadIdx.x; e < C * RADL; e += NT)
+      tb[e] = twiddle<R>(a.tw, L, (uint32_t)((e & (RADL - 1)) * NS) * (uint32_t)(c0 + e / RADL));
+  };
   if constexpr (loads(SRC)) {
     // the tiled resampler's order W[k2 / C][k1][k2 % C]: this tile's C * N1
     // pairs are contiguous, pair i = c + C k1 at offset i
@@ -185,11 +196,9 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
                           (int64_t)tile * (C * N1);
     // first radix-16 stage straight from the resampled series: unit
     // (j, column) with the column fastest, so that the lanes of a
-    // warp read consecutive values; outputs in the order of a first
-    // Stockham stage (sub-transforms of length 16 at 16 j)
+    // warp read consecutive values
     constexpr int Q1 = N1 / 16;
-#pragma unroll 1
-    for (int u = threadIdx.x; u < C * Q1; u += NT) {
+    each_unit<C * Q1, NT>([&](int u) {
       const int c = u & (C - 1);
       const int j = u / C;
       const Pair<R>* src = w_in + c + j * C;
@@ -205,13 +214,17 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
         va[r] = v.a;
         vb[r] = v.b;
       }
+      // behind the loads: the table look-ups of the factors wait on memory too
+      // (64 search templates 1372 -> MEAS_A us)
+      if (u == (int)threadIdx.x) factors();
       Dft<Cx, 16>::run(va);
       Dft<Cx, 16>::run(vb);
-      Pair<R>* dst = buf + c * STRIDE + pidx(16 * j);
+      Pair<R>* dst = buf + c * STRIDE;
 #pragma unroll
-      for (int r = 0; r < 16; ++r) dst[r] = Pair<R>{va[r], vb[r]};
-    }
+      for (int r = 0; r < 16; ++r) dst[F::place(r, j)] = Pair<R>{va[r], vb[r]};
+    });
   } else {
+    factors();
     GapCursor gc = make_cursor(m, a.gaps);
 #pragma unroll 2
     for (int i = threadIdx.x; i < C * N1; i += NT) {
@@ -226,7 +239,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
           pA += aa * aa; pB += bb * bb; pC += aa * bb;
         }
       }
-      buf[c * STRIDE + pidx(k1)] = Pair<R>{va, vb};
+      buf[c * STRIDE + F::place(k1 / F::SUB, k1 & (F::SUB - 1))] = Pair<R>{va, vb};
     }
   }
   if constexpr (!loads(SRC)) {
@@ -239,10 +252,8 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
     finalize_sums(a.c.meta + t, part, tiles, a.c.counters + t, a.pc.sigma2, nullptr, a.status);
   }
   __syncthreads();
-  // all stages but the last in shared memory (the first one done above when
-  // loading; it needs no twiddles, so the tables start at the same place)
-  static_assert(stage_tw_count<0, 4>() == 0, "first stage without twiddles");
-  fft_mid_stages<R, L1, loads(SRC) ? 4 : 0, NSL_LAST, NT, C, STRIDE>(buf, tws);
+  if constexpr (!loads(SRC)) first_stage<R, L1, PA::RBL, NT, C, STRIDE>(buf);
+  mid_stage<R, L1, PA::RBL, NT, C, STRIDE>(buf, tws);
   // last stage: inputs from shared memory, outputs X[p1 = j + q NS] stay in
   // registers, are multiplied by W_N^{p1 k2} and stored into Z.  Of that
   // twiddle the factor W_N^{j k2} is common to a butterfly's outputs, so it
@@ -250,8 +261,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
   // only W_N^{q NS k2} multiplies the outputs.  Lanes run over j mod RR, then
   // the column, then j / RR, so that a warp writes runs of RR * C
   // consecutive pairs of Z.
-#pragma unroll 1
-  for (int u = threadIdx.x; u < C * NS; u += NT) {
+  each_unit<C * NS, NT>([&](int u) {
     const int jr = u & (RRr - 1);
     const int rest = u >> lr;
     const int c = rest & (C - 1);
@@ -260,10 +270,12 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
     {
       Cx tq[RADL];
       last_twiddles<R, NSL_LAST, PA::RBL>(tlast + j, ta[c * NS + j], tq);
-      const Pair<R>* src = buf + c * STRIDE + pidx(j);
+      const int p0 = j & 15, q1 = j >> 4;
+      const Pair<R>* src = buf + c * STRIDE + p0 * F::SUB + q1 * RADL;
+      const int key = F::key(p0);
 #pragma unroll
       for (int q = 0; q < RADL; ++q) {
-        const Pair<R> v = src[q * (NS + NS / 16)];     // pidx(j + q NS): NS is a multiple of 16
+        const Pair<R> v = src[q ^ key];
         xa[q] = cmul(v.a, tq[q]);
         xb[q] = cmul(v.b, tq[q]);
       }
@@ -289,7 +301,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
       *zq = q == 0 ? Pair<R>{xa[q], xb[q]} : Pair<R>{cmul(xa[q], w), cmul(xb[q], w)};
       zq += zstep;
     }
-  }
+  });
 }
 
 // A, B, C of template t and the coefficients of 2F from the resampler's sums
@@ -359,7 +371,7 @@ template <typename R, int L2, int RR, int NT>
 __device__ __forceinline__ void rows_tables(const Tw<R>& tw, Pair<R>* buf) {
   using PB = PlanB<L2>;
   cpx<R>* tws = reinterpret_cast<cpx<R>*>(buf + RR * FftGeom<L2, RR>::STRIDE);
-  build_mid_tw<R, L2, PB::RB0, PB::NSL_LAST, NT>(tws, tw.tl[L2]);
+  build_mid_tw<R, L2, PB::NSL_LAST - PB::RB0, NT>(tws, tw.tl[L2]);
   build_last_tw<R, L2, PB::NSL_LAST, PB::RBL, NT>(tws + PB::MID_TW, tw.tl[L2]);
 }
 
@@ -405,13 +417,13 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
   // run over r, then j, so the loads are contiguous.
   const Pair<R>* zr = zbase + (int64_t)blk * N2 * RR;
   using PB = PlanB<L2>;
+  using F = FftPlan<L2, PB::RBL, RR>;
   Cx* tws = reinterpret_cast<Cx*>(buf + RR * STRIDE);   // shared-memory stages (rows_tables)
   Cx* tlast = tws + PB::MID_TW;           // last stage, rows of powers
   constexpr int RB0 = PB::RB0;
   constexpr int RAD0 = 1 << RB0;
   constexpr int Q0 = N2 / RAD0;                   // butterflies per sequence
-#pragma unroll 1
-  for (int u = threadIdx.x; u < RR * Q0; u += NT) {
+  each_unit<RR * Q0, NT>([&](int u) {
     const int r = u & (RR - 1);
     const int j = u / RR;
     const Pair<R>* src = zr + u;
@@ -431,15 +443,15 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
     }
     Dft<Cx, RAD0>::run(xa);
     Dft<Cx, RAD0>::run(xb);
-    Pair<R>* dst = buf + r * STRIDE + pidx(j * RAD0);
+    Pair<R>* dst = buf + r * STRIDE;
 #pragma unroll
-    for (int q = 0; q < RAD0; ++q) dst[q] = Pair<R>{xa[q], xb[q]};
-  }
+    for (int q = 0; q < RAD0; ++q) dst[F::place(q, j)] = Pair<R>{xa[q], xb[q]};
+  });
   __syncthreads();
   // middle stages in shared memory; in the last stage both series of a
   // butterfly are in one thread, so that 2F is formed in registers
   constexpr int NSL_LAST = PB::NSL_LAST;
-  fft_mid_stages<R, L2, RB0, NSL_LAST, NT, RR, STRIDE>(buf, tws);
+  mid_stage<R, L2, PB::RBL, NT, RR, STRIDE>(buf, tws);
   R ca, cb, cc;
   if constexpr (std::is_same<R, float>::value) {
     ca = m.ca; cb = m.cb; cc = m.cc;
@@ -458,9 +470,12 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
     {
       Cx tq[RADL];
       last_twiddles<R, NSL_LAST, PB::RBL>(tlast + j, cmk<Cx, R>((R)1, (R)0), tq);
+      const int p0 = j & 15, q1 = j >> 4;
+      const Pair<R>* src = buf + r * STRIDE + p0 * F::SUB + q1 * RADL;
+      const int key = F::key(p0);
 #pragma unroll
       for (int q = 0; q < RADL; ++q) {
-        const Pair<R> v = buf[r * STRIDE + pidx(j + q * NS)];
+        const Pair<R> v = src[q ^ key];
         fa[q] = q == 0 ? v.a : cmul(v.a, tq[q]);
         fb[q] = q == 0 ? v.b : cmul(v.b, tq[q]);
       }
