@@ -63,9 +63,9 @@ static cudaError_t do_cols(const PlanConst& pc, const Chunk& c, const Shape& sh,
                            int* status, cudaStream_t s) {
   ColsArgs<R> a;
   a.status = status;
-  a.rr = sh.rows;
+  a.rr = rows_group<R>(sh.l2);
   a.log2rr = 0;
-  while ((1 << a.log2rr) < sh.rows) ++a.log2rr;
+  while ((1 << a.log2rr) < a.rr) ++a.log2rr;
   a.pc = pc; a.c = c; a.x = nullptr; a.gaps = nullptr; a.wcs = nullptr;
   a.tw = *reinterpret_cast<const Tw<R>*>(tw);
   const int tiles = (1 << sh.l2) / sh.cols;

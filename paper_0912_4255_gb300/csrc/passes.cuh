@@ -44,7 +44,7 @@ struct ColsArgs {
   int tiles_max; // column tiles of one template
   int covered;   // tiles per template that the resampling grid covered
   int* status;
-  int rr, log2rr; // rows per block of the second pass (layout of Z)
+  int rr, log2rr; // rows of one group of Z (rows_group)
 };
 
 template <typename R>
@@ -67,13 +67,24 @@ struct RowsArgs {
 // independent blocks share an SM: one loads or stores while the other
 // computes.  Pass B, FP32: 16k (one block of 512 threads per SM), because
 // its 2F leaves in runs of R values and R = 8 rows at N = 2^22 fill a 32-byte
-// sector (runs of 4 measured 1.25 times the time).  FP64: 4k, bound by the
-// FP64 pipe at any size.
+// sector (runs of 4 measured 1.25 times the time); at N2 = 2^9, where 8k is
+// enough for that, two blocks of 256 threads (12 templates of 2^21: 126 ->
+// 110 us).  FP64: 4k, bound by the FP64 pipe at any size.
 template <typename R> constexpr int points_a() { return std::is_same<R, float>::value ? 8192 : 4096; }
-template <typename R> constexpr int points_b() { return std::is_same<R, float>::value ? 16384 : 4096; }
+template <typename R> constexpr int points_b(int L2) { return !std::is_same<R, float>::value ? 4096 : L2 == 9 ? 8192 : 16384; }
 template <int P> constexpr int cols_for(int L1) {
   const int c = (P / 2) >> L1;
   return c > 16 ? 16 : (c < 1 ? 1 : c);
+}
+template <typename R> constexpr int rows_for(int L2) {
+  const int c = (points_b<R>(L2) / 2) >> L2;
+  return c > 16 ? 16 : (c < 1 ? 1 : c);
+}
+// Rows of one group of the intermediate, Z[p1 / G][k2][p1 % G]: those of a
+// block of pass B, but 16 at N2 = 2^9, two blocks' worth, because pass A writes
+// runs of G C pairs (256 bytes instead of 128: 147 us, 160 with 128).
+template <typename R> constexpr int rows_group(int L2) {
+  return std::is_same<R, float>::value && L2 == 9 ? 16 : rows_for<R>(L2);
 }
 // one thread per 16 points of both series
 template <typename R> constexpr int threads_for(int logn, int count) {
@@ -215,7 +226,7 @@ __device__ __forceinline__ void cols_tile(const ColsArgs<R>& a, int t, int tile,
         vb[r] = v.b;
       }
       // behind the loads: the table look-ups of the factors wait on memory too
-      // (64 search templates 1372 -> MEAS_A us)
+      // (64 search templates 1372 -> 1343 us)
       if (u == (int)threadIdx.x) factors();
       Dft<Cx, 16>::run(va);
       Dft<Cx, 16>::run(vb);
@@ -381,7 +392,7 @@ __device__ __forceinline__ void rows_tables(const Tw<R>& tw, Pair<R>* buf) {
 // instead of row blocks.
 // BAND: the plan writes a partial output band (bins band_lo <= q < band_hi
 // only); without it every bin is stored, with no band test.
-template <typename R, int L2, int RR, int NT, bool BAND, bool INPLACE>
+template <typename R, int L2, int RR, int G, int NT, bool BAND, bool INPLACE>
 __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, Pair<R>* __restrict__ buf,
                                           const Pair<R>* __restrict__ zbase) {
   using Cx = cpx<R>;
@@ -412,10 +423,10 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
     }
     return;
   }
-  // this block's rows are one contiguous run of N2 * RR pairs, element
-  // (k2, r) at k2 * RR + r.  First radix-16 stage straight from there: lanes
-  // run over r, then j, so the loads are contiguous.
-  const Pair<R>* zr = zbase + (int64_t)blk * N2 * RR;
+  // this block's rows lie in one contiguous run of N2 * G pairs, element
+  // (k2, r) at k2 * G + r.  First radix-16 stage straight from there: lanes
+  // run over r, then j.
+  const Pair<R>* zr = zbase + (int64_t)(r0 / G) * (N2 * G) + (r0 & (G - 1));
   using PB = PlanB<L2>;
   using F = FftPlan<L2, PB::RBL, RR>;
   Cx* tws = reinterpret_cast<Cx*>(buf + RR * STRIDE);   // shared-memory stages (rows_tables)
@@ -426,7 +437,7 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
   each_unit<RR * Q0, NT>([&](int u) {
     const int r = u & (RR - 1);
     const int j = u / RR;
-    const Pair<R>* src = zr + u;
+    const Pair<R>* src = zr + r + j * G;
     Cx xa[RAD0], xb[RAD0];
 #pragma unroll
     for (int q = 0; q < RAD0; ++q) {
@@ -436,7 +447,7 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
         v = ldcs(zbase + ((int64_t)(k2 >> a.log2cols) << (L - L2 + a.log2cols)) + ((r0 + r) << a.log2cols) +
                  (k2 & (a.cols - 1)));
       } else {
-        v = ldcs(src + q * (Q0 * RR));
+        v = ldcs(src + q * (Q0 * G));
       }
       xa[q] = v.a;
       xb[q] = v.b;
@@ -513,21 +524,22 @@ __global__ void __launch_bounds__(NT, (min_blocks<R>(NT, rows_smem<R, L2, RR>())
     const int blk = w - t * a.blocks_max;
     const TmplMeta& m = a.c.meta[t];
     if constexpr (!INPLACE) {
-      // the next row block's run of the intermediate, into L2
+      // the run of the intermediate that the next row block needs, into L2
+      // (by the block that has the run's first rows)
+      constexpr int G = rows_group<R>(L2);
       const int wn = w + gridDim.x;
       if (threadIdx.x == 0 && wn < total) {
         const int tn = wn / a.blocks_max;
-        const int blkn = wn - tn * a.blocks_max;
+        const int rn = (wn - tn * a.blocks_max) * RR;
         const int ln = a.c.meta[tn].log2n;
-        if (blkn * RR < (1 << (ln - L2)))
-          prefetch_l2(reinterpret_cast<const Pair<R>*>(a.c.za) + (int64_t)tn * a.c.z_stride +
-                          (int64_t)blkn * ((1 << L2) * RR),
-                      (unsigned)((1u << L2) * RR * sizeof(Pair<R>)));
+        if (rn < (1 << (ln - L2)) && (rn & (G - 1)) == 0)
+          prefetch_l2(reinterpret_cast<const Pair<R>*>(a.c.za) + (int64_t)tn * a.c.z_stride + (int64_t)rn * (1 << L2),
+                      (unsigned)((1u << L2) * G * sizeof(Pair<R>)));
       }
     }
     if (blk * RR >= (1 << (m.log2n - L2))) continue;
     const Pair<R>* za = reinterpret_cast<const Pair<R>*>(a.c.za) + (int64_t)t * a.c.z_stride;
-    rows_tile<R, L2, RR, NT, BAND, INPLACE>(a, t, blk, buf, za);
+    rows_tile<R, L2, RR, rows_group<R>(L2), NT, BAND, INPLACE>(a, t, blk, buf, za);
     __syncthreads();                      // the next block reuses buf
   }
 }

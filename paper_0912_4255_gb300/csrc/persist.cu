@@ -90,7 +90,7 @@ template <int L2>
 __device__ __noinline__ void rows_call(const RowsArgs<float>& a, int t, int blk, Pair<float>* buf, const Pair<float>* za) {
   rows_tables<float, L2, cols_for<kPP>(L2), kPT>(a.tw, buf);
   __syncthreads();
-  rows_tile<float, L2, cols_for<kPP>(L2), kPT, true, false>(a, t, blk, buf, za);
+  rows_tile<float, L2, cols_for<kPP>(L2), cols_for<kPP>(L2), kPT, true, false>(a, t, blk, buf, za);
 }
 
 template <int SRC, int TAPS>

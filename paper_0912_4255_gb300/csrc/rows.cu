@@ -17,7 +17,7 @@ namespace fs {
 cudaError_t FS_CAT(rows, FS_REAL, FS_L2)(const RowsArgs<FS_REAL>& a, int inplace, dim3 grid, cudaStream_t s) {
   using R = FS_REAL;
   constexpr int L2 = FS_L2;
-  constexpr int RR = cols_for<points_b<R>()>(L2);
+  constexpr int RR = rows_for<R>(L2);
   constexpr int NT = threads_for<R>(L2, RR);
   constexpr size_t SM = rows_smem<R, L2, RR>();
   auto kern = inplace ? (a.band ? k_rows<R, L2, RR, NT, true, true> : k_rows<R, L2, RR, NT, false, true>)
@@ -32,6 +32,6 @@ cudaError_t FS_CAT(rows, FS_REAL, FS_L2)(const RowsArgs<FS_REAL>& a, int inplace
   kern<<<total < (unsigned)resident ? total : (unsigned)resident, NT, SM, s>>>(a);
   return cudaGetLastError();
 }
-int FS_CAT(rowsR, FS_REAL, FS_L2)() { return cols_for<points_b<FS_REAL>()>(FS_L2); }
+int FS_CAT(rowsR, FS_REAL, FS_L2)() { return rows_for<FS_REAL>(FS_L2); }
 
 }  // namespace fs
