@@ -99,3 +99,46 @@ def test_no_bins_or_templates_is_a_no_op():
     tm = fs.pack_templates(synth.make_templates([1.0], [0.2], [0.0], 0, 1), device="cuda")
     out = fs.fstat_sft_demod(p, sd, torch.from_numpy(X).cuda(), torch.from_numpy(t_sft).cuda(), tm, 100, 0)
     assert out.numel() == 0 and fs.fstat_status(p, raise_error=False) == 0
+
+
+@pytest.mark.parametrize("log2_n_fft,n_q", [(12, 1111), (14, 1111), (14, 9001), (15, 1111), (15, 9001), (16, 1111),
+                                            (17, 9001), (18, 1111), (20, 1111), (20, 9001)])
+@pytest.mark.parametrize("dk", [0, 1, 2, 3, 16])
+def test_every_step_of_kappa_and_every_kernel_length(log2_n_fft, n_q, dk):
+    """The step of kappa per frequency decides how the kernel's far terms are
+    summed (expansions over 64 or 32 frequencies, term by term): steps on both
+    sides of each line, lengths down to the single term, few and many
+    frequencies (no whole number of segments) across a whole kappa.  R15 metric <= 1e-4 as
+    above.  On a band of 2 dk + 2 bins the windows that leave it give NaN and
+    the others the same values."""
+    import torch
+    import paper_0912_4255_gb300 as fs
+    X, t_sft, plan, sd, inj, _ = _data()
+    X, t_sft = X[:37], t_sft[:37]
+    plan.n_data, plan.n_fft = int(37 * T / 0.5), 1 << log2_n_fft
+    sd.dirichlet_terms = dk
+    a, d = synth.random_sky(2, synth.SEED_BASE + 98)
+    tm = synth.make_templates([inj.alpha, a[0]], [inj.delta, d[0]], [inj.fdot, -1e-9], 0, 1)
+    p = fs.Plan(plan, device=torch.device("cuda:0"))
+    q0 = plan.n_fft // 2 - (500 if n_q < 2000 else 4000)
+
+    def run(sd, X):
+        return fs.fstat_sft_demod(p, sd, torch.from_numpy(np.ascontiguousarray(X)).cuda(),
+                                  torch.from_numpy(t_sft).cuda(), fs.pack_templates(tm, device="cuda"), q0,
+                                  n_q).cpu().numpy()
+
+    out = run(sd, X)
+    assert fs.fstat_status(p, raise_error=False) == 0
+    df = 1.0 / (plan.n_fft * plan.dt)
+    qs = np.arange(0, n_q, 1 if n_q < 2000 else 9)
+    f = F_H + (q0 + qs - plan.n_fft // 2) * df
+    for i in range(2):
+        want = DM.two_f(X.astype(np.complex128), sd, plan, t_sft, tm["alpha"][i], tm["delta"][i], f,
+                        fdot=tm["fdot"][i])
+        assert np.max(np.abs(out[i, qs] - want) / np.maximum(want, 4.0)) < 1e-4
+    k0 = sd.k_het - dk - sd.k_lo
+    sd.k_lo, sd.n_bins = sd.k_lo + k0, 2 * dk + 2
+    narrow = run(sd, X[:, k0:k0 + 2 * dk + 2])
+    ok = np.isfinite(narrow)
+    assert 0 < ok.sum() < ok.size and fs.fstat_status(p, raise_error=False) == -2
+    assert np.max(np.abs(narrow[ok] - out[ok]) / np.maximum(out[ok], 4.0)) < 1e-4
