@@ -372,7 +372,7 @@ k_demod(const DemodRec* __restrict__ rec, const float2* __restrict__ X, int n_sf
 }  // namespace
 
 size_t demod_workspace(int64_t n_sft, int64_t n_t) {
-  return (((size_t)n_t * (size_t)n_sft * sizeof(DemodRec) + 255) & ~(size_t)255) + (size_t)n_t * 32;
+  return ((size_t)n_t * (size_t)n_sft * sizeof(DemodRec) + 255) & ~(size_t)255;
 }
 
 cudaError_t launch_demod(const PlanConst& pc, const fstat_sft_desc& d, const float2* X, const double* t_sft,

@@ -110,3 +110,24 @@ def test_topk_into_given_tensors_on_a_second_stream():
         fs.fstat_topk(a, 4096, 8, n_rows=3, val=v[:2], bins=b)
     with pytest.raises(ValueError):
         fs.fstat_topk(a, 4096, 8, n_rows=3, val=v, bins=b.float())
+
+
+@pytest.mark.parametrize("n_rows,row_len,band_len,k",
+                         [(1, 2048, 2048, 1), (160, 4096, 2048, 64), (77, 8192, 4096, 33), (110, 18432, 6144, 1),
+                          (61, 51200, 10240, 64), (310, 18432, 18432, 16), (2, 262144, 131072, 64)])
+def test_topk_of_few_and_many_bands(n_rows, row_len, band_len, k):
+    """Up to two bands an SM and more, of one short sample to many pieces:
+    noise, and rows that make the bound's work hard: all values equal,
+    rising, rising in steps, few finite values, infinities of both signs
+    (only finite values count), the two zeros as equals."""
+    g = synth.rng(75)
+    a = g.chisquare(4, size=(n_rows, row_len)).astype(np.float32)
+    odd = [np.full(row_len, 3.5), np.arange(row_len), np.arange(row_len) // 700, np.full(row_len, np.nan),
+           np.where(np.arange(row_len) % 3 == 0, np.inf, a[0]), np.where(np.arange(row_len) % 5, -np.inf, -a[0]),
+           np.where(np.arange(row_len) % 2, -0.0, 0.0)]
+    odd[3][::1500] = -2.0
+    for i, r in enumerate(odd[:n_rows - 1]):
+        a[3 * i % n_rows] = r
+    v, b = _gpu_topk(a, band_len, k)
+    ov, ob = CA.band_top_k(np.where(np.isfinite(a), a, np.nan).astype(np.float64), band_len, k)
+    assert np.array_equal(v.astype(np.float64), ov) and np.array_equal(b.astype(np.int64), ob)
