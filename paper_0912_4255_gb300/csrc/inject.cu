@@ -72,23 +72,30 @@ __device__ int check_injection(const PlanConst& pc, const fstat_injection& in, i
   return FSTAT_OK;
 }
 
-// One block per segment of up to kInjSeg knot intervals of one injection
-// (grid (ceil(max_span / (kInjSeg H)), min(n_inj, 65535)); blocks stride over
+// One block per segment of up to seg <= kInjSeg knot intervals of one injection
+// (grid (ceil(max_span / (seg H)), min(n_inj, 65535)); blocks stride over
 // the injections in y).  The FP64 work is spread over the lanes: one thread
 // per knot (phase, beams and their derivatives), one per interval (Hermite
 // coefficients), one per run (the phase factor at the run's start), since a
 // warp's FP64 instruction costs the same for one active lane as for 32.
 // Every thread then evaluates, interval by interval, one sample of each run
-// in FP32.
-constexpr int kInjSeg = 64;
+// in FP32.  31 intervals have 32 knots, a warp's; where that leaves SMs idle
+// eight intervals shorten the chain: (8 | 31 | 64 intervals) 1 injection of
+// 200001 samples 17 | 27 | 41 us, 16 of them 25 | 27 | 41; 128 of 86401 76 | 49 |
+// 64, 256 of 20001 43 | 29 | 29, 256 of 200001 283 | 180 | 201.  The amplitudes'
+// coefficients are made once an interval and the phase factor by expm2pi
+// (128 of 86401 49 -> 47 us).  Bound by the FP64 set-up and, with many long
+// spans, by the atomic adds.
+constexpr int kInjSeg = 31;
+constexpr int kInjSegFew = 8;
 
 __global__ void __launch_bounds__(kInjThreads)
-k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, int64_t max_span,
+k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, int64_t max_span, int seg,
          float2* __restrict__ x, int* status) {
   __shared__ InjKnot kn[kInjSeg + 1];
   __shared__ double pcoef[kInjSeg][4];  // P0 (reduced), c1, c2, c3 of the phase
   __shared__ float cf[kInjSeg][4];      // c1_hi, c1_lo, c2, c3
-  __shared__ float ab[kInjSeg][8];      // a0..a3, b0..b3
+  __shared__ float amp[kInjSeg][8];     // 1/2 A_+ F_+ and 1/2 A_x F_x: coefficients p0..p3, c0..c3
   __shared__ float2 rot[kInjSeg][kInjRuns];   // exp(2 pi i P) at the start of each run
   for (int64_t j = blockIdx.y; j < n_inj; j += gridDim.y) {
     const fstat_injection in = inj[j];
@@ -97,11 +104,11 @@ k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, i
       if (blockIdx.x == 0 && threadIdx.x == 0) set_status(status, st);
       continue;
     }
-    const int64_t s0 = (int64_t)blockIdx.x * kInjSeg * kInjH;     // first sample of the segment
+    const int64_t s0 = (int64_t)blockIdx.x * seg * kInjH;     // first sample of the segment
     if (s0 >= in.span_len) continue;
     const int64_t n0 = in.span_start + s0;
     const int64_t left = in.span_len - s0;
-    const int n_int = (int)(left >= (int64_t)kInjSeg * kInjH ? kInjSeg : (left + kInjH - 1) >> kInjLog2H);
+    const int n_int = (int)(left >= (int64_t)seg * kInjH ? seg : (left + kInjH - 1) >> kInjLog2H);
     // knots at the ends of the segment's intervals
     if ((int)threadIdx.x <= n_int) {
       const Sky<double> sky = make_sky<double>(pc, in.alpha, in.delta);
@@ -120,10 +127,18 @@ k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, i
       cf[i][1] = (float)(c1 - (double)hi);
       cf[i][2] = (float)c2;
       cf[i][3] = (float)c3;
-      hermite3(kn[i].a, kn[i].da, kn[i + 1].a, kn[i + 1].da, &c1, &c2, &c3);
-      ab[i][0] = (float)kn[i].a; ab[i][1] = (float)c1; ab[i][2] = (float)c2; ab[i][3] = (float)c3;
-      hermite3(kn[i].b, kn[i].db, kn[i + 1].b, kn[i + 1].db, &c1, &c2, &c3);
-      ab[i][4] = (float)kn[i].b; ab[i][5] = (float)c1; ab[i][6] = (float)c2; ab[i][7] = (float)c3;
+      // F_+ = a cos 2 psi + b sin 2 psi, F_x = b cos 2 psi - a sin 2 psi
+      double a[4] = {kn[i].a}, b[4] = {kn[i].b};
+      hermite3(kn[i].a, kn[i].da, kn[i + 1].a, kn[i + 1].da, a + 1, a + 2, a + 3);
+      hermite3(kn[i].b, kn[i].db, kn[i + 1].b, kn[i + 1].db, b + 1, b + 2, b + 3);
+      float s2p, c2p;
+      sincosf(2.0f * (float)in.psi, &s2p, &c2p);
+      const double Ap = 0.25 * in.h0 * (1.0 + in.cosi * in.cosi), Ax = 0.5 * in.h0 * in.cosi;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        amp[i][j] = (float)(Ap * (a[j] * c2p + b[j] * s2p));
+        amp[i][4 + j] = (float)(Ax * (b[j] * c2p - a[j] * s2p));
+      }
     }
     __syncthreads();
     // the phase factor at the start of each run, from the FP64 phase
@@ -136,11 +151,6 @@ k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, i
       rot[i][r] = make_float2((float)cb, (float)sb);
     }
     __syncthreads();
-    float s2p, c2p;
-    sincosf(2.0f * (float)in.psi, &s2p, &c2p);
-    const float cosi = (float)in.cosi, h0 = (float)in.h0;
-    const float Ap = 0.5f * h0 * 0.5f * (1.0f + cosi * cosi);   // 1/2 A_+
-    const float Ax = 0.5f * h0 * cosi;                          // 1/2 A_x
     const int v = threadIdx.x;
     const float fv = (float)v;
 #pragma unroll 1
@@ -156,19 +166,18 @@ k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, i
         // (u + v)^2 - u^2 = v (2u + v); (u + v)^3 - u^3 = v (3u^2 + 3uv + v^2)
         const float ph = pv_frac + cf[i][1] * fv + cf[i][2] * (fv * (2.0f * u + fv)) +
                          cf[i][3] * (fv * (3.0f * u * u + 3.0f * u * fv + fv * fv));
-        float so, co;
-        sincospif(2.0f * ph, &so, &co);
+        int whole;
+        const float2 e = expm2pi(round_nearest(ph, &whole) - ph);        // e^{2 pi i ph}
         const float2 b0 = rot[i][r];
-        const float cs = b0.x * co - b0.y * so, sn = b0.y * co + b0.x * so;
+        const float cs = b0.x * e.x - b0.y * e.y, sn = b0.y * e.x + b0.x * e.y;
         const float fs_ = (float)s;
-        const float a = ab[i][0] + fs_ * (ab[i][1] + fs_ * (ab[i][2] + fs_ * ab[i][3]));
-        const float b = ab[i][4] + fs_ * (ab[i][5] + fs_ * (ab[i][6] + fs_ * ab[i][7]));
-        const float Fp = a * c2p + b * s2p, Fx = b * c2p - a * s2p;
-        const float2 add = make_float2(Fp * Ap * cs + Fx * Ax * sn, Fp * Ap * sn - Fx * Ax * cs);
+        const float p = amp[i][0] + fs_ * (amp[i][1] + fs_ * (amp[i][2] + fs_ * amp[i][3]));
+        const float c = amp[i][4] + fs_ * (amp[i][5] + fs_ * (amp[i][6] + fs_ * amp[i][7]));
+        const float2 add = make_float2(p * cs + c * sn, p * sn - c * cs);
         atomicAdd(x + n0 + (int64_t)i * kInjH + s, add);
       }
     }
-    __syncthreads();     // kn, pcoef, cf, ab, rot are rewritten for the next injection
+    __syncthreads();     // kn, pcoef, cf, amp, rot are rewritten for the next injection
   }
 }
 
@@ -176,11 +185,13 @@ k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, i
 
 cudaError_t launch_inject(const PlanConst& pc, const fstat_injection* inj, int64_t n_inj, int64_t max_span,
                           float2* x, int* status, cudaStream_t s) {
-  const int64_t bx = (max_span + (int64_t)kInjSeg * kInjH - 1) / ((int64_t)kInjSeg * kInjH);
+  const auto blocks = [&](int seg) { return (max_span + (int64_t)seg * kInjH - 1) / ((int64_t)seg * kInjH); };
+  const int seg = n_inj <= 64 && n_inj * blocks(kInjSegFew) <= 3 * 152 ? kInjSegFew : kInjSeg;
+  const int64_t bx = blocks(seg);
   if (n_inj <= 0 || bx <= 0) return cudaSuccess;
   if (bx > 0x7fffffff) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)bx, (unsigned)(n_inj < 65535 ? n_inj : 65535));
-  k_inject<<<grid, kInjThreads, 0, s>>>(pc, inj, n_inj, max_span, x, status);
+  k_inject<<<grid, kInjThreads, 0, s>>>(pc, inj, n_inj, max_span, seg, x, status);
   return cudaGetLastError();
 }
 

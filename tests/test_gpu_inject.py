@@ -118,3 +118,26 @@ def test_no_injections_is_a_no_op():
     fs.fstat_inject(plan, x, synth.injection_records(_injections()[:1], 1.0, 0, 0))   # empty span
     assert fs.fstat_status(plan, raise_error=False) == 0
     assert bool((x == 1).all())
+
+
+@pytest.mark.parametrize("n_inj", [9, 72])
+def test_spans_around_the_segments_of_a_block(n_inj):
+    """Few injections take blocks of 8 knot intervals of 1024 samples, more
+    than 64 blocks of 31: spans of one sample to a few segments with a
+    remainder, side by side.  Tolerance as above."""
+    import torch
+    import paper_0912_4255_gb300 as fs
+    spans = [1, 1023, 1025, 8191, 8192, 8193, 31743, 31744, 33793]
+    lens = [spans[i % len(spans)] for i in range(n_inj)]
+    starts = [int(a) for a in np.concatenate([[0], np.cumsum(lens)[:-1]])]
+    desc = synth.tiny_plan(n_data=sum(lens))
+    injs = [synth.random_injection(synth.SEED_BASE + 400 + k, df=0.3 - 0.008 * k, fdot=-1e-10 * k) for k in range(n_inj)]
+    plan = _plan(desc)
+    x = torch.zeros(desc.n_data, dtype=torch.complex64, device="cuda")
+    fs.fstat_inject(plan, x, synth.injection_records(injs, [1.0] * n_inj, starts, lens))
+    assert fs.fstat_status(plan, raise_error=False) == 0
+    got = x.cpu().numpy().astype(np.complex128)
+    for i in range(0, n_inj, 1 if n_inj < 20 else 7):
+        part = slice(starts[i], starts[i] + lens[i])
+        want = I.signal(injs[i], desc, h0=1.0)[part]
+        assert np.abs(got[part] - want).max() < 3e-6 * max(np.abs(want).max(), 0.05), (i, lens[i])
