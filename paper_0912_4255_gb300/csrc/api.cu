@@ -437,8 +437,10 @@ int fstat_grad(fstat_plan_t p, const float* x_h, const fstat_template* t, const 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const float2* x = reinterpret_cast<const float2*>(x_h);
   double* work = reinterpret_cast<double*>(p->ws + p->off_grad);
-  for (int64_t t0 = 0; t0 < n_t; t0 += p->chunk) {
-    const int nt = (int)(n_t - t0 < p->chunk ? n_t - t0 : p->chunk);
+  // the workspace of a persistent plan holds the sums of one template
+  const int step = p->tune.mode == FSTAT_MODE_PERSISTENT ? 1 : p->chunk;
+  for (int64_t t0 = 0; t0 < n_t; t0 += step) {
+    const int nt = (int)(n_t - t0 < step ? n_t - t0 : step);
     Chunk c = chunk_at(p, t + t0, nt);
     cudaError_t e = cudaMemsetAsync(c.counters, 0, sizeof(int) * 2 * nt, s);
     if (e == cudaSuccess)

@@ -144,3 +144,27 @@ def test_gradient_ascent_recovers_injections():
     final = FStatBin.apply(theta, search).detach()
     frac = (final / true_2f).cpu().numpy()
     assert np.all(frac > 0.9), (frac, (start / true_2f).cpu().numpy())
+
+
+def test_gradient_of_several_templates_on_a_persistent_plan():
+    """A persistent plan's workspace holds the gradient sums of one template:
+    several in one call give what a split plan gives (each mode its own time
+    map storage; the arithmetic is the same)."""
+    import torch
+    import paper_0912_4255_gb300 as fs
+    d, gaps, injs, x = _setup(60_000, 71, n_inj=1)
+    tm = synth.make_templates([injs[0].alpha + 1e-3 * i for i in range(7)], [injs[0].delta] * 7,
+                              [injs[0].fdot] * 7, 0, d.n_data, 0, len(gaps))
+    df = torch.tensor([injs[0].df + 1e-6 * i for i in range(7)], dtype=torch.float64)
+    dev = torch.device("cuda:0")
+    got = []
+    for mode in (fs.MODE_SPLIT, fs.MODE_PERSISTENT):
+        plan = fs.Plan(d, device=dev)
+        plan.set_tuning(mode=mode)
+        y, g = fs.fstat_grad(plan, torch.from_numpy(x).to(dev), fs.pack_templates(tm, device=dev), df,
+                             torch.from_numpy(gaps.reshape(-1).copy()).to(dev))
+        assert fs.fstat_status(plan, raise_error=False) == 0
+        got.append((y.cpu().numpy(), g.cpu().numpy()))
+        plan.close()
+    np.testing.assert_allclose(got[1][0], got[0][0], rtol=1e-6)
+    np.testing.assert_allclose(got[1][1], got[0][1], rtol=1e-5, atol=1e-6 * np.abs(got[0][1]).max())
