@@ -152,7 +152,7 @@ def fp32_peak_tflops(sm_mhz: float) -> float:
     return 152 * 128 * 2 * sm_mhz * 1e6 / 1e12
 
 
-def algorithmic_per_template(desc, fused=True, l1=None):
+def algorithmic_per_template(desc, in_pass=False, l1=None):
     """(FLOPs, design bytes) of one template in each kernel.
 
     FLOPs, counted from the algorithm:
@@ -165,9 +165,9 @@ def algorithmic_per_template(desc, fused=True, l1=None):
     Design bytes, the HBM traffic the four-step design needs (N_d data
     samples ~ N_b grid points, N = n_fft):
     * time map: an 80-byte knot record per 2^10 grid points;
-    * resample (split): read x_h 8 N_d, write w_a, w_b 16 N_b;
-    * first pass: read w_a, w_b 16 N_b (split) or x_h 8 N_d (fused), write the
-      intermediate 16 N;
+    * resample: read x_h 8 N_d, write w_a, w_b 16 N_b;
+    * first pass: read w_a, w_b 16 N_b, or x_h 8 N_d where it takes its own
+      samples (in_pass: the persistent mode), write the intermediate 16 N;
     * second pass: read the intermediate 16 N, write 2F 4 N.
     The path's own algorithmic bytes are 8 N_d + 4 N (path_bytes)."""
     n = int(desc.n_fft)
@@ -182,7 +182,7 @@ def algorithmic_per_template(desc, fused=True, l1=None):
     rows = 2 * 5 * n * l2 + 12 * n
     out = {"fft_rows": (rows, 16.0 * n + 4.0 * n), "timemap": (0.0, 80.0 * (n >> 10)), "sums": (0.0, 0.0),
            "persistent": (fft_a + res + rows, 8.0 * nd + 32.0 * n + 4.0 * n)}
-    if fused:
+    if in_pass:
         out["fft_cols"] = (fft_a + res, 8.0 * nd + 16.0 * n)
     else:
         out["resample"] = (res, 8.0 * nd + 16.0 * nd)
@@ -382,7 +382,7 @@ def main():
     peak_gbs, peak_kind = measured_peaks()
     sm_mhz = clocks.get("sm_mhz") or 2070.0
     peak_tf = fp32_peak_tflops(sm_mhz)
-    per_tpl = algorithmic_per_template(desc, fused=mode in (fs.MODE_FUSED, fs.MODE_PERSISTENT),
+    per_tpl = algorithmic_per_template(desc, in_pass=mode == fs.MODE_PERSISTENT,
                                        l1=plan.tuning()["log2_n1"])
     kernels = {}
     for k in ("timemap", "resample", "fft_cols", "fft_rows", "persistent", "sums"):

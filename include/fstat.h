@@ -249,10 +249,9 @@ int fstat_grad(fstat_plan_t p, const float *x_h, const fstat_template *templates
  * on the call's stream around every kernel it launches.  fstat_profile_read
  * waits for the recorded events and returns, per kernel kind (0 time map,
  * 1 resample stage, 2 first FFT pass, 3 second FFT pass, 4 gradient
- * forward, 5 gradient adjoint, 6 persistent batch, 7 the reduction of A, B,
- * C after the unfused resample stage), the summed device
- * milliseconds and the number of launches since the last read, then clears
- * them.  Launch counts are kept whether or not timing is enabled.  ms and
+ * forward, 5 gradient adjoint, 6 persistent batch, 7 nothing any more: the
+ * resample stage sums A, B, C), the summed device milliseconds and the
+ * number of launches since the last read, then clears them.  Launch counts are kept whether or not timing is enabled.  ms and
  * launches are host arrays of n_kinds entries (n_kinds <= 8). */
 int fstat_profile(fstat_plan_t p, int enable);
 int fstat_profile_read(fstat_plan_t p, double *ms, int64_t *launches, int n_kinds);

@@ -61,10 +61,10 @@ def _sources_digest() -> str:
 
 
 # sources that compile or sequence the kernels of fstat_compute (time map,
-# resampler, A/B/C reduction, both FFT passes); other entry points (top-k,
+# resampler, both FFT passes); other entry points (top-k,
 # injection, gradient, persistent and allocation-free modes) live elsewhere
 PATH_SOURCES = ("fstat_internal.cuh", "passes.cuh", "timemap.cu", "resample.cu", "cols.cu", "rows.cu",
-                "api.cu", "dispatch.cu")
+                "api.cu", "dispatch.cu", "sinc_run.cuh")
 
 
 def path_digest() -> str:

@@ -1,6 +1,6 @@
 // Internal declarations of the F-statistic library: plan constants, the
 // per-template metadata, knot records of the time map, device math helpers
-// and the shared-memory Stockham FFT used by both FFT passes.
+// and the in-place shared-memory FFT stages used by both FFT passes.
 #pragma once
 
 #include <cuda_runtime.h>

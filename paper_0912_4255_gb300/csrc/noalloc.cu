@@ -14,8 +14,8 @@
 // loading is the first call of this entry point on that device (its
 // cudaGetSymbolAddress); from then on the device holds it until the process
 // exits.  It holds:
-// the FFT intermediate of one template, its knot records, block partial
-// sums, counters, the twiddle tables and the window constants.  Templates
+// the series of one template (transformed in place), its knot records and
+// metadata, the twiddle tables and the window constants.  Templates
 // are processed one after another through that single scratch area.
 //
 // Limits: FFT length at most 2^20 (kNaMaxLog), single-precision evaluation
@@ -51,7 +51,6 @@ constexpr int kNaMaxLog = 20;
 constexpr int64_t kNaMaxN = (int64_t)1 << kNaMaxLog;
 constexpr int kNaMinLog2h = 9;
 constexpr int64_t kNaKnots = (kNaMaxN >> kNaMinLog2h) + 2;
-constexpr int64_t kNaParts = kNaMaxN / 256 + 1;
 constexpr int kNaMaxHalf = 8;
 
 constexpr int64_t tw_entries() {
@@ -65,9 +64,7 @@ constexpr int64_t al256(int64_t v) { return (v + 255) & ~(int64_t)255; }
 constexpr int64_t kOffZ = 0;
 constexpr int64_t kOffKnots = al256(kOffZ + 2 * kNaMaxN * (int64_t)sizeof(float2));
 constexpr int64_t kOffMeta = al256(kOffKnots + kNaKnots * (int64_t)sizeof(KnotF));
-constexpr int64_t kOffPart = al256(kOffMeta + (int64_t)sizeof(TmplMeta));
-constexpr int64_t kOffCnt = al256(kOffPart + 3 * kNaParts * (int64_t)sizeof(double));
-constexpr int64_t kOffStatus = al256(kOffCnt + 2 * (int64_t)sizeof(int));
+constexpr int64_t kOffStatus = al256(kOffMeta + (int64_t)sizeof(TmplMeta));
 constexpr int64_t kOffTw = al256(kOffStatus + (int64_t)sizeof(int));
 constexpr int64_t kOffWcs = al256(kOffTw + tw_entries() * (int64_t)sizeof(float2));
 constexpr int kWinRow = 96;        // doubles per H: 64 FP64 values, then 64 FP32 copies
@@ -237,9 +234,9 @@ extern "C" int fstat_compute_noalloc(const fstat_plan_desc* d, const float* x_h,
     c.meta = reinterpret_cast<TmplMeta*>(base + kOffMeta);
     c.knots = base + kOffKnots;
     c.knot_stride = kNaKnots;
-    c.partials = reinterpret_cast<double*>(base + kOffPart);
-    c.part_stride = kNaParts;
-    c.counters = reinterpret_cast<int*>(base + kOffCnt);
+    c.partials = nullptr;     // (of the modes that reduce A, B, C themselves)
+    c.part_stride = 0;
+    c.counters = nullptr;
     c.za = base + kOffZ;
     c.z_stride = d->n_fft;
     c.wa = c.za;              // the resampled series, transformed in place by pass A
