@@ -30,8 +30,7 @@ cudaError_t run(const ColsArgs<R>& a, dim3 grid, cudaStream_t s) {
   if (resident < 1) resident = 1;
   const unsigned total = grid.x * grid.y;
   const unsigned cap = (unsigned)resident;
-  kern<<<total < cap ? total : cap, NT, SM, s>>>(a);
-  return cudaGetLastError();
+  return launch_after(starts_early<R>((int64_t)total * (C << L1)), kern, dim3(total < cap ? total : cap), NT, SM, s, a);
 }
 }  // namespace
 

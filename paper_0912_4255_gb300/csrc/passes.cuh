@@ -340,7 +340,9 @@ __global__ void __launch_bounds__(NT, (min_blocks<R>(NT, cols_smem<R, L1, C>()))
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[96];
   Pair<R>* buf = reinterpret_cast<Pair<R>*>(smem_raw);
+  let_next_start();
   cols_tables<R, L1, C, NT>(a.tw, buf);
+  wait_for_previous();
   const int total = a.tiles_max * a.c.nt;
 #pragma unroll 1
   for (int w = blockIdx.x; w < total; w += gridDim.x) {
@@ -516,6 +518,7 @@ __global__ void __launch_bounds__(NT, (min_blocks<R>(NT, rows_smem<R, L2, RR>())
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Pair<R>* buf = reinterpret_cast<Pair<R>*>(smem_raw);
   rows_tables<R, L2, RR, NT>(a.tw, buf);
+  wait_for_previous();
   __syncthreads();
   const int total = a.blocks_max * a.c.nt;
 #pragma unroll 1

@@ -154,6 +154,8 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* 
   using Cx = cpx<R>;
   using Knot = typename KnotOf<R>::T;
   __shared__ Pair<R> tiles[kTileWarps][kTilePts];
+  let_next_start();
+  wait_for_previous();
   const int t = blockIdx.y;
   const TmplMeta& m = c.meta[t];
   if (m.status != FSTAT_OK) return;
@@ -250,6 +252,8 @@ k_resample_run(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2
   __shared__ __align__(128) Pair<float> tiles[kTileWarps][kTilePts];
   __shared__ float4 rows[kTileWarps][2][kTileRows * kRowUnits];
   __shared__ float4 recs[kTileWarps][kTileRows][5];
+  let_next_start();
+  wait_for_previous();
   const int t = blockIdx.y;
   const TmplMeta& m = c.meta[t];
   if (m.status != FSTAT_OK) return;
@@ -530,7 +534,12 @@ cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& 
   const TileGrid tg = tile_grid(pc, sh, c.nt);
   if (tg.blocks == 0) return cudaSuccess;
   const dim3 grid((unsigned)tg.blocks, (unsigned)c.nt);
-  auto go = [&](auto kern) { kern<<<grid, kTileThreads, 0, s>>>(pc, c, sh.l2, lc, tg.per_warp, x, gaps, wcs); };
+  cudaError_t e = cudaSuccess;
+  const int64_t points = (int64_t)c.nt << (sh.l1 + sh.l2);
+  const bool early = pc.precision == FSTAT_PREC_FP64 ? starts_early<double>(points) : starts_early<float>(points);
+  auto go = [&](auto kern) {
+    e = launch_after(early, kern, grid, kTileThreads, 0, s, pc, c, sh.l2, lc, tg.per_warp, x, gaps, wcs);
+  };
   if (pc.precision == FSTAT_PREC_FP64) {
     if (pc.interp == FSTAT_NEAREST) go(k_resample_t<double, FSTAT_NEAREST, 8>);
     else if (pc.taps == 8) go(k_resample_t<double, FSTAT_SINC, 8>);
@@ -553,7 +562,7 @@ cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& 
       else go(k_resample_run<RUN_RECT, false>);
     }
   }
-  return cudaGetLastError();
+  return e;
 }
 
 // Tiles per template that the resampling grid covers.

@@ -29,8 +29,8 @@ cudaError_t FS_CAT(rows, FS_REAL, FS_L2)(const RowsArgs<FS_REAL>& a, int inplace
   if (e != cudaSuccess) return e;
   if (resident < 1) resident = 1;
   const unsigned total = grid.x * grid.y;
-  kern<<<total < (unsigned)resident ? total : (unsigned)resident, NT, SM, s>>>(a);
-  return cudaGetLastError();
+  const dim3 blocks(total < (unsigned)resident ? total : (unsigned)resident);
+  return launch_after(starts_early<R>((int64_t)total * (RR << L2)), kern, blocks, NT, SM, s, a);
 }
 int FS_CAT(rowsR, FS_REAL, FS_L2)() { return rows_for<FS_REAL>(FS_L2); }
 

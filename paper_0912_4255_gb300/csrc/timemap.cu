@@ -213,6 +213,7 @@ k_timemap(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* __res
   __shared__ double val[4][kTmKnots], slope[4][kTmKnots];   // u, P, a, b at the knots
   __shared__ double geo[5][kTmKnots];              // t_m, rate, sin H, cos H, dT/dk
   __shared__ TmplGrid grid_sh;
+  let_next_start();
   const int t = blockIdx.y;
   const fstat_template tp = tmpl[t];
   const int64_t g0 = (int64_t)blockIdx.x * groups;
@@ -324,6 +325,7 @@ k_timemap_f32(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* _
               const int64_t* __restrict__ gaps, int64_t n_gaps_total, int* status, int64_t tmpl_base) {
   __shared__ KnotVal<float> kv[kKnotThreads];
   __shared__ double tb_sh[2];
+  let_next_start();
   const int t = blockIdx.y;
   const fstat_template tp = tmpl[t];
   const int64_t j0 = (int64_t)blockIdx.x * (kKnotThreads - 1);

@@ -203,3 +203,47 @@ def test_band_lengths_and_chunk_lengths(n1, n_slots):
     want = FE.sft_to_series(X.astype(np.complex128), t, d, 0.0, n_out)
     got = fs.fstat_sft_series(d, torch.from_numpy(X).cuda(), t, 0.0, n_out).cpu().numpy()
     assert np.abs(got - want).max() < 3e-5 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("n_t,l_fft", [(1, 12), (1, 17), (64, 17), (65, 17), (2, 22)])
+@pytest.mark.parametrize("mode", ["split", "fused", "plain"])
+def test_calls_one_after_another(n_t, l_fft, mode):
+    """Up to 2^23 points per launch the kernels of a call start while the one
+    before still runs: calls on different series, eager and from a CUDA graph,
+    without a pause between them give what each gives alone, bit for bit."""
+    import torch
+    import paper_0912_4255_gb300 as fs
+    n = 1 << l_fft
+    d = synth.PlanDesc(dt=max(0.5, 65536 / n), n_data=int(0.7 * n) | 1, n_fft=n, f_het=40.0, max_templates=n_t,
+                       interp=R.SINC)
+    dev = torch.device("cuda:0")
+    plan = fs.Plan(d, device=dev)
+    plan.set_tuning(mode=MODES[mode])
+    g = synth.rng(95)
+    tm = synth.make_templates(g.uniform(0, 6, n_t), g.uniform(-1, 1, n_t), g.uniform(-1e-9, 0, n_t), 0, d.n_data)
+    tm = fs.pack_templates(tm, device=dev)
+    xs = [torch.from_numpy(synth.complex_noise(d.n_data, 1.0, 96 + i)).to(dev) for i in range(3)]
+    alone = []
+    for x in xs:
+        alone.append(fs.fstat_compute(plan, x, tm))
+        torch.cuda.synchronize()
+    outs = [torch.empty_like(a) for a in alone]
+
+    def calls():
+        for _ in range(2):
+            for x, o in zip(xs, outs):
+                fs.fstat_compute(plan, x, tm, twoF=o)
+
+    calls()
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, a) for o, a in zip(outs, alone))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        calls()
+    for _ in range(2):
+        for o in outs:
+            o.zero_()
+        graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, a) for o, a in zip(outs, alone))
+    plan.close()
