@@ -462,7 +462,10 @@ __device__ __forceinline__ float round_nearest(float x, int* i) {
 // own have (they take what room is left), and the second waits, before it
 // touches anything the first writes, until the first is complete and its writes
 // are visible.  Every block waits, also one with nothing to do: a kernel that
-// is complete then vouches for all before it.
+// is complete then vouches for all before it.  Loads that the compiler may move
+// (read-only and streaming ones) of what the first kernel wrote stand behind a
+// branch on the template's metadata, which is loaded after the wait; before it
+// a kernel reads the plan's tables only and writes its own shared memory only.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
