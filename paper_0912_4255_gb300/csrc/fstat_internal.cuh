@@ -59,9 +59,12 @@ struct TmplMeta {
   int64_t span_lo, span_hi, gap_off, n_gaps;
   int32_t n_int;     // knot intervals
   int32_t log2n;     // FFT length of this template
-  int32_t status;    // FSTAT_OK or the error of this template
+  int32_t status;    // FSTAT_OK or the error of this template, as the time map found it
   float ca, cb, cc;  // 2F = ca |Fa|^2 + cb |Fb|^2 + cc Re(Fa Fb*)
-  int32_t pad_;
+  // FSTAT_OK, or FSTAT_ERANGE where A, B, C give no 2F.  Not in `status`: pass A
+  // sets it while other blocks still choose by `status` whether a tile of this
+  // template is theirs, and the warps of a block have to choose alike.
+  int32_t sums;
 };
 
 // Knot interval record, single precision evaluation (80 bytes).  On the
@@ -1145,7 +1148,7 @@ __device__ __forceinline__ void set_sums(TmplMeta* meta, double A, double B, dou
   const double D = A * B - Cc * Cc;
   meta->A = A; meta->B = B; meta->C = Cc;
   if (!(D > 0.0) || !isfinite(D)) {
-    meta->status = FSTAT_ERANGE;
+    meta->sums = FSTAT_ERANGE;
     set_status(status, FSTAT_ERANGE);
   }
   const double s = 1.0 / (sigma2 * D);

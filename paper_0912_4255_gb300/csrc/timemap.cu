@@ -172,7 +172,7 @@ __device__ __forceinline__ void write_meta(const PlanConst& pc, const fstat_temp
     m.log2n = g.log2n;
     m.status = st;
     m.ca = m.cb = m.cc = 0.f;
-    m.pad_ = 0;
+    m.sums = FSTAT_OK;
     *meta = m;
     if (st != FSTAT_OK) set_status(status, st);
   }

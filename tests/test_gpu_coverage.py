@@ -221,6 +221,30 @@ def test_degenerate_template_inside_a_gap(mode):
         assert r15(got[i], oracle_two_f(desc, x, tm[i], gaps)) <= TOL, i
 
 
+@pytest.mark.parametrize("where", [0, 1])
+@pytest.mark.parametrize("mode", ["split", "fused"])
+def test_degenerate_template_among_many_tiles(mode, where):
+    """2^22 points a template, so that every resident block of the first pass
+    takes several column tiles of each: that a template turns out to have no
+    valid sample (found while its other tiles are still being handed out)
+    must not disturb the tiles of the others, which are bit for bit those of a
+    call without it."""
+    desc = synth.PlanDesc(dt=0.5, n_data=1_728_000, n_fft=1 << 22, f_het=100.0, max_templates=3)
+    gaps = np.array([[800_000, 900_000]], np.int64)
+    a, dl = synth.random_sky(3, synth.SEED_BASE + 196)
+    tm = synth.make_templates(a, dl, np.zeros(3), 0, desc.n_data, 0, 1)
+    tm["span_start"][where], tm["span_len"][where] = 810_000, 50_000
+    x, _ = injected_series(desc, synth.SEED_BASE + 197, [], gaps)
+    keep = [i for i in range(3) if i != where]
+    want, rc = run_compute(desc, x, tm[keep], gaps, mode=MODES[mode])
+    assert rc == 0 and np.all(np.isfinite(want))
+    for _ in range(5):
+        got, rc = run_compute(desc, x, tm, gaps, mode=MODES[mode])
+        assert rc == -2
+        assert np.all(np.isnan(got[where]))
+        assert np.array_equal(got[keep], want)
+
+
 def test_sky_edges_poles_and_angle_wrap():
     """Sky positions at the edges of their ranges: both celestial poles
     (delta = +-pi/2, where the sidereal term of the Roemer delay vanishes),
