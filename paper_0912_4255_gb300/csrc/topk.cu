@@ -127,8 +127,11 @@ __device__ void topk_sweep(const float* __restrict__ src, int base, int64_t o, i
     append(v4.z, b0 + 2, tau, sv, si, &cnt, k);
     append(v4.w, b0 + 3, tau, sv, si, &cnt, k);
     __syncthreads();
+    // every warp has to see the same count: none goes on to append before all have read it
+    const int n = cnt;
+    __syncthreads();
     // the next step adds at most F::STEP candidates: merge while they still fit
-    if (cnt > F::SORT_N - k - F::STEP || s0 + F::STEP >= band_len) tau = merge<F>(sv, si, &cnt, k);
+    if (n > F::SORT_N - k - F::STEP || s0 + F::STEP >= band_len) tau = merge<F>(sv, si, &cnt, k);
   }
   for (int i = threadIdx.x; i < k; i += F::THREADS) {
     val[o + i] = sv[i];

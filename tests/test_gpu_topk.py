@@ -131,3 +131,25 @@ def test_topk_of_few_and_many_bands(n_rows, row_len, band_len, k):
     v, b = _gpu_topk(a, band_len, k)
     ov, ob = CA.band_top_k(np.where(np.isfinite(a), a, np.nan).astype(np.float64), band_len, k)
     assert np.array_equal(v.astype(np.float64), ov) and np.array_equal(b.astype(np.int64), ob)
+
+
+@pytest.mark.parametrize("n_rows", [3, 320])
+@pytest.mark.parametrize("k", [1, 64])
+def test_topk_sweeps_whose_buffer_fills_at_any_step(n_rows, k):
+    """Bands that overflow the buffer and are swept, in both block shapes:
+    rising, with stretches below the bound of any length, so that the count
+    stands at and about the line where the buffer is merged, and some warps of
+    a step append while others have nothing."""
+    n = 65536
+    g = synth.rng(76)
+    a = np.arange(n, dtype=np.float64)[None, :] + 0.25 * g.random((n_rows, n))
+    for r in range(n_rows):
+        for s in g.integers(0, n, 12 + r % 40):
+            a[r, s:s + int(g.integers(1, 3000))] = -1.0 - g.random()
+        if r % 3 == 1:
+            a[r, (np.arange(n) // 32) % int(g.integers(2, 9)) > 0] = -5.0      # whole warps of values out
+    a = a.astype(np.float32)
+    ov, ob = CA.band_top_k(a.astype(np.float64), n, k)
+    for _ in range(4):
+        v, b = _gpu_topk(a, n, k)
+        assert np.array_equal(v.astype(np.float64), ov) and np.array_equal(b.astype(np.int64), ob)
