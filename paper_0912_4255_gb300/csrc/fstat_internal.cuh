@@ -60,11 +60,12 @@ struct TmplMeta {
   int32_t n_int;     // knot intervals
   int32_t log2n;     // FFT length of this template
   int32_t status;    // FSTAT_OK or the error of this template, as the time map found it
+  // the same, or FSTAT_ERANGE where A, B, C give no 2F, for the second pass.  Not
+  // in `status`: the first pass sets it while other blocks still choose by
+  // `status` whether a tile of this template is theirs, and the warps of a
+  // block have to choose alike.
+  int32_t status_2f;
   float ca, cb, cc;  // 2F = ca |Fa|^2 + cb |Fb|^2 + cc Re(Fa Fb*)
-  // FSTAT_OK, or FSTAT_ERANGE where A, B, C give no 2F.  Not in `status`: pass A
-  // sets it while other blocks still choose by `status` whether a tile of this
-  // template is theirs, and the warps of a block have to choose alike.
-  int32_t sums;
 };
 
 // Knot interval record, single precision evaluation (80 bytes).  On the
@@ -1148,7 +1149,7 @@ __device__ __forceinline__ void set_sums(TmplMeta* meta, double A, double B, dou
   const double D = A * B - Cc * Cc;
   meta->A = A; meta->B = B; meta->C = Cc;
   if (!(D > 0.0) || !isfinite(D)) {
-    meta->sums = FSTAT_ERANGE;
+    meta->status_2f = FSTAT_ERANGE;
     set_status(status, FSTAT_ERANGE);
   }
   const double s = 1.0 / (sigma2 * D);

@@ -324,7 +324,7 @@ template <typename R>
 __device__ __forceinline__ void finish_sums(const ColsArgs<R>& a, int t, int l2) {
   TmplMeta* m = a.c.meta + t;
   if (live_tiles(m->n_b, l2) > a.covered) {
-    m->sums = FSTAT_ERANGE;
+    m->status_2f = FSTAT_ERANGE;
     set_status(a.status, FSTAT_ERANGE);
     return;
   }
@@ -413,7 +413,7 @@ __device__ __forceinline__ void rows_tile(const RowsArgs<R>& a, int t, int blk, 
     hi = (int)(a.pc.band_hi < ((int64_t)1 << L) ? a.pc.band_hi : ((int64_t)1 << L));
     out -= lo;
   }
-  if (m.status != FSTAT_OK || m.sums != FSTAT_OK) {
+  if (m.status_2f != FSTAT_OK) {
     for (int i = threadIdx.x; i < RR * N2; i += NT) {
       const int r = i & (RR - 1), p2 = i / RR;
       if constexpr (BAND) {

@@ -172,7 +172,7 @@ __device__ __forceinline__ void write_meta(const PlanConst& pc, const fstat_temp
     m.log2n = g.log2n;
     m.status = st;
     m.ca = m.cb = m.cc = 0.f;
-    m.sums = FSTAT_OK;
+    m.status_2f = st;
     *meta = m;
     if (st != FSTAT_OK) set_status(status, st);
   }
