@@ -372,7 +372,7 @@ int fstat_resample(fstat_plan_t p, const float* x_h, const fstat_template* t, in
     Chunk c = chunk_at(p, t + t0, nt);
     cudaError_t e = cudaMemsetAsync(c.counters, 0, sizeof(int) * nt, s);
     if (e == cudaSuccess)
-      e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, gaps, n_gaps_total, p->status, t0, s); });
+      e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, false, gaps, n_gaps_total, p->status, t0, s); });
     if (e == cudaSuccess)
       e = timed(p, K_RESAMPLE, s, [&] {
         return launch_resample_w(p->pc, c, -1, p->log2n, reinterpret_cast<const float2*>(x_h), gaps, p->wcs,
@@ -398,7 +398,7 @@ int fstat_compute(fstat_plan_t p, const float* x_h, const fstat_template* t, int
     cudaError_t e = cudaMemsetAsync(c.counters, 0, sizeof(int) * nt, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(pcnt, 0, sizeof(int) * (2 * (size_t)nt + 2), s);
     if (e == cudaSuccess)
-      e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, gaps, n_gaps_total, p->status, 0, s); });
+      e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, false, gaps, n_gaps_total, p->status, 0, s); });
     const int stall = p->stall_template >= 0 && p->stall_template < n_t ? (int)p->stall_template : -1;
     const int limit = stall >= 0 ? (1 << 12) : p->spin_limit;
     p->stall_template = -1;
@@ -418,7 +418,7 @@ int fstat_compute(fstat_plan_t p, const float* x_h, const fstat_template* t, int
     // pass A transforms each column in place
     const int inplace = p->tune.mode == FSTAT_MODE_FUSED;
     if (inplace) c.wa = c.za;
-    cudaError_t e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, gaps, n_gaps_total, p->status, t0, s); });
+    cudaError_t e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, true, gaps, n_gaps_total, p->status, t0, s); });
     if (e == cudaSuccess) e = timed(p, K_RESAMPLE, s, [&] { return launch_resample_t(p->pc, c, p->sh, x, gaps, p->wcs, s); });
     if (e == cudaSuccess) e = timed(p, K_COLS, s, [&] { return launch_cols_w(p->pc, c, p->sh, inplace, &p->twf, &p->twd, p->status, s); });
     if (e == cudaSuccess) e = timed(p, K_ROWS, s, [&] { return launch_rows_w(p->pc, c, p->sh, inplace, &p->twf, &p->twd, twoF, s); });
@@ -444,7 +444,7 @@ int fstat_grad(fstat_plan_t p, const float* x_h, const fstat_template* t, const 
     Chunk c = chunk_at(p, t + t0, nt);
     cudaError_t e = cudaMemsetAsync(c.counters, 0, sizeof(int) * 2 * nt, s);
     if (e == cudaSuccess)
-      e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, gaps, n_gaps_total, p->status, t0, s); });
+      e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, false, gaps, n_gaps_total, p->status, t0, s); });
     if (e == cudaSuccess)
       e = timed(p, K_GRADF, s, [&] {
         return launch_grad_pass(p->pc, c, x, gaps, p->wcs, df + t0, work, twoF + t0, grad + 4 * t0, p->status, 0, s);

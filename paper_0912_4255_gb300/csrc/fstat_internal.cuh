@@ -46,13 +46,17 @@ struct PlanConst {
   int64_t band_lo, band_hi;
 };
 
+// Bits of a unit of the sums of A, B, C: 2^24 points of scaled beam patterns,
+// |a|, |b| <= 1 (scale_beams), stay below 2^61.
+constexpr int kSumBits = 36;
+
 // Per-template state produced by the time-map kernel and completed by the
 // first FFT pass (sums A, B, C and the 2F coefficients).
 struct TmplMeta {
   double tb0;        // t_b of grid point 0
   double A, B, C;    // masked antenna sums (Eq. 9 as sums)
-  // the same while the tiled resampler adds them up, in units of 2^-32: whole
-  // numbers, so that the order of the warps' additions does not matter
+  // the same while the tiled resampler adds them up, in units of 2^-kSumBits:
+  // whole numbers, so that the order of the warps' additions does not matter
   unsigned long long acc[3];
   int64_t n_b;       // resampled length N_b
   int64_t out_off;   // output offset in floats
@@ -266,6 +270,27 @@ __device__ __forceinline__ Sky<R> make_sky(const PlanConst& pc, R alpha, R delta
   rsincos<R>(alpha, &sa, &ca);
   rsincos<R>(delta, &sd, &cd);
   return make_sky<R>(pc, alpha, sa, ca, sd, cd);
+}
+
+// 2^-e with 2^e above the sum of the amplitudes, the bound of a pattern at any
+// hour angle (a pattern whose squares FP32 cannot hold is left as it is)
+__device__ __forceinline__ float beam_scale(float amplitudes) {
+  return amplitudes > 1e-18f && amplitudes < 1e18f ? __int_as_float((253 << 23) - (__float_as_int(amplitudes) & 0x7f800000))
+                                                   : 1.0f;
+}
+
+// a and b each times a power of two that brings its bound to 1/2 .. 1.  2F is
+// the same to the last bit (a^2 |Fb|^2, b^2 |Fa|^2 and ab Fa Fb* all over a^2 b^2 in
+// Eq. 6), and the sums of A, B, C in fixed units keep their accuracy for
+// patterns of any size: for a detector at the pole b is sin(delta) of its size
+// elsewhere.
+template <typename R>
+__device__ __forceinline__ void scale_beams(Sky<R>& s) {
+  const float ka = beam_scale(fabsf((float)s.e0) + fabsf((float)s.e1) + fabsf((float)s.e2) + fabsf((float)s.e3) +
+                              fabsf((float)s.e4));
+  const float kb = beam_scale(fabsf((float)s.f1) + fabsf((float)s.f2) + fabsf((float)s.f3) + fabsf((float)s.f4));
+  s.e0 *= ka; s.e1 *= ka; s.e2 *= ka; s.e3 *= ka; s.e4 *= ka;
+  s.f1 *= kb; s.f2 *= kb; s.f3 *= kb; s.f4 *= kb;
 }
 
 // t_m(t) and dt_m/dt; sH, cH: sin and cos of the hour angle theta(t) - alpha.
@@ -1239,7 +1264,7 @@ cudaError_t launch_demod(const PlanConst& pc, const fstat_sft_desc& d, const flo
                          float* out, void* ws, int* status, cudaStream_t s);
 cudaError_t launch_inject(const PlanConst& pc, const fstat_injection* inj, int64_t n_inj, int64_t max_span,
                           float2* x, int* status, cudaStream_t s);
-cudaError_t launch_timemap(const PlanConst& pc, const Chunk& c, int log2n_plan, int mode,
+cudaError_t launch_timemap(const PlanConst& pc, const Chunk& c, int log2n_plan, int mode, bool scaled,
                            const int64_t* gaps, int64_t n_gaps_total, int* status,
                            int64_t tmpl_base, cudaStream_t s);
 cudaError_t launch_resample_w(const PlanConst& pc, const Chunk& c, int ti, int log2n, const float2* x,

@@ -328,7 +328,7 @@ __device__ __forceinline__ void finish_sums(const ColsArgs<R>& a, int t, int l2)
     set_status(a.status, FSTAT_ERANGE);
     return;
   }
-  constexpr double u = 1.0 / 4294967296.0;
+  constexpr double u = 1.0 / (double)(1ll << kSumBits);
   set_sums(m, u * (double)(long long)m->acc[0], u * (double)(long long)m->acc[1], u * (double)(long long)m->acc[2],
            a.pc.sigma2, nullptr, a.status);
 }

@@ -125,8 +125,8 @@ __device__ __forceinline__ void store_tile(Pair<R>* __restrict__ w_out, const Pa
   }
 }
 
-// Adds the warp's sums of a^2, b^2, a b to the template's (|a|, |b| <= 2: the
-// whole numbers stay below 2^59 for 2^24 points).  One atomic addition per
+// Adds the warp's sums of a^2, b^2, a b to the template's, in units of 2^-36 of
+// what one point can add (scale_beams).  One atomic addition per
 // warp and sum: partial sums in memory and a kernel to reduce them took 10 us
 // of every call, a barrier over the block's warps held them until the slowest
 // was done.
@@ -140,7 +140,7 @@ __device__ __forceinline__ void add_sums(float pa, float pb, float pcc, TmplMeta
   const int lane = threadIdx.x & 31;
   if (lane < 3) {
     const float v = lane == 0 ? pa : (lane == 1 ? pb : pcc);
-    atomicAdd(&m->acc[lane], (unsigned long long)__double2ll_rn((double)v * 4294967296.0));
+    atomicAdd(&m->acc[lane], (unsigned long long)__double2ll_rn((double)v * (double)(1ll << kSumBits)));
   }
 }
 

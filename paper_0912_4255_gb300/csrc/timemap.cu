@@ -205,7 +205,7 @@ constexpr int kTmKnots = 32;
 template <typename REC>
 __global__ void __launch_bounds__(kTmThreads)
 k_timemap(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* __restrict__ meta,
-          REC* __restrict__ knots, int64_t knot_stride, int log2n_plan, int allow_ragged,
+          REC* __restrict__ knots, int64_t knot_stride, int log2n_plan, int allow_ragged, bool scaled,
           const int64_t* __restrict__ gaps, int64_t n_gaps_total, int* status, int64_t tmpl_base, int groups) {
   __shared__ double tb_sh[2];
   __shared__ Sky<double> sky;
@@ -272,6 +272,8 @@ k_timemap(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* __res
       geo[4][lane] = pc.dt * inv1r;
       val[0][lane] = (T1 + dT - pc.t_start) * pc.inv_dt;
       slope[0][lane] = inv1r;
+    } else if (warp == 3 && lane == 0 && gi == g0 && scaled) {
+      scale_beams(sky);                            // (warp 0 reads the orbit only)
     }
     __syncthreads();
     // --- P (cycles to remove), a, b and their slopes along the grid
@@ -321,7 +323,7 @@ constexpr int kKnotThreads = 128;
 
 __global__ void __launch_bounds__(kKnotThreads)
 k_timemap_f32(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* __restrict__ meta,
-              KnotF* __restrict__ knots, int64_t knot_stride, int log2n_plan, int allow_ragged,
+              KnotF* __restrict__ knots, int64_t knot_stride, int log2n_plan, int allow_ragged, bool scaled,
               const int64_t* __restrict__ gaps, int64_t n_gaps_total, int* status, int64_t tmpl_base) {
   __shared__ KnotVal<float> kv[kKnotThreads];
   __shared__ double tb_sh[2];
@@ -336,7 +338,8 @@ k_timemap_f32(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* _
   const TmplGrid g = tmpl_grid(pc, tp, tb0, tb_sh[1], log2n_plan, allow_ragged, n_gaps_total);
   if (blockIdx.x == 0) write_meta(pc, tp, g, tb0, tmpl_base + t, meta + t, gaps, status);
   if (g.status != FSTAT_OK || j0 >= g.n_int) return;
-  const Sky<float> sky = make_sky<float>(pc, (float)tp.alpha, (float)tp.delta);
+  Sky<float> sky = make_sky<float>(pc, (float)tp.alpha, (float)tp.delta);
+  if (scaled) scale_beams(sky);
   const int64_t j = j0 + threadIdx.x;
   if (j <= g.n_int) kv[threadIdx.x] = knot_value<float>(pc, sky, tb0, j << pc.log2h, (float)tp.fdot, (float)tp.fddot);
   __syncthreads();
@@ -346,7 +349,9 @@ k_timemap_f32(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* _
 
 }  // namespace
 
-cudaError_t launch_timemap(const PlanConst& pc, const Chunk& c, int log2n_plan, int mode,
+// scaled: a, b times the powers of two of scale_beams, for the passes that only
+// form 2F from them
+cudaError_t launch_timemap(const PlanConst& pc, const Chunk& c, int log2n_plan, int mode, bool scaled,
                            const int64_t* gaps, int64_t n_gaps_total, int* status,
                            int64_t tmpl_base, cudaStream_t s) {
   const int64_t max_int = (((int64_t)1 << log2n_plan) >> pc.log2h) + 1;
@@ -354,7 +359,7 @@ cudaError_t launch_timemap(const PlanConst& pc, const Chunk& c, int log2n_plan, 
   if (pc.precision == FSTAT_PREC_FP32) {
     const dim3 grid((unsigned)((max_int + kKnotThreads - 2) / (kKnotThreads - 1)), (unsigned)c.nt);
     k_timemap_f32<<<grid, kKnotThreads, 0, s>>>(pc, c.tmpl, c.meta, (KnotF*)c.knots, c.knot_stride, log2n_plan,
-                                                ragged, gaps, n_gaps_total, status, tmpl_base);
+                                                ragged, scaled, gaps, n_gaps_total, status, tmpl_base);
     return cudaGetLastError();
   }
   // one group of knots per block while the blocks are few enough to be on the
@@ -364,10 +369,10 @@ cudaError_t launch_timemap(const PlanConst& pc, const Chunk& c, int log2n_plan, 
   const int groups = all * c.nt <= 8 * 152 ? 1 : 2;
   const dim3 grid((unsigned)((all + groups - 1) / groups), (unsigned)c.nt);
   if (pc.precision == FSTAT_PREC_FP64)
-    k_timemap<<<grid, kTmThreads, 0, s>>>(pc, c.tmpl, c.meta, (KnotD*)c.knots, c.knot_stride, log2n_plan, ragged, gaps,
+    k_timemap<<<grid, kTmThreads, 0, s>>>(pc, c.tmpl, c.meta, (KnotD*)c.knots, c.knot_stride, log2n_plan, ragged, scaled, gaps,
                                           n_gaps_total, status, tmpl_base, groups);
   else
-    k_timemap<<<grid, kTmThreads, 0, s>>>(pc, c.tmpl, c.meta, (KnotF*)c.knots, c.knot_stride, log2n_plan, ragged, gaps,
+    k_timemap<<<grid, kTmThreads, 0, s>>>(pc, c.tmpl, c.meta, (KnotF*)c.knots, c.knot_stride, log2n_plan, ragged, scaled, gaps,
                                           n_gaps_total, status, tmpl_base, groups);
   return cudaGetLastError();
 }

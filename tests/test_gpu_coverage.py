@@ -20,7 +20,7 @@ import synth
 from oracle import fstat as F
 from oracle import resample as R
 
-from _gpu import MODES, injected_series, oracle_two_f, r15, run_compute
+from _gpu import MODES, injected_series, oracle_two_f, r15, run_compute, tie_margin
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-4
@@ -287,3 +287,27 @@ def test_search_size_common_phase_invariance():
     assert rc == 0
     plan.close()
     assert r15(got, ref) <= 2e-6
+
+
+@pytest.mark.parametrize("prec,interp,taps", [(synth.PREC_MIXED, synth.SINC, 8), (synth.PREC_MIXED, synth.SINC, 4),
+                                              (synth.PREC_MIXED, synth.NEAREST, 8), (synth.PREC_FP64, synth.SINC, 8)])
+def test_small_beam_patterns_at_the_pole(prec, interp, taps):
+    """2F does not depend on the scale of a(t) or b(t) (B, C^2 and |Fb|^2 scale
+    alike in Eq. 6).  For a detector at the pole b is sin(delta) times a
+    function of order one, so a source near the equator has B and C as small as
+    one likes with D far from degenerate in proportion: as the oracle for every
+    delta, split and fused."""
+    det = synth.Detector(lat_rad=np.pi / 2)
+    d = synth.PlanDesc(dt=1.0, n_data=90_001, n_fft=1 << 17, interp=interp, taps=taps, f_het=20.0, precision=prec,
+                       det=det, max_templates=5)
+    deltas = [0.4, 1e-3, 1e-5, -1e-7, 1e-9]
+    tm = synth.make_templates([0.3, 1.0, 2.0, 4.0, 5.5], deltas, -1e-10, 0, d.n_data)
+    for t in tm:
+        while interp == synth.NEAREST and tie_margin(d, t) <= 1e-6:      # positions are held to ~1e-8
+            t["alpha"] += 0.01
+    x = synth.complex_noise(d.n_data, 1.0, synth.SEED_BASE + 198)
+    for mode in ("split", "fused"):
+        got, rc = run_compute(d, x, tm, mode=MODES[mode])
+        assert rc == 0
+        for i in range(5):
+            assert r15(got[i], oracle_two_f(d, x, tm[i])) <= TOL, (mode, deltas[i])
