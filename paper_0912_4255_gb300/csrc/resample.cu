@@ -146,7 +146,18 @@ __device__ __forceinline__ void add_sums(float pa, float pb, float pcc, TmplMeta
 
 // Other tap counts, FP64 (and knot intervals of fewer than 32 points): one point
 // per lane and row (32 consecutive points of a row at a time: one knot record
-// for all lanes, taps from one contiguous run of x).
+// for all lanes, taps from one contiguous run of x).  A tile's points start
+// below those at which the tile before ended; in a long gap list they are found
+// by binary search.  2000 gaps in 8 templates of 1,728,000 samples, FP32 with
+// knots 16 apart, took 2406 us when every tile walked the list from its
+// beginning, 1109 now.  Lists of up to 16 are walked; the search is out of line, so
+// that the registers are those of the loop without it (a cursor kept from tile to
+// tile: 4 taps, 16 templates of 2^20 points, 301 -> 324 us).
+constexpr int kGapsWalked = 16;
+__device__ __noinline__ void find_gap(GapCursor& gc, int j) { gc.seek(j); }
+__device__ __forceinline__ int knot_base(const KnotF& r) { return __ldg(&r.I); }
+__device__ __forceinline__ int knot_base(const KnotD& r) { return (int)floor(__ldg(&r.U)); }
+
 template <typename R, int INTERP, int TAPS>
 __global__ void __launch_bounds__(kTileThreads)
 k_resample_t(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* __restrict__ x,
@@ -174,7 +185,11 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* 
   for (int b = b0; b < b0 + per_warp && b < nlive; ++b) {
     const int c0 = (b & ((1 << (l2 - 5)) - 1)) << 5;
     const int r0 = (b >> (l2 - 5)) * kTileRows;
+    const int k0 = c0 + lane + (r0 << l2);
     GapCursor gc = make_cursor(m, gaps);      // the points of a new tile start lower
+    // u grows with k: the tile's samples lie above its first knot's, less the taps
+    if (gc.n > kGapsWalked && c0 + lane + (r0 << l2) < n_b)
+      find_gap(gc, knot_base(kn[(c0 + lane + (r0 << l2)) >> pc.log2h]) - 64);
 #pragma unroll 1
     for (int row = 0; row < kTileRows; ++row) {
       const int k = c0 + lane + ((r0 + row) << l2);

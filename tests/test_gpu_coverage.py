@@ -311,3 +311,26 @@ def test_small_beam_patterns_at_the_pole(prec, interp, taps):
         assert rc == 0
         for i in range(5):
             assert r15(got[i], oracle_two_f(d, x, tm[i])) <= TOL, (mode, deltas[i])
+
+
+@pytest.mark.parametrize("prec,taps,knot", [(synth.PREC_MIXED, 8, 4), (synth.PREC_MIXED, 4, 0), (synth.PREC_FP64, 8, 6),
+                                            (synth.PREC_FP64, 2, 6)])
+def test_many_gaps_point_by_point(prec, taps, knot):
+    """The resampler that takes one point a lane, with a thousand gaps of one to
+    40 samples, a few apart in places: its cursor is found by search and
+    taken from tile to tile.  The last template's span starts late and its list
+    starts at another offset.  Against the oracle (FP64 with knots 64 apart, where
+    the cubics between them are below 1e-7)."""
+    d = synth.PlanDesc(dt=0.5, n_data=300_001, n_fft=1 << 19, interp=synth.SINC, taps=taps, precision=prec, f_het=100.0,
+                       max_templates=2)
+    g = synth.rng(synth.SEED_BASE + 199)
+    edges = np.cumsum(g.integers(1, 41, 2000) + np.where(np.arange(2000) % 2, 0, g.choice([0, 300, 400], 2000)))
+    gaps = edges.reshape(-1, 2).astype(np.int64)
+    assert 250_000 < gaps[-1, 1] < d.n_data
+    tm = synth.make_templates([0.3, 2.0], [0.4, -0.7], -1e-9, [0, 150_001], [d.n_data, 140_000], [0, 400], [1000, 600])
+    x = synth.complex_noise(d.n_data, 1.0, synth.SEED_BASE + 200)
+    for mode in ("split", "fused"):
+        got, rc = run_compute(d, x, tm, gaps, mode=MODES[mode], tuning=dict(knot_log2=knot))
+        assert rc == 0
+        for i in range(2):
+            assert r15(got[i], oracle_two_f(d, x, tm[i], gaps)) <= (1e-6 if prec == synth.PREC_FP64 else TOL), (mode, i)
