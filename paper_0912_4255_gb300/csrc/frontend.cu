@@ -138,8 +138,82 @@ cudaError_t run_normalize(const float2* X, float2* Xh, int64_t n_sft, int K, int
   return cudaGetLastError();
 }
 
-// Step 2 on n_sft SFTs, by the window's places per lane.
+// The same for short windows: a thread takes a run of consecutive bins and keeps
+// its window sorted in a column of shared memory ([j][thread]), one removal and
+// one insertion a bin.  The same element of the same multiset, in the same order.
+__global__ void __launch_bounds__(kFeThreads)
+k_normalize_sorted(const float2* __restrict__ X, float2* __restrict__ Xh, int K, int w) {
+  extern __shared__ unsigned P[];
+  const float2* x = X + (int64_t)blockIdx.x * K;
+  float2* y = Xh + (int64_t)blockIdx.x * K;
+  for (int k = threadIdx.x; k < K; k += blockDim.x) {
+    const float2 v = x[k];
+    P[k] = __float_as_uint(v.x * v.x + v.y * v.y) & 0x7fffffffu;
+  }
+  __syncthreads();
+  const int h = w / 2;
+  const int run = (K + kFeThreads - 1) / kFeThreads;
+  const int k0 = threadIdx.x * run, k1 = min(K, k0 + run);
+  if (k0 >= k1) return;
+  unsigned* win = P + K + threadIdx.x;             // element j at win[j * kFeThreads]
+  int cnt = 0;
+  auto insert = [&](unsigned v) {
+    int j = cnt;
+    while (j > 0 && win[(j - 1) * kFeThreads] > v) { win[j * kFeThreads] = win[(j - 1) * kFeThreads]; --j; }
+    win[j * kFeThreads] = v;
+    ++cnt;
+  };
+  auto remove = [&](unsigned v) {
+    int j = 0;
+    while (j < cnt - 1 && win[j * kFeThreads] != v) ++j;
+    for (; j < cnt - 1; ++j) win[j * kFeThreads] = win[(j + 1) * kFeThreads];
+    --cnt;
+  };
+  for (int i = max(0, k0 - h); i < min(K, k0 + h + 1); ++i) insert(P[i]);
+  for (int k = k0; k < k1; ++k) {
+    if (k > k0) {
+      if (k - h - 1 >= 0) remove(P[k - h - 1]);
+      if (k + h < K) insert(P[k + h]);
+    }
+    const float med = __uint_as_float(win[((cnt - 1) / 2) * kFeThreads]);
+    const float sc = med > 0.f ? rsqrtf(med * 1.4426950408889634f) : 0.f;
+    const float2 v = x[k];
+    y[k] = make_float2(v.x * sc, v.y * sc);
+  }
+}
+
+size_t sorted_smem(int K, int w) { return ((size_t)K + (size_t)kFeThreads * (size_t)w) * sizeof(unsigned); }
+
+// Whether the sorted windows are faster, by the time of each in microseconds
+// (windows of 1 .. 61, bands of 200 .. 32000 bins, 1 .. 2000 SFTs, within 15 %
+// of the fits).  Sorted: a thread's first window costs the square of its length,
+// a bin its length, and shared memory limits the blocks that run at once.
+// Counts: a warp's runs of 64 bins one after another, 16 warps a block; a
+// second block on an SM already shares its issue slots.  (sorted | counts) 432
+// SFTs of 3648 bins, window 5 22 | 150, 31 74 | 148, 51 136 | 148, 61 307 | 148; 20 of 932
+// bins, window 5 9 | 19, 31 31 | 19.
+bool sorted_is_faster(int64_t n_sft, int K, int w) {
+  const size_t smem = sorted_smem(K, w);
+  if (w > 63 || smem > 200 * 1024) return false;
+  const int run = (K + kFeThreads - 1) / kFeThreads;
+  const size_t room = 228 * 1024 / (smem + 1024);
+  const int64_t at_once = 152 * (int64_t)(room < 8 ? room : 8);
+  const double waves = (double)((n_sft + at_once - 1) / at_once);
+  const double sorted = waves * (4.0 + 0.0185 * w * w + (run - 1) * (0.3 + 0.095 * w));
+  const double shared = 3.0 + 12.2 * (double)n_sft / 152.0;
+  const double counts = ((K + 1023) / 1024) * (shared > 16.0 ? shared : 16.0);
+  return 1.06 * sorted < counts;
+}
+
+// Step 2 on n_sft SFTs: sorted windows or, by the window's places per lane, counts.
 cudaError_t launch_normalize(const float2* X, float2* Xh, int64_t n_sft, int K, int w, cudaStream_t s) {
+  if (sorted_is_faster(n_sft, K, w)) {
+    static DeviceOnce once;
+    const cudaError_t e = kernel_setup(once, k_normalize_sorted, kFeThreads, (size_t)200 * 1024, nullptr);
+    if (e != cudaSuccess) return e;
+    k_normalize_sorted<<<(unsigned)n_sft, kFeThreads, sorted_smem(K, w), s>>>(X, Xh, K, w);
+    return cudaGetLastError();
+  }
   if (w <= 32 * 2) return run_normalize<2>(X, Xh, n_sft, K, w, s);
   if (w <= 32 * 4) return run_normalize<4>(X, Xh, n_sft, K, w, s);
   if (w <= 32 * 8) return run_normalize<8>(X, Xh, n_sft, K, w, s);

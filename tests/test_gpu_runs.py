@@ -247,3 +247,36 @@ def test_calls_one_after_another(n_t, l_fft, mode):
     torch.cuda.synchronize()
     assert all(torch.equal(o, a) for o, a in zip(outs, alone))
     plan.close()
+
+
+@pytest.mark.parametrize("n_sft,K", [(1, 200), (3, 932), (3, 3648), (320, 932), (3, 20000)])
+def test_running_median_of_short_windows(n_sft, K):
+    """Windows on both sides of the line between the two kernels, which moves
+    with the number of SFTs and the band: against the oracle; with a NaN, an
+    infinity and zeros in a row, every bin whose window has no NaN; a NaN counts
+    above every number in both kernels; in place."""
+    import torch
+    import paper_0912_4255_gb300 as fs
+    g = synth.rng(110 + K)
+    X = (g.normal(size=(3, K)) + 1j * g.normal(size=(3, K))).astype(np.complex64)
+    X[1] = np.round(X[1] * 2) / 2
+    bad = K // 3
+    X[2, bad] = np.nan
+    X[2, bad + 70 if K > 400 else 0] = np.inf
+    full = np.tile(X, ((n_sft + 2) // 3, 1))[:n_sft]
+    for w in (1, 3, 7, 15, 21, 23, 31, 35, 45, 51, 61, 63):
+        sd = synth.SftDesc(sft_len=8192, dt_raw=1.0 / 32, k_lo=0, n_bins=K, k_het=K // 2, band_bins=2, dirichlet_terms=0,
+                           median_window=w)
+        t = torch.from_numpy(full).cuda()
+        got = fs.fstat_sft_normalize(sd, t)
+        assert torch.equal(torch.nan_to_num(fs.fstat_sft_normalize(sd, t, out=t), 7.0), torch.nan_to_num(got, 7.0))
+        got = got.cpu().numpy()
+        for i in range(min(3, n_sft)):
+            with np.errstate(invalid="ignore", over="ignore", divide="ignore"):
+                p = np.abs(X[i].astype(np.complex128)) ** 2
+                med = np.array([np.sort(p[max(0, k - w // 2):k + w // 2 + 1])[(len(p[max(0, k - w // 2):k + w // 2 + 1]) - 1) // 2]
+                                for k in range(K)])                                # (NaN sorts last)
+                want = X[i] * np.where(med > 0, 1 / np.sqrt(med / np.log(2.0)), 0)
+            ok = np.isfinite(want)
+            assert ok.sum() >= K - 2 * w - 2 and np.abs(got[i] - want)[ok].max() < 2e-5 * np.abs(want[ok]).max(), (w, i)
+            assert np.array_equal(got[i::3], np.broadcast_to(got[i], got[i::3].shape), equal_nan=True)
