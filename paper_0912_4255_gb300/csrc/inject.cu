@@ -80,16 +80,18 @@ __device__ int check_injection(const PlanConst& pc, const fstat_injection& in, i
 // warp's FP64 instruction costs the same for one active lane as for 32.
 // Every thread then evaluates, interval by interval, one sample of each run
 // in FP32.  31 intervals have 32 knots, a warp's; where that leaves SMs idle
-// eight intervals shorten the chain: (8 | 31 | 64 intervals) 1 injection of
-// 200001 samples 17 | 27 | 41 us, 16 of them 25 | 27 | 41; 128 of 86401 76 | 49 |
-// 64, 256 of 20001 43 | 29 | 29, 256 of 200001 283 | 180 | 201.  The amplitudes'
-// coefficients are made once an interval and the phase factor by expm2pi
-// (128 of 86401 49 -> 47 us).  Bound by the FP64 set-up and, with many long
-// spans, by the atomic adds.
+// eight intervals shorten the chain: (at most 8 | 31 | 64 intervals) 1 injection of
+// 200001 samples 17 | 27 | 41 us; 128 of 86401 76 | 49 | 64, 256 of 200001 283 | 180 |
+// 201.  A span's intervals are spread evenly over its blocks: 128 injections of 32
+// intervals 33 us in blocks of 31 and 1, 25 in one of 64, 23 in two of 16.  The
+// amplitudes' coefficients are made once an interval, beside the phase factors,
+// and 64 registers let four blocks share an SM: 128 of 86401 44 -> 43 us, 64 of
+// 1,728,000 278 -> 260, 1 of 1000 12.9 -> 11.4.  Bound by the FP64 set-up and, with
+// many long spans, by the atomic adds.
 constexpr int kInjSeg = 31;
 constexpr int kInjSegFew = 8;
 
-__global__ void __launch_bounds__(kInjThreads)
+__global__ void __launch_bounds__(kInjThreads, 4)
 k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, int64_t max_span, int seg,
          float2* __restrict__ x, int* status) {
   __shared__ InjKnot kn[kInjSeg + 1];
@@ -127,6 +129,20 @@ k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, i
       cf[i][1] = (float)(c1 - (double)hi);
       cf[i][2] = (float)c2;
       cf[i][3] = (float)c3;
+    }
+    __syncthreads();
+    // the phase factor at the start of each run, from the FP64 phase; beside it, by
+    // other warps, the amplitudes' coefficients
+    static_assert(kInjSeg * kInjRuns <= kInjThreads / 2, "the first half of the block has a thread per run");
+    if ((int)threadIdx.x < n_int * kInjRuns) {
+      const int i = threadIdx.x / kInjRuns, r = threadIdx.x - i * kInjRuns;
+      const double u = (double)(r * kInjThreads);
+      const double base = pcoef[i][0] + u * (pcoef[i][1] + u * (pcoef[i][2] + u * pcoef[i][3]));
+      double sb, cb;
+      sincospi(2.0 * (base - floor(base)), &sb, &cb);
+      rot[i][r] = make_float2((float)cb, (float)sb);
+    }
+    if (const int i = (int)threadIdx.x - kInjThreads / 2; i >= 0 && i < n_int) {
       // F_+ = a cos 2 psi + b sin 2 psi, F_x = b cos 2 psi - a sin 2 psi
       double a[4] = {kn[i].a}, b[4] = {kn[i].b};
       hermite3(kn[i].a, kn[i].da, kn[i + 1].a, kn[i + 1].da, a + 1, a + 2, a + 3);
@@ -139,16 +155,6 @@ k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, i
         amp[i][j] = (float)(Ap * (a[j] * c2p + b[j] * s2p));
         amp[i][4 + j] = (float)(Ax * (b[j] * c2p - a[j] * s2p));
       }
-    }
-    __syncthreads();
-    // the phase factor at the start of each run, from the FP64 phase
-    for (int e = threadIdx.x; e < n_int * kInjRuns; e += kInjThreads) {
-      const int i = e / kInjRuns, r = e - i * kInjRuns;
-      const double u = (double)(r * kInjThreads);
-      const double base = pcoef[i][0] + u * (pcoef[i][1] + u * (pcoef[i][2] + u * pcoef[i][3]));
-      double sb, cb;
-      sincospi(2.0 * (base - floor(base)), &sb, &cb);
-      rot[i][r] = make_float2((float)cb, (float)sb);
     }
     __syncthreads();
     const int v = threadIdx.x;
@@ -185,9 +191,13 @@ k_inject(PlanConst pc, const fstat_injection* __restrict__ inj, int64_t n_inj, i
 
 cudaError_t launch_inject(const PlanConst& pc, const fstat_injection* inj, int64_t n_inj, int64_t max_span,
                           float2* x, int* status, cudaStream_t s) {
-  const auto blocks = [&](int seg) { return (max_span + (int64_t)seg * kInjH - 1) / ((int64_t)seg * kInjH); };
-  const int seg = n_inj <= 64 && n_inj * blocks(kInjSegFew) <= 3 * 152 ? kInjSegFew : kInjSeg;
-  const int64_t bx = blocks(seg);
+  // as many blocks a span as its intervals need at kInjSeg or kInjSegFew each, and
+  // the intervals spread evenly over them: a span of 32 in blocks of 31 and 1
+  // took as long as one of 62
+  const int64_t intervals = (max_span + kInjH - 1) >> kInjLog2H;
+  const auto blocks = [&](int seg) { return (intervals + seg - 1) / seg; };
+  const int64_t bx = blocks(n_inj <= 64 && n_inj * blocks(kInjSegFew) <= 3 * 152 ? kInjSegFew : kInjSeg);
+  const int seg = bx > 0 ? (int)((intervals + bx - 1) / bx) : 1;
   if (n_inj <= 0 || bx <= 0) return cudaSuccess;
   if (bx > 0x7fffffff) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)bx, (unsigned)(n_inj < 65535 ? n_inj : 65535));
