@@ -205,6 +205,77 @@ constexpr int kSample = 4;
 constexpr int kRefineAt = 512;
 constexpr int kRankAll = 128;      // so few are ranked as they are
 
+// The largest of the warp's candidates, in every lane.
+__device__ __forceinline__ unsigned long long warp_best(unsigned long long c) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(c >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(c >> 32) == hi ? (unsigned)c : 0u);
+  return ((unsigned long long)hi << 32) | lo;
+}
+
+// Few values of a short band: k <= 2 of up to four values a step, or k <= 4 of one
+// step, whose values the threads hold.  Every warp draws its k largest by rounds,
+// then one warp the block's: one barrier, where a bound, a buffer and ranks take
+// five.  In a graph (buffer | rounds): one band of 2048 at k = 1 2.7 | 1.7 us, k = 4
+// 2.8 | 2.3, 128 bands at k = 1 3.7 | 2.0, one of 8192 at k = 2 3.3 | 2.9.
+template <class F> bool few_of_short(int band_len, int k) {
+  const int n_steps = band_len / F::STEP;
+  return (k <= 2 && n_steps <= 4) || (k <= 4 && n_steps == 1);
+}
+
+template <class F>
+__global__ void __launch_bounds__(F::THREADS, F::MIN_BLOCKS)
+k_topk_short(const float* __restrict__ two_f, int64_t row_len, int band_len, int k, float* __restrict__ val,
+             int* __restrict__ bin) {
+  using Cand = unsigned long long;
+  __shared__ Cand lists[4][F::WARPS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int base = blockIdx.x * band_len;
+  const int64_t o = ((int64_t)blockIdx.y * (row_len / band_len) + blockIdx.x) * k;
+  const float4* src = reinterpret_cast<const float4*>(two_f + blockIdx.y * row_len + base) + threadIdx.x;
+  const int n_steps = band_len / F::STEP;
+  Cand c[4], d[4];                             // descending; no candidate is 0
+  const auto load = [&](Cand (&q)[4], float4 x, int u) {
+    const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      q[e] = fabsf(v[e]) < INFINITY ? pack(v[e], base + u * F::STEP + 4 * (int)threadIdx.x + e) : 0;
+  };
+  const auto down = [](Cand& x, Cand& y) {     // the larger of the two to x
+    const Cand hi = x > y ? x : y;
+    y = x > y ? y : x;
+    x = hi;
+  };
+  float4 xs[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) xs[u] = __ldg(src + (int64_t)(u < n_steps ? u : 0) * F::THREADS);
+  load(c, xs[0], 0);
+  down(c[0], c[1]); down(c[2], c[3]); down(c[0], c[2]); down(c[1], c[3]); down(c[1], c[2]);
+#pragma unroll
+  for (int u = 1; u < 4; ++u)
+    if (u < n_steps) {                         // two are enough
+      load(d, xs[u], u);
+      down(d[0], d[1]); down(d[2], d[3]); down(d[0], d[2]); down(d[1], d[2]);
+      down(c[0], d[0]); down(c[1], d[0]); down(c[1], d[1]);
+    }
+  for (int r = 0; r < k; ++r) {
+    const Cand w = warp_best(c[0]);
+    if (lane == 0) lists[r][warp] = w;
+    if (c[0] == w) { c[0] = c[1]; c[1] = c[2]; c[2] = c[3]; c[3] = 0; }
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  int p = 0;
+  c[0] = lane < F::WARPS ? lists[0][lane] : 0;
+  for (int r = 0; r < k; ++r) {
+    const Cand w = warp_best(c[0]);
+    if (lane == 0) {
+      val[o + r] = w ? packed_value(w) : -INFINITY;
+      bin[o + r] = w ? (int)~(unsigned)w : -1;
+    }
+    if (c[0] == w && w != 0) c[0] = ++p < k ? lists[p][lane] : 0;
+  }
+}
+
 template <class F>
 __global__ void __launch_bounds__(F::THREADS, F::MIN_BLOCKS)
 k_topk(const float* __restrict__ two_f, int64_t row_len, int band_len, int k, float* __restrict__ val,
@@ -314,7 +385,9 @@ extern "C" int fstat_topk(const float* twoF, int64_t n_rows, int64_t row_len, in
   // With no more bands than two to an SM, more threads and more loads in flight
   // for each (many | few): 16 bands of 262144 65 | 35 us, 256 of them 71 | 46, 256 of
   // 8192 12.4 | 10.3; 512 bands of 65536 31 | 34, 1024 of them 43 | 60.
-  if ((int64_t)grid.x * grid.y <= 2 * 152)
+  if ((int64_t)grid.x * grid.y <= 2 * 152 && few_of_short<TopFew>((int)band_len, k))
+    k_topk_short<TopFew><<<grid, TopFew::THREADS, 0, static_cast<cudaStream_t>(stream)>>>(twoF, row_len, (int)band_len, k, val, bin);
+  else if ((int64_t)grid.x * grid.y <= 2 * 152)
     k_topk<TopFew><<<grid, TopFew::THREADS, 0, static_cast<cudaStream_t>(stream)>>>(twoF, row_len, (int)band_len, k, val, bin);
   else
     k_topk<TopMany><<<grid, TopMany::THREADS, 0, static_cast<cudaStream_t>(stream)>>>(twoF, row_len, (int)band_len, k, val, bin);

@@ -153,3 +153,34 @@ def test_topk_sweeps_whose_buffer_fills_at_any_step(n_rows, k):
     for _ in range(4):
         v, b = _gpu_topk(a, n, k)
         assert np.array_equal(v.astype(np.float64), ov) and np.array_equal(b.astype(np.int64), ob)
+
+
+@pytest.mark.parametrize("n_rows,row_len,band_len,k", [(1, 2048, 2048, 4), (9, 2048, 2048, 2), (9, 6144, 2048, 3),
+                                                       (9, 4096, 4096, 2), (9, 12288, 6144, 1), (9, 8192, 8192, 2),
+                                                       (9, 10240, 10240, 2), (152, 4096, 2048, 4), (153, 4096, 2048, 4)])
+def test_topk_few_values_of_short_bands(n_rows, row_len, band_len, k):
+    """Both sides of the lines of the kernel that draws few values of short bands
+    by rounds: noise, all the loudest in one thread or one warp, equal values,
+    the two zeros, fewer finite values than asked for, none, infinities."""
+    g = synth.rng(77)
+    a = g.chisquare(4, size=(n_rows, row_len)).astype(np.float32)
+    for i in range(1, n_rows):
+        kind, at = i % 8, int(g.integers(0, row_len // 4)) * 4
+        if kind == 1:
+            a[i, at:at + 4] = [90.0, 91.0, 90.0, 92.0]
+        elif kind == 2:
+            a[i, at // 128 * 128:at // 128 * 128 + 128] += 50.0
+        elif kind == 3:
+            a[i] = 2.5
+        elif kind == 4:
+            a[i] = np.where(np.arange(row_len) % 2, -0.0, 0.0)
+        elif kind == 5:
+            a[i] = np.nan
+            a[i, at] = -3.0
+        elif kind == 6:
+            a[i] = -np.inf
+        elif kind == 7:
+            a[i, ::3] = np.inf
+    v, b = _gpu_topk(a, band_len, k)
+    ov, ob = CA.band_top_k(a.astype(np.float64), band_len, k)
+    assert np.array_equal(v.astype(np.float64), ov) and np.array_equal(b.astype(np.int64), ob)
