@@ -115,18 +115,22 @@ __device__ __forceinline__ void sincospi_half(float v, float* s, float* c) {
 // is sum_n (-d)^n c_n with c_n = sum_j X_j / y_j^(n+1), and what is left out is
 // below (2 spread / NEAR)^ORDER of a term: 2.4e-8 and 6e-8 in the forms below.
 // WARPS a block, PARTS of them share a segment (SFTs p, p + PARTS, ..).
+// ORDER 0: no expansions, every term one by one.
 template <int PL_, int NEAR_, int ORDER_, int WARPS_, int PARTS_> struct DemodForm {
-  static constexpr int PL = PL_, NEAR = NEAR_, ORDER = ORDER_, SEG = 32 * PL_;
+  static constexpr bool EXPANDS = ORDER_ > 0;
+  static constexpr int PL = PL_, SEG = 32 * PL_;
+  [[maybe_unused]] static constexpr int NEAR = NEAR_, ORDER = ORDER_;
   static constexpr int WARPS = WARPS_, PARTS = PARTS_, SEGS = WARPS_ / PARTS_, THREADS = 32 * WARPS_;
   static constexpr int TILE = THREADS / SEGS < 128 ? THREADS / SEGS : 128;   // SFTs at a time
-  static constexpr int MIN_BLOCKS = (NEAR_ == 2 ? 28 : 20) / WARPS_;
-  static constexpr float kSpread = NEAR_ == 2 ? 0.03f : 0.25f;
-  static constexpr int BITS = NEAR_ == 2 ? 41 : 36;      // of the step: below 2^31 with the spread
+  static constexpr int MIN_BLOCKS = (!EXPANDS ? (PARTS_ == 8 ? 32 : 40) : NEAR_ == 2 ? 28 : 20) / WARPS_;
+  [[maybe_unused]] static constexpr float kSpread = NEAR_ == 2 ? 0.03f : 0.25f;
+  [[maybe_unused]] static constexpr int BITS = NEAR_ == 2 ? 41 : 36;      // of the step: below 2^31 with the spread
 };
 template <int WARPS, int PARTS> struct DemodForms {
   using Fine = DemodForm<2, 2, 5, WARPS, PARTS>;
   using Mid = DemodForm<2, 4, 8, WARPS, PARTS>;
   using Wide = DemodForm<1, 4, 8, WARPS, PARTS>;
+  using Terms = DemodForm<1, 0, 0, WARPS, PARTS>;
 };
 
 template <class F> struct __align__(16) DemodFar {
@@ -208,7 +212,8 @@ __global__ void __launch_bounds__(F::THREADS, F::MIN_BLOCKS)
 k_demod(const DemodRec* __restrict__ rec, const float2* __restrict__ X, int n_sft, int K, int dk, int64_t n_q,
         float* __restrict__ out, int* status) {
   __shared__ DemodRec rs[F::TILE];
-  __shared__ DemodFar<F> far[F::TILE][F::SEGS];
+  using Far = std::conditional_t<F::EXPANDS, DemodFar<F>, int>;
+  __shared__ Far far[F::EXPANDS ? F::TILE : 1][F::SEGS];
   __shared__ float4 sum[F::SEGS][F::PARTS - 1][F::PL][32];
   __shared__ int bads[F::SEGS][F::PARTS - 1][F::PL][32];
   __shared__ double abc_sh[3][F::WARPS];
@@ -231,24 +236,25 @@ k_demod(const DemodRec* __restrict__ rec, const float2* __restrict__ X, int n_sf
       A += (double)r.a * (double)r.a; B += (double)r.b * (double)r.b; C += (double)r.a * (double)r.b;
     }
     __syncthreads();
-    {
+    if constexpr (F::EXPANDS) {
       const int i = threadIdx.x / F::SEGS, sg = threadIdx.x % F::SEGS;
       if (i < an)
         far[i][sg] = expand_far<F>(rs[i], X + (int64_t)(a0 + i) * K,
                                    ((long long)blockIdx.x * F::SEGS + sg) * F::SEG + F::SEG / 2, K, dk);
+      __syncthreads();
     }
-    __syncthreads();
     if (qs >= n_q) continue;
 #pragma unroll 1
     for (int i = part; i < an; i += F::PARTS) {
-      const DemodFar<F>& fm = far[i][seg];
-      const int mode = fm.mode;
+      const Far& fm = far[F::EXPANDS ? i : 0][seg];
+      int mode = FAR_NONE;
+      if constexpr (F::EXPANDS) mode = fm.mode;
       const float2* xs = X + (int64_t)(a0 + i) * K;
       float2 T[F::PL];
       float fr[F::PL];
       unsigned th[F::PL];                            // 2^-32 cycles
       float a, b;
-      if (mode != FAR_NONE) {
+      if constexpr (F::EXPANDS) if (mode != FAR_NONE) {
         const DemodFar<F> f = fm;
         a = f.a; b = f.b;
 #pragma unroll
@@ -285,7 +291,8 @@ k_demod(const DemodRec* __restrict__ rec, const float2* __restrict__ X, int n_sf
 #pragma unroll
           for (int n = 0; n < F::NEAR; ++n) add_term(T[u], f.x[n], y[n]);
         }
-      } else {
+      }
+      if (mode == FAR_NONE) {
         const DemodRec r = rs[i];
         a = r.a; b = r.b;
 #pragma unroll
@@ -313,7 +320,7 @@ k_demod(const DemodRec* __restrict__ rec, const float2* __restrict__ X, int n_sf
         float sc = sinpi_over_pi(fr[u]);
         if (fr[u] == 0.f) {
           sc = 1.f;
-          if (mode != FAR_NONE) {
+          if constexpr (F::EXPANDS) if (mode != FAR_NONE) {
             const int dq = lane + 32 * u - F::SEG / 2;
             T[u] = __ldg(xs + fm.k0 + (far_pos<F>(fm.rel, fm.drel, dq) >> 30));
           }
@@ -390,13 +397,20 @@ cudaError_t launch_demod(const PlanConst& pc, const fstat_sft_desc& d, const flo
   };
   // The step of kappa decides how far a segment reaches.  (The Doppler factor is
   // within 2e-4 of 1; the kernel checks each SFT's own step all the same and
-  // takes the terms one by one where it is wider, as in the last form with
-  // fewer than about 32 SFTs.)  4 templates x 32768 frequencies, expanded | one
+  // takes the terms one by one where it is wider.)  4 templates x 32768 frequencies,
+  // expanded | one
   // by one in the kernel before: 240 SFTs (Mid) 190 | 600 us, 48 (Wide) 68 | 140.
   const double step = fabs(df * t_len) * 1.0003;
+  // No SFT is expanded where the step is too wide for any form, or where the kernel
+  // has near terms only: a form without the expansions' registers and shared
+  // memory.  8 SFTs, 4 templates x 32768 frequencies, dk = 16: 55 us in the last form,
+  // 47 in this one; 240 SFTs, 4 x 16384, dk = 1: 139 | 90.
+  const bool any = fabs(df * t_len) * 0.9997 * (DemodForms<4, 2>::Wide::SEG / 2) <= DemodForms<4, 2>::Wide::kSpread &&
+                   d.dirichlet_terms > 1;
   const auto demod = [&](auto forms) {
     using L = decltype(forms);
-    if (step * (L::Fine::SEG / 2) <= L::Fine::kSpread) launch(typename L::Fine{});
+    if (!any) launch(typename L::Terms{});
+    else if (step * (L::Fine::SEG / 2) <= L::Fine::kSpread) launch(typename L::Fine{});
     else if (step * (L::Mid::SEG / 2) <= L::Mid::kSpread) launch(typename L::Mid{});
     else launch(typename L::Wide{});
   };
