@@ -91,7 +91,8 @@ __device__ __forceinline__ void add_term(float2& T, float2 x, float d) {
 
 // sin(pi f) / pi, f in [0, 1) a multiple of 2^-24 (1 - f is exact, so the
 // result is accurate relative to the distance from 0 and 1): polynomial in x^2
-// on [0, 1/2] fitted for the least relative error, 5.3e-9.
+// on [0, 1/2] fitted for the least relative error, 1.2e-8 with the coefficients as
+// written.
 __device__ __forceinline__ float sinpi_over_pi(float f) {
   const float x = fminf(f, 1.0f - f);
   const float u = x * x;
@@ -99,7 +100,7 @@ __device__ __forceinline__ float sinpi_over_pi(float f) {
 }
 
 // sin(pi v) and cos(pi v), |v| <= 1/2: the polynomial above times pi, and one
-// in v^2 with its value at 0 held at 1 (absolute error 2.4e-10).
+// in v^2 with its value at 0 held at 1 (absolute error 2.5e-8).
 __device__ __forceinline__ void sincospi_half(float v, float* s, float* c) {
   const float u = v * v;
   *s = v * fmaf(u, fmaf(u, fmaf(u, fmaf(u, 0.0775603876f, -0.598242104f), 2.55006981f), -5.16770983f), 3.14159274f);

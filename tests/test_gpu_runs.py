@@ -280,3 +280,80 @@ def test_running_median_of_short_windows(n_sft, K):
             ok = np.isfinite(want)
             assert ok.sum() >= K - 2 * w - 2 and np.abs(got[i] - want)[ok].max() < 2e-5 * np.abs(want[ok]).max(), (w, i)
             assert np.array_equal(got[i::3], np.broadcast_to(got[i], got[i::3].shape), equal_nan=True)
+
+
+def _orbit(speed):
+    return synth.Ephem(au_m=synth.Ephem.au_m * speed)
+
+
+@pytest.mark.parametrize("speed", [2.0, 4.2, 8.0])
+@pytest.mark.parametrize("kind", ["nearest", "rect", "lanczos"])
+def test_runs_on_a_faster_orbit(speed, kind):
+    """Beyond 1.25 times the Earth's speed the runs' weights keep their square in
+    the offset, beyond about 4.3 a run's offset leaves the expansion and its points
+    are taken one by one, at 4.2 both happen in one call: every bin against the
+    oracle, gaps included."""
+    d = synth.PlanDesc(dt=1.0, n_data=120_001, n_fft=1 << 17, f_het=50.0, eph=_orbit(speed), max_templates=2,
+                       interp=R.NEAREST if kind == "nearest" else R.SINC,
+                       window=R.WIN_RECT if kind == "rect" else R.WIN_LANCZOS)
+    gaps = np.array([[5000, 5003], [5010, 9000], [70_000, 70_001]], np.int64)
+    x, _ = injected_series(d, 121, [synth.random_injection(122, df=0.1)], gaps)
+    tm = _templates(d, [(0, d.n_data), (1001, 100_000)], len(gaps), 123, gap_free=False)
+    got, rc = run_compute(d, x, tm, gaps, mode=MODES["split"], tuning=dict(knot_log2=6))
+    assert rc == 0
+    for i in range(2):
+        assert r15(got[i], oracle_two_f(d, x, tm[i], gaps)) <= TOL, i
+
+
+@pytest.mark.parametrize("speed", [2.0, 4.2, 8.0])
+@pytest.mark.parametrize("window", [R.WIN_LANCZOS, R.WIN_RECT])
+def test_gradient_runs_on_a_faster_orbit(window, speed):
+    """The same for the gradient's runs, against the FP64 plan's gradient; the
+    tolerances of the test on the Earth's orbit."""
+    import torch
+    import paper_0912_4255_gb300 as fs
+    n, df = 90_001, 0.2
+    d = synth.PlanDesc(dt=1.0, n_data=n, n_fft=1 << 17, interp=R.SINC, window=window, f_het=50.0, eph=_orbit(speed),
+                       max_templates=2)
+    gaps = np.array([[9, 10], [40_000, 44_001]], np.int64)
+    inj = synth.random_injection(124, df=df)
+    x, _ = injected_series(d, 125, [inj], gaps)
+    tm = synth.make_templates([inj.alpha, inj.alpha + 1e-4], [inj.delta] * 2, [inj.fdot] * 2, [0, 77], [n, n - 1000], 0,
+                              len(gaps))
+    dev = torch.device("cuda:0")
+    out = []
+    for prec in (synth.PREC_MIXED, synth.PREC_FP64):
+        plan = fs.Plan(d.replace(precision=prec), device=dev)
+        plan.set_tuning(knot_log2=6)
+        y, g = fs.fstat_grad(plan, torch.from_numpy(x).to(dev), fs.pack_templates(tm, device=dev),
+                             torch.full((2,), df, dtype=torch.float64), torch.from_numpy(gaps.reshape(-1).copy()).to(dev))
+        assert fs.fstat_status(plan, raise_error=False) == 0
+        out.append((y.cpu().numpy(), g.cpu().numpy()))
+        plan.close()
+    (y, g), (y64, g64) = out
+    T = n * d.dt
+    scale = np.array([1e-3, 1e-3, 1.0 / T, 1.0 / T ** 2])
+    for i in range(2):
+        assert abs(y[i] - y64[i]) / max(y64[i], 4.0) < 1e-4, i
+        assert np.linalg.norm((g[i] - g64[i]) * scale) < 1e-3 * max(np.linalg.norm(g64[i] * scale),
+                                                                    1e-3 * max(y64[i], 4.0)), i
+
+
+@pytest.mark.parametrize("l_fft,l1,prec", [(12, 6, 0), (14, 8, 0), (18, 12, 0), (18, 6, 0), (20, 8, 0), (21, 9, 0), (21, 12, 0),
+                                           (22, 10, 0), (24, 12, 0), (12, 6, 1), (18, 12, 1), (18, 6, 1), (20, 10, 1)])
+def test_fft_shapes_without_ties(l_fft, l1, prec):
+    """The passes at their extreme shapes with the 8-tap sinc, which has no ties,
+    so that every bin is held to the path's tolerance; the intermediate by row
+    groups (split) and in place (fused)."""
+    n = 1 << l_fft
+    dt = max(0.5, 65536 / n)
+    d = synth.PlanDesc(dt=dt, n_data=n - n // 50 - 9, n_fft=n, f_het=20.0, max_templates=1, interp=R.SINC,
+                       precision=synth.PREC_FP64 if prec else synth.PREC_MIXED)
+    x = synth.complex_noise(d.n_data, 1.0, 130 + l_fft)
+    tm = synth.make_templates(0.4, 0.3, -1e-10, 0, d.n_data)
+    want = oracle_two_f(d, x, tm[0])
+    knot = 5 if dt > 2 else 7 if prec else 0
+    for mode in ("split", "fused"):
+        got, rc = run_compute(d, x, tm, mode=MODES[mode], tuning=dict(log2_n1=l1, knot_log2=knot))
+        assert rc == 0
+        assert r15(got[0], want) <= (1e-6 if prec else TOL), mode
