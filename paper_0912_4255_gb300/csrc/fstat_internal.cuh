@@ -51,7 +51,7 @@ struct PlanConst {
 constexpr int kSumBits = 36;
 
 // Per-template state produced by the time-map kernel and completed by the
-// first FFT pass (sums A, B, C and the 2F coefficients).
+// first FFT pass (sums A, B, C and the 2F coefficients).  One cache line.
 struct TmplMeta {
   double tb0;        // t_b of grid point 0
   double A, B, C;    // masked antenna sums (Eq. 9 as sums)
@@ -61,7 +61,6 @@ struct TmplMeta {
   int64_t n_b;       // resampled length N_b
   int64_t out_off;   // output offset in floats
   int64_t span_lo, span_hi, gap_off, n_gaps;
-  int32_t n_int;     // knot intervals
   int32_t log2n;     // FFT length of this template
   int32_t status;    // FSTAT_OK or the error of this template, as the time map found it
   // the same, or FSTAT_ERANGE where A, B, C give no 2F, for the second pass.  Not
@@ -71,6 +70,7 @@ struct TmplMeta {
   int32_t status_2f;
   float ca, cb, cc;  // 2F = ca |Fa|^2 + cb |Fb|^2 + cc Re(Fa Fb*)
 };
+static_assert(sizeof(TmplMeta) == 128, "the second pass reads one line of it before its tile");
 
 // Knot interval record, single precision evaluation (80 bytes).  On the
 // interval [k_j, k_j + h) with s = k - k_j:
@@ -291,6 +291,21 @@ __device__ __forceinline__ void scale_beams(Sky<R>& s) {
   const float kb = beam_scale(fabsf((float)s.f1) + fabsf((float)s.f2) + fabsf((float)s.f3) + fabsf((float)s.f4));
   s.e0 *= ka; s.e1 *= ka; s.e2 *= ka; s.e3 *= ka; s.e4 *= ka;
   s.f1 *= kb; s.f2 *= kb; s.f3 *= kb; s.f4 *= kb;
+}
+// The same by a warp, a coefficient a lane, on constants in shared memory: three
+// instructions of the FP64 pipe, which the time map's other warps wait for.
+__device__ __forceinline__ void scale_beams_warp(Sky<double>& s) {
+  static_assert(sizeof(Sky<double>) == 17 * sizeof(double), "e0 .. e4, f1 .. f4 are the last nine of 17");
+  const int lane = threadIdx.x & 31;
+  double* c = reinterpret_cast<double*>(&s) + 8 + (lane < 9 ? lane : 0);
+  const double v = *c;
+  float a = lane < 5 ? fabsf((float)v) : 0.f, b = lane >= 5 && lane < 9 ? fabsf((float)v) : 0.f;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  if (lane < 9) *c = v * (double)beam_scale(lane < 5 ? a : b);
 }
 
 // t_m(t) and dt_m/dt; sH, cH: sin and cos of the hour angle theta(t) - alpha.

@@ -168,7 +168,6 @@ __device__ __forceinline__ void write_meta(const PlanConst& pc, const fstat_temp
     m.span_hi = tp.span_start + tp.span_len;
     m.gap_off = tp.gap_off;
     m.n_gaps = tp.n_gaps;
-    m.n_int = st == FSTAT_OK ? g.n_int : 0;
     m.log2n = g.log2n;
     m.status = st;
     m.ca = m.cb = m.cc = 0.f;
@@ -272,8 +271,8 @@ k_timemap(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* __res
       geo[4][lane] = pc.dt * inv1r;
       val[0][lane] = (T1 + dT - pc.t_start) * pc.inv_dt;
       slope[0][lane] = inv1r;
-    } else if (warp == 3 && lane == 0 && gi == g0 && scaled) {
-      scale_beams(sky);                            // (warp 0 reads the orbit only)
+    } else if (warp == 3 && gi == g0 && scaled) {
+      scale_beams_warp(sky);                       // (warp 0 reads the orbit only)
     }
     __syncthreads();
     // --- P (cycles to remove), a, b and their slopes along the grid
