@@ -164,7 +164,8 @@ def algorithmic_per_template(desc, in_pass=False, l1=None):
     * 2F: 12 flop per bin.
     Design bytes, the HBM traffic the four-step design needs (N_d data
     samples ~ N_b grid points, N = n_fft):
-    * time map: an 80-byte knot record per 2^10 grid points;
+    * time map: an 80-byte knot record per 2^11 grid points (the default
+      spacing at 100 Hz and 2 Hz sampling);
     * resample: read x_h 8 N_d, write w_a, w_b 16 N_b;
     * first pass: read w_a, w_b 16 N_b, or x_h 8 N_d where it takes its own
       samples (in_pass: the persistent mode), write the intermediate 16 N;
@@ -180,7 +181,7 @@ def algorithmic_per_template(desc, in_pass=False, l1=None):
     fft_a = 2 * 5 * n * l1 + 2 * 6 * n
     res = nd * (taps * 9 + 16)
     rows = 2 * 5 * n * l2 + 12 * n
-    out = {"fft_rows": (rows, 16.0 * n + 4.0 * n), "timemap": (0.0, 80.0 * (n >> 10)), "sums": (0.0, 0.0),
+    out = {"fft_rows": (rows, 16.0 * n + 4.0 * n), "timemap": (0.0, 80.0 * (n >> 11)),
            "persistent": (fft_a + res + rows, 8.0 * nd + 32.0 * n + 4.0 * n)}
     if in_pass:
         out["fft_cols"] = (fft_a + res, 8.0 * nd + 16.0 * n)
@@ -385,7 +386,7 @@ def main():
     per_tpl = algorithmic_per_template(desc, in_pass=mode == fs.MODE_PERSISTENT,
                                        l1=plan.tuning()["log2_n1"])
     kernels = {}
-    for k in ("timemap", "resample", "fft_cols", "fft_rows", "persistent", "sums"):
+    for k in ("timemap", "resample", "fft_cols", "fft_rows", "persistent"):
         k_ms, k_n = prof[k]
         if not k_n:
             continue

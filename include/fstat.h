@@ -221,7 +221,9 @@ int fstat_template_nb(fstat_plan_t p, const fstat_template *host_t, int64_t n_t,
 /* Steps 1-5 only (debug/parity stage): writes the weighted series
  * wa = m a z e^{-2 pi i (f_h tau + fdot tau_b^2/2 + fddot tau_b^3/6)} and wb (complex64,
  * interleaved re/im, [n_t][n_fft], zero beyond N_b) and abcd[n_t][4] =
- * (A, B, C, D) in float64.  x_h: complex64 [n_data] (8-byte aligned);
+ * (A, B, C, D) in float64.  One point a thread; the series that fstat_compute
+ * transforms comes from tiled kernels and agrees with this one to the rounding
+ * of the plan's precision.  x_h: complex64 [n_data] (8-byte aligned);
  * templates: device [n_t]; gaps: device int64 [2 * n_gaps_total]. */
 int fstat_resample(fstat_plan_t p, const float *x_h, const fstat_template *templates,
                    int64_t n_t, const int64_t *gaps, int64_t n_gaps_total,
@@ -251,8 +253,9 @@ int fstat_grad(fstat_plan_t p, const float *x_h, const fstat_template *templates
  * 1 resample stage, 2 first FFT pass, 3 second FFT pass, 4 gradient
  * forward, 5 gradient adjoint, 6 persistent batch, 7 nothing any more: the
  * resample stage sums A, B, C), the summed device milliseconds and the
- * number of launches since the last read, then clears them.  Launch counts are kept whether or not timing is enabled.  ms and
- * launches are host arrays of n_kinds entries (n_kinds <= 8). */
+ * number of launches since the last read, then clears them.  Launch counts
+ * are kept whether or not timing is enabled.  ms and launches are host arrays
+ * of n_kinds entries (n_kinds <= 8). */
 int fstat_profile(fstat_plan_t p, int enable);
 int fstat_profile_read(fstat_plan_t p, double *ms, int64_t *launches, int n_kinds);
 

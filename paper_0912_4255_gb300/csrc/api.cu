@@ -16,7 +16,7 @@ using namespace fs;
 namespace {
 constexpr int kKinds = 8;
 enum { K_TIMEMAP = 0, K_RESAMPLE = 1, K_COLS = 2, K_ROWS = 3, K_GRADF = 4, K_GRADB = 5, K_PERSIST = 6,
-       K_SUMS = 7 };    // K_SUMS: no kernel of its own any more (pass A does it)
+       K_RESERVED = 7 };    // (was the reduction of A, B, C, which the resampler does now)
 }
 
 struct fstat_plan_s {

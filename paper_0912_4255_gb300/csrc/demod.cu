@@ -10,9 +10,12 @@
 //
 // The per-(template, SFT) quantities are computed once in FP64
 // (k_demod_setup); along the frequency grid f_q = f_0 + q df both kappa and
-// the phase are linear in q, so each thread steps them exactly in fixed
-// point: kappa - k_lo with 44 fractional bits, the phase as a 64-bit
-// fraction of a cycle.  The sum over SFTs and kernel terms is FP32.
+// the phase are linear in q.  They are laid down in 64-bit fixed point (kappa -
+// k_lo with 44 fractional bits, the phase as a fraction of a cycle) and taken
+// from there at every frequency where the terms are summed one by one, and at
+// the centre of a segment of 32 or 64 frequencies where the far terms are
+// expanded; inside a segment they are stepped in 32 bits (2^-30 bins, the step
+// to 2^-36 bins or finer; 2^-32 cycles).  The sum over SFTs and terms is FP32.
 #include "fstat_internal.cuh"
 
 #include <math.h>
@@ -399,8 +402,8 @@ cudaError_t launch_demod(const PlanConst& pc, const fstat_sft_desc& d, const flo
   // The step of kappa decides how far a segment reaches.  (The Doppler factor is
   // within 2e-4 of 1; the kernel checks each SFT's own step all the same and
   // takes the terms one by one where it is wider.)  4 templates x 32768 frequencies,
-  // expanded | one
-  // by one in the kernel before: 240 SFTs (Mid) 190 | 600 us, 48 (Wide) 68 | 140.
+  // expanded | one by one in every thread: 240 SFTs (Mid) 190 | 600 us, 48 (Wide)
+  // 68 | 140.
   const double step = fabs(df * t_len) * 1.0003;
   // No SFT is expanded where the step is too wide for any form, or where the kernel
   // has near terms only: a form without the expansions' registers and shared

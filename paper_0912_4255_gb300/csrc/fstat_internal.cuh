@@ -392,28 +392,28 @@ __device__ __forceinline__ void advance(R a, R d, R* s, R* c) {
 // rounding of T.  The orbital phase and hour angle at T0 and T are those at
 // tb rotated by small angles (|t_m| <= AU/c + R/c), so only tb needs full
 // sines and cosines.  Returns t_m(T), its rate and the hour-angle
-// sine/cosine at T, and 1 / (1 + dt_m/dt).
-template <typename R>
-__device__ __forceinline__ R inverse_time(const PlanConst& pc, const Sky<R>& s, R tb,
-                                          R* tm_out, R* rate_out, R* sH, R* cH, R* inv1r_out) {
-  const R wo = (R)pc.wo, ws = (R)pc.ws;
-  const R phi = (R)pc.orb0 + wo * tb, hh = (R)pc.th0 + ws * tb - s.alpha;
-  R sp, cp, st, ct;
-  rsincos<R>(phi, &sp, &cp);
-  rsincos<R>(hh, &st, &ct);
-  R tm = s.ox * cp + s.oy * sp + s.rxy * ct + s.rz;
+// sine/cosine at T, and 1 / (1 + dt_m/dt).  Used by the all-FP32 time map; the
+// FP64 one steps twice from the detector grid (timemap.cu).
+__device__ __forceinline__ float inverse_time(const PlanConst& pc, const Sky<float>& s, float tb, float* tm_out,
+                                              float* rate_out, float* sH, float* cH, float* inv1r_out) {
+  const float wo = (float)pc.wo, ws = (float)pc.ws;
+  const float phi = (float)pc.orb0 + wo * tb, hh = (float)pc.th0 + ws * tb - s.alpha;
+  float sp, cp, st, ct;
+  rsincos<float>(phi, &sp, &cp);
+  rsincos<float>(hh, &st, &ct);
+  float tm = s.ox * cp + s.oy * sp + s.rxy * ct + s.rz;
   // T0 = tb - tm: phases move by -w tm
-  const R d0 = -tm;
-  advance<R>(phi, wo * d0, &sp, &cp);
-  advance<R>(hh, ws * d0, &st, &ct);
-  const R T0 = tb + d0;
+  const float d0 = -tm;
+  advance<float>(phi, wo * d0, &sp, &cp);
+  advance<float>(hh, ws * d0, &st, &ct);
+  const float T0 = tb + d0;
   tm = s.ox * cp + s.oy * sp + s.rxy * ct + s.rz;
-  const R rate = wo * (s.oy * cp - s.ox * sp) - ws * s.rxy * st;
-  const R inv1r = 1 / (1 + rate);
-  const R dT = -(T0 + tm - tb) * inv1r;
+  const float rate = wo * (s.oy * cp - s.ox * sp) - ws * s.rxy * st;
+  const float inv1r = 1 / (1 + rate);
+  const float dT = -(T0 + tm - tb) * inv1r;
   *inv1r_out = inv1r;
   // the hour angle at T to first order in ws dT (|ws dT| <~ 4e-6)
-  const R e = ws * dT;
+  const float e = ws * dT;
   *sH = st + ct * e;
   *cH = ct - st * e;
   *tm_out = tm + rate * dT;
@@ -834,7 +834,9 @@ __device__ __forceinline__ bool sample_weights(
     if (!gc.valid(jnn)) { wa = czero<C>(); wb = czero<C>(); return false; }
     z = ldx<R>(x, jnn);
   } else {
-    const int taps = TAPS > 0 ? TAPS : pc.taps;
+    // (8 taps have a form of their own above)
+    static_assert(TAPS == 0, "the number of taps is the plan's");
+    const int taps = pc.taps;
     const int half = taps >> 1;
     // offset from the nearest sample, dn = u - jnn in [-1/2, 1/2]; every
     // weight is formed from sin/cos of pi dn and pi dn / H, so the tap next
@@ -850,7 +852,7 @@ __device__ __forceinline__ bool sample_weights(
     } else {
       // x = u - j = dn + mq with mq = jnn - j; sin(pi x) = (-1)^mq sin(pi dn);
       // sin(pi x / H) = sin(pi dn/H) cos(pi mq/H) + cos(pi dn/H) sin(pi mq/H)
-      constexpr int NTAP = TAPS > 0 ? TAPS : 16;
+      constexpr int NTAP = 16;
       // the common case: the whole window is valid data; the loads then go
       // out from one base pointer before any weight arithmetic
       const int jlo = n0 + 1 - half;
@@ -860,27 +862,21 @@ __device__ __forceinline__ bool sample_weights(
         const float2* xb = x + jlo;
 #pragma unroll
         for (int i = 0; i < NTAP; ++i) {
-          if (TAPS == 0 && i >= taps) break;
+          if (i >= taps) break;
           const float2 t2 = __ldg(xb + i);
           v[i] = cmk<C, R>((R)t2.x, (R)t2.y);
         }
       } else {
 #pragma unroll
         for (int i = 0; i < NTAP; ++i) {
-          if (TAPS == 0 && i >= taps) break;
+          if (i >= taps) break;
           int j = jlo + i;
           j = j < gc.lo ? gc.lo : (j >= gc.hi ? gc.hi - 1 : j);
           v[i] = ldx<R>(x, j);
         }
       }
       R S, Cd, sh, chh;
-      if constexpr (std::is_same<R, float>::value && TAPS == 8) {
-        // one polynomial at pi dn / 4, then two angle doublings
-        sincospi_small(0.25f * dn, &sh, &chh);
-        const float s2 = 2.0f * sh * chh, c2 = fmaf(chh, chh, -sh * sh);
-        S = 2.0f * s2 * c2;
-        Cd = fmaf(c2, c2, -s2 * s2);
-      } else if constexpr (std::is_same<R, float>::value) {
+      if constexpr (std::is_same<R, float>::value) {
         sincospif(dn, &S, &Cd);
         sincospif(dn / (R)half, &sh, &chh);
       } else {
@@ -891,8 +887,8 @@ __device__ __forceinline__ bool sample_weights(
       const bool lanczos = pc.window == FSTAT_WIN_LANCZOS;
       const R* wt = win_table<R>(wcs);
       // tap i sits at x = dn + mq with mq = (half - 1 - i) + qoff: dn is added
-      // to an exact small integer (a select between two constants), so the
-      // tap at the nearest sample keeps x = dn exactly;
+      // to an exact small integer, so the tap at the nearest sample keeps x = dn
+      // exactly;
       // (-1)^mq = (-1)^(half-1-i) (-1)^qoff: the qoff factor goes into Sp
       const R Sp = (qoff ? -S : S) * inv_pi2;
       C acc = czero<C>();
@@ -900,12 +896,10 @@ __device__ __forceinline__ bool sample_weights(
       [[maybe_unused]] R inv = (R)0, inv_next = (R)0;
 #pragma unroll
       for (int i = 0; i < NTAP; ++i) {
-        if (TAPS == 0 && i >= taps) break;
+        if (i >= taps) break;
         const int mq = half - 1 - i + qoff;       // jnn - j
         const int j = n0 + 1 - half + i;
-        R xx;
-        if constexpr (TAPS > 0) xx = dn + (qoff ? (R)(TAPS / 2 - i) : (R)(TAPS / 2 - 1 - i));
-        else xx = dn + (R)mq;
+        const R xx = dn + (R)mq;
         R w;
         if constexpr (std::is_same<R, float>::value) {
           w = __fdividef(Sp, xx * xx);
@@ -921,24 +915,9 @@ __device__ __forceinline__ bool sample_weights(
           }
           w = Sp * (inv * inv);
         }
-        if constexpr (TAPS > 0) {
-          if ((TAPS / 2 - 1 - i) & 1) w = -w;
-        } else {
-          if ((mq & 1) != qoff) w = -w;
-        }
+        if ((mq & 1) != qoff) w = -w;
         if (lanczos) {
-          R cm, sm;
-          if constexpr (TAPS == 8) {
-            // cos, sin(pi mq / 4) = cos, sin(2 pi (2 mq) / 16) with mq = 3 - i + qoff:
-            // two compile-time candidates per tap, chosen by qoff
-            const int m0 = (2 * (3 - i) + 32) & 15, m1 = (2 * (4 - i) + 32) & 15;
-            const R c0 = (R)c16(m0), c1v = (R)c16(m1), s0 = (R)s16(m0), s1v = (R)s16(m1);
-            cm = qoff ? c1v : c0;
-            sm = qoff ? s1v : s0;
-          } else {
-            cm = __ldg(wt + 2 * (mq + half));
-            sm = __ldg(wt + 2 * (mq + half) + 1);
-          }
+          const R cm = __ldg(wt + 2 * (mq + half)), sm = __ldg(wt + 2 * (mq + half) + 1);
           w *= (R)half * (sh * cm + chh * sm);
         } else {
           w *= (R)3.14159265358979323846 * xx;   // plain truncated sinc: sin(pi x)/(pi x)

@@ -567,7 +567,6 @@ __device__ __forceinline__ void for_slow_runs(bool slow_run, int k0, int g, F&& 
   }
 }
 
-template <bool LANCZOS>
 __device__ __noinline__ void fwd_slow(const GradArgs<float>& g, const KnotF* kn, int k, int n_b, GapCursor gc, int gi,
                                       unsigned long long fdt64, float c0f, float (&acc)[7]) {
   if (k >= n_b) return;
@@ -801,7 +800,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_grad_run(GradArgs<float> g)
       }
       for_slow_runs(live && !fast && !masked, r.k0, gc.g, [&](int k, int gi) {
         if constexpr (ADJ) adj_slow(g, kn, k, n_b, gc, gi, q, ct, fdt64, c0f, (float)dfd, acc);
-        else fwd_slow<LANCZOS>(g, kn, k, n_b, gc, gi, fdt64, c0f, acc);
+        else fwd_slow(g, kn, k, n_b, gc, gi, fdt64, c0f, acc);
       });
       __syncwarp();
       r = nx;

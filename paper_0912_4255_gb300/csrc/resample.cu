@@ -1,8 +1,9 @@
-// Steps 2-5 of Sec. III.A.2 as a stand-alone stage: one thread per point of
-// the barycentric grid writes the weighted series w_a, w_b (zero-padded to
-// the FFT length) and the block partial sums of A, B, C.  Used by
-// fstat_resample (parity/debug output) and by the unfused single-template
-// path, whose first FFT pass then loads these series from memory.
+// Steps 2-5 of Sec. III.A.2.  k_resample, one thread per point of the
+// barycentric grid, writes the weighted series w_a, w_b (zero-padded to the
+// FFT length) and the block partial sums of A, B, C for fstat_resample (parity
+// and debug output).  fstat_compute takes the tiled kernels below
+// (launch_resample_t), which leave both series in the first FFT pass's order
+// and agree with k_resample to the rounding of single precision.
 #include "passes.cuh"
 #include "sinc_run.cuh"
 
@@ -246,7 +247,8 @@ __device__ __noinline__ void slow_point(const PlanConst& pc, const KnotF* __rest
 // With the Lanczos window a slip of at most e = kRunNarrow needs no care: the
 // tap that it drops and the one that it adds sit where the kernel is e^2 / 16.
 //
-// The samples of a row (48 from the one before its first tap) are copied as
+// The samples of a row (44 from the one before its first tap: the last run's first
+// tap lies at 28 at most and a run takes 16) are copied as
 // 16-byte pieces into the warp's shared memory, a tile ahead (cp.async): read
 // straight from memory, the lanes' 64-byte stride cost 16 wavefronts a load.  Instruction issue
 // bounds the kernel (60 % of the cycles at 16 warps per SM, 128 registers; 96

@@ -1,7 +1,9 @@
-// fstat_selftest_math: evaluates the single-precision device math that the
-// resampler writes out by hand (step 4 of Sec. III.A.2 and the heterodyne
-// and spindown rotation of Eq. absorb), next to CUDA's own functions, so
-// that tests can bound each against exact values and against CUDA:
+// fstat_selftest_math: evaluates single-precision device math written out by
+// hand (step 4 of Sec. III.A.2 and the heterodyne and spindown rotation of Eq.
+// absorb), next to CUDA's own functions, so that tests can bound each against
+// exact values and against CUDA.  (Runs of eight points take their weights from
+// the tables of sinc_run.cuh instead of sinc8_f32, which is left for single
+// points; tests read those tables from the source.)
 //   sincospi_small  Taylor series of sin, cos (pi x), |x| <= 1/4;
 //   expm2pi         exp(-2 pi i r), |r| <= 1/2, by exact quarter turns;
 //   sinc8_f32       the 8-tap windowed sinc (Lanczos or plain truncation)

@@ -19,28 +19,26 @@ namespace fs {
 
 namespace {
 
-// Values at one knot, in FP64 (or FP32 for the precision study).
-template <typename R>
+// Values at one knot in FP32 (the precision study).
 struct KnotVal {
-  R U, dU, P, dP, a, da, b, db;
+  float U, dU, P, dP, a, da, b, db;
 };
 
-template <typename R>
-__device__ KnotVal<R> knot_value(const PlanConst& pc, const Sky<R>& sky, double tb0, int64_t k, R fdot,
-                                 R fddot) {
-  KnotVal<R> v;
-  const R tb = (R)(tb0 + (double)k * pc.dt);
-  R tm, rate, sH, cH, inv1r;
-  const R T = inverse_time<R>(pc, sky, tb, &tm, &rate, &sH, &cH, &inv1r);
-  const R dTdk = (R)pc.dt * inv1r;
-  v.U = (T - (R)pc.t_start) * (R)pc.inv_dt;
+__device__ KnotVal knot_value(const PlanConst& pc, const Sky<float>& sky, double tb0, int64_t k, float fdot,
+                              float fddot) {
+  KnotVal v;
+  const float tb = (float)(tb0 + (double)k * pc.dt);
+  float tm, rate, sH, cH, inv1r;
+  const float T = inverse_time(pc, sky, tb, &tm, &rate, &sH, &cH, &inv1r);
+  const float dTdk = (float)pc.dt * inv1r;
+  v.U = (T - (float)pc.t_start) * (float)pc.inv_dt;
   v.dU = inv1r;
-  const R taub = tb - (R)pc.t_start;
+  const float taub = tb - (float)pc.t_start;
   // spindown phase of Eq. 4 to s = 2 in barycentric time, and its rate
-  v.P = (R)pc.f_het * tm + taub * taub * ((R)0.5 * fdot + fddot * taub * (R)(1.0 / 6));
-  v.dP = (R)pc.f_het * rate * dTdk + taub * (fdot + (R)0.5 * fddot * taub) * (R)pc.dt;
-  R a, b, da, db;
-  beams_h<R>(pc, sky, sH, cH, &a, &b, &da, &db);
+  v.P = (float)pc.f_het * tm + taub * taub * ((float)0.5 * fdot + fddot * taub * (float)(1.0 / 6));
+  v.dP = (float)pc.f_het * rate * dTdk + taub * (fdot + (float)0.5 * fddot * taub) * (float)pc.dt;
+  float a, b, da, db;
+  beams_h<float>(pc, sky, sH, cH, &a, &b, &da, &db);
   v.a = a; v.b = b; v.da = da * dTdk; v.db = db * dTdk;
   return v;
 }
@@ -56,7 +54,7 @@ __device__ __forceinline__ void hermite(R f0, R d0, R f1, R d1, R H, R iH, R* c1
 }
 
 // FP32 time map (precision study): the same record built from FP32 values.
-__device__ __forceinline__ void write_record(KnotF* out, const KnotVal<float>& k0, const KnotVal<float>& k1, float H) {
+__device__ __forceinline__ void write_record(KnotF* out, const KnotVal& k0, const KnotVal& k1, float H) {
   KnotF r;
   const float iH = (float)1 / H;
   float c1, c2, c3;
@@ -324,7 +322,7 @@ __global__ void __launch_bounds__(kKnotThreads)
 k_timemap_f32(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* __restrict__ meta,
               KnotF* __restrict__ knots, int64_t knot_stride, int log2n_plan, int allow_ragged, bool scaled,
               const int64_t* __restrict__ gaps, int64_t n_gaps_total, int* status, int64_t tmpl_base) {
-  __shared__ KnotVal<float> kv[kKnotThreads];
+  __shared__ KnotVal kv[kKnotThreads];
   __shared__ double tb_sh[2];
   let_next_start();
   const int t = blockIdx.y;
@@ -340,7 +338,7 @@ k_timemap_f32(PlanConst pc, const fstat_template* __restrict__ tmpl, TmplMeta* _
   Sky<float> sky = make_sky<float>(pc, (float)tp.alpha, (float)tp.delta);
   if (scaled) scale_beams(sky);
   const int64_t j = j0 + threadIdx.x;
-  if (j <= g.n_int) kv[threadIdx.x] = knot_value<float>(pc, sky, tb0, j << pc.log2h, (float)tp.fdot, (float)tp.fddot);
+  if (j <= g.n_int) kv[threadIdx.x] = knot_value(pc, sky, tb0, j << pc.log2h, (float)tp.fdot, (float)tp.fddot);
   __syncthreads();
   if (threadIdx.x < kKnotThreads - 1 && j < g.n_int)
     write_record(knots + (int64_t)t * knot_stride + j, kv[threadIdx.x], kv[threadIdx.x + 1], (float)(1 << pc.log2h));
