@@ -419,7 +419,7 @@ int fstat_compute(fstat_plan_t p, const float* x_h, const fstat_template* t, int
     const int inplace = p->tune.mode == FSTAT_MODE_FUSED;
     if (inplace) c.wa = c.za;
     cudaError_t e = timed(p, K_TIMEMAP, s, [&] { return launch_timemap(p->pc, c, p->log2n, p->tune.mode, true, gaps, n_gaps_total, p->status, t0, s); });
-    if (e == cudaSuccess) e = timed(p, K_RESAMPLE, s, [&] { return launch_resample_t(p->pc, c, p->sh, x, gaps, p->wcs, s); });
+    if (e == cudaSuccess) e = timed(p, K_RESAMPLE, s, [&] { return launch_resample_t(p->pc, c, p->sh, x, gaps, n_gaps_total, p->wcs, s); });
     if (e == cudaSuccess) e = timed(p, K_COLS, s, [&] { return launch_cols_w(p->pc, c, p->sh, inplace, &p->twf, &p->twd, p->status, s); });
     if (e == cudaSuccess) e = timed(p, K_ROWS, s, [&] { return launch_rows_w(p->pc, c, p->sh, inplace, &p->twf, &p->twd, twoF, s); });
     if (e != cudaSuccess) return FSTAT_ECUDA;

@@ -1266,7 +1266,7 @@ cudaError_t launch_resample_w(const PlanConst& pc, const Chunk& c, int ti, int l
                               int64_t out_stride, int out_double, double* abcd, int* status,
                               cudaStream_t s);
 cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& sh, const float2* x,
-                              const int64_t* gaps, const double* wcs, cudaStream_t s);
+                              const int64_t* gaps, int64_t n_gaps_total, const double* wcs, cudaStream_t s);
 int resample_covered(const PlanConst& pc, const Shape& sh);
 cudaError_t launch_cols_w(const PlanConst& pc, const Chunk& c, const Shape& sh, int inplace, const void* twf,
                           const void* twd, int* status, cudaStream_t s);

@@ -242,7 +242,7 @@ extern "C" int fstat_compute_noalloc(const fstat_plan_desc* d, const float* x_h,
     c.wa = c.za;              // the resampled series, transformed in place by pass A
     c.nt = 1;
     cudaError_t e = launch_timemap(pc, c, L, FSTAT_MODE_FUSED, true, gaps, n_gaps_total, status, t, s);
-    if (e == cudaSuccess) e = launch_resample_t(pc, c, sh, x, gaps, wcs, s);
+    if (e == cudaSuccess) e = launch_resample_t(pc, c, sh, x, gaps, n_gaps_total, wcs, s);
     if (e == cudaSuccess) e = launch_cols_w(pc, c, sh, 1, &twf, &twd, status, s);
     if (e == cudaSuccess) e = launch_rows_w(pc, c, sh, 1, &twf, &twd, twoF, s);
     if (e != cudaSuccess) return FSTAT_ECUDA;

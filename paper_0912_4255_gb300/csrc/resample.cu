@@ -151,15 +151,15 @@ __device__ __forceinline__ void add_sums(float pa, float pb, float pcc, TmplMeta
 // below those at which the tile before ended; in a long gap list they are found
 // by binary search.  2000 gaps in 8 templates of 1,728,000 samples, FP32 with
 // knots 16 apart, took 2406 us when every tile walked the list from its
-// beginning, 1109 now.  Lists of up to 16 are walked; the search is out of line, so
-// that the registers are those of the loop without it (a cursor kept from tile to
-// tile: 4 taps, 16 templates of 2^20 points, 301 -> 324 us).
+// beginning, 1100 now.  Lists of up to 16 are walked; a call without longer ones
+// takes the form without the search, which costs registers (one template of 2^20
+// points, 16 taps, 54 -> 59 us).
 constexpr int kGapsWalked = 16;
 __device__ __noinline__ void find_gap(GapCursor& gc, int j) { gc.seek(j); }
 __device__ __forceinline__ int knot_base(const KnotF& r) { return __ldg(&r.I); }
 __device__ __forceinline__ int knot_base(const KnotD& r) { return (int)floor(__ldg(&r.U)); }
 
-template <typename R, int INTERP, int TAPS>
+template <typename R, int INTERP, int TAPS, bool SEARCH>
 __global__ void __launch_bounds__(kTileThreads)
 k_resample_t(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* __restrict__ x,
              const int64_t* __restrict__ gaps, const double* __restrict__ wcs) {
@@ -189,8 +189,10 @@ k_resample_t(PlanConst pc, Chunk c, int l2, int lc, int per_warp, const float2* 
     const int k0 = c0 + lane + (r0 << l2);
     GapCursor gc = make_cursor(m, gaps);      // the points of a new tile start lower
     // u grows with k: the tile's samples lie above its first knot's, less the taps
-    if (gc.n > kGapsWalked && c0 + lane + (r0 << l2) < n_b)
-      find_gap(gc, knot_base(kn[(c0 + lane + (r0 << l2)) >> pc.log2h]) - 64);
+    if constexpr (SEARCH) {
+      if (gc.n > kGapsWalked && c0 + lane + (r0 << l2) < n_b)
+        find_gap(gc, knot_base(kn[(c0 + lane + (r0 << l2)) >> pc.log2h]) - 64);
+    }
 #pragma unroll 1
     for (int row = 0; row < kTileRows; ++row) {
       const int k = c0 + lane + ((r0 + row) << l2);
@@ -550,7 +552,7 @@ TileGrid tile_grid(const PlanConst& pc, const Shape& sh, int nt) {
 }  // namespace
 
 cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& sh, const float2* x,
-                              const int64_t* gaps, const double* wcs, cudaStream_t s) {
+                              const int64_t* gaps, int64_t n_gaps_total, const double* wcs, cudaStream_t s) {
   const int lc = log2_cols(sh);
   const TileGrid tg = tile_grid(pc, sh, c.nt);
   if (tg.blocks == 0) return cudaSuccess;
@@ -561,16 +563,25 @@ cudaError_t launch_resample_t(const PlanConst& pc, const Chunk& c, const Shape& 
   auto go = [&](auto kern) {
     e = launch_after(early, kern, grid, kTileThreads, 0, s, pc, c, sh.l2, lc, tg.per_warp, x, gaps, wcs);
   };
-  if (pc.precision == FSTAT_PREC_FP64) {
-    if (pc.interp == FSTAT_NEAREST) go(k_resample_t<double, FSTAT_NEAREST, 8>);
-    else if (pc.taps == 8) go(k_resample_t<double, FSTAT_SINC, 8>);
-    else go(k_resample_t<double, FSTAT_SINC, 0>);
-  } else if (pc.interp == FSTAT_SINC && pc.taps != 8) {
-    go(k_resample_t<float, FSTAT_SINC, 0>);
-  } else if (pc.log2h < 5) {
-    // knot intervals shorter than a tile's 32 columns
-    if (pc.interp == FSTAT_NEAREST) go(k_resample_t<float, FSTAT_NEAREST, 8>);
-    else go(k_resample_t<float, FSTAT_SINC, 8>);
+  const auto points_of = [&](auto search) {
+    constexpr bool S = decltype(search)::value;
+    if (pc.precision == FSTAT_PREC_FP64) {
+      if (pc.interp == FSTAT_NEAREST) go(k_resample_t<double, FSTAT_NEAREST, 8, S>);
+      else if (pc.taps == 8) go(k_resample_t<double, FSTAT_SINC, 8, S>);
+      else go(k_resample_t<double, FSTAT_SINC, 0, S>);
+    } else if (pc.interp == FSTAT_NEAREST) {
+      go(k_resample_t<float, FSTAT_NEAREST, 8, S>);
+    } else if (pc.taps == 8) {
+      go(k_resample_t<float, FSTAT_SINC, 8, S>);
+    } else {
+      go(k_resample_t<float, FSTAT_SINC, 0, S>);
+    }
+  };
+  // point by point: FP64, other tap counts, and knot intervals shorter than a
+  // tile's 32 columns
+  if (pc.precision == FSTAT_PREC_FP64 || (pc.interp == FSTAT_SINC && pc.taps != 8) || pc.log2h < 5) {
+    if (n_gaps_total > kGapsWalked) points_of(std::true_type{});
+    else points_of(std::false_type{});
   } else {
     const bool quad = runs_need_square(pc);
     if (pc.interp == FSTAT_NEAREST) {
