@@ -273,9 +273,9 @@ __device__ __forceinline__ Sky<R> make_sky(const PlanConst& pc, R alpha, R delta
 }
 
 // 2^-e with 2^e above the sum of the amplitudes, the bound of a pattern at any
-// hour angle (a pattern whose squares FP32 cannot hold is left as it is)
+// hour angle (a pattern below what FP32 holds is left as it is)
 __device__ __forceinline__ float beam_scale(float amplitudes) {
-  return amplitudes > 1e-18f && amplitudes < 1e18f ? __int_as_float((253 << 23) - (__float_as_int(amplitudes) & 0x7f800000))
+  return amplitudes > 1e-37f && amplitudes < 1e37f ? __int_as_float((253 << 23) - (__float_as_int(amplitudes) & 0x7f800000))
                                                    : 1.0f;
 }
 
