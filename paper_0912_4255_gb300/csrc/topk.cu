@@ -22,6 +22,8 @@
 // threads' maxima of the first 1024 values give the bound, and the buffer is
 // merged with the running list by a bitonic sort, which raises the bound to the
 // list's k-th value.
+//
+// Few values of short bands are drawn by rounds instead (k_topk_short).
 #include "fstat_internal.cuh"
 
 #include <climits>
