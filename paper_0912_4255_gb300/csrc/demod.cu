@@ -126,7 +126,7 @@ template <int PL_, int NEAR_, int ORDER_, int WARPS_, int PARTS_> struct DemodFo
   [[maybe_unused]] static constexpr int NEAR = NEAR_, ORDER = ORDER_;
   static constexpr int WARPS = WARPS_, PARTS = PARTS_, SEGS = WARPS_ / PARTS_, THREADS = 32 * WARPS_;
   static constexpr int TILE = THREADS / SEGS < 128 ? THREADS / SEGS : 128;   // SFTs at a time
-  static constexpr int MIN_BLOCKS = (!EXPANDS ? (PARTS_ == 8 ? 32 : 40) : NEAR_ == 2 ? 28 : 20) / WARPS_;
+  static constexpr int MIN_BLOCKS = (!EXPANDS && PARTS_ == 8 ? 32 : NEAR_ == 2 ? 28 : 20) / WARPS_;
   [[maybe_unused]] static constexpr float kSpread = NEAR_ == 2 ? 0.03f : 0.25f;
   [[maybe_unused]] static constexpr int BITS = NEAR_ == 2 ? 41 : 36;      // of the step: below 2^31 with the spread
 };
@@ -408,7 +408,8 @@ cudaError_t launch_demod(const PlanConst& pc, const fstat_sft_desc& d, const flo
   // No SFT is expanded where the step is too wide for any form, or where the kernel
   // has near terms only: a form without the expansions' registers and shared
   // memory.  8 SFTs, 4 templates x 32768 frequencies, dk = 16: 55 us in the last form,
-  // 47 in this one; 240 SFTs, 4 x 16384, dk = 1: 139 | 90.
+  // 45 in this one; 240 SFTs, 4 x 16384, dk = 1: 139 | 84.  (In 48 registers 47 and 90, and
+  // 16 SFTs, 4 x 8192, 37 where both others take 33 to 35.)
   const bool any = fabs(df * t_len) * 0.9997 * (DemodForms<4, 2>::Wide::SEG / 2) <= DemodForms<4, 2>::Wide::kSpread &&
                    d.dirichlet_terms > 1;
   const auto demod = [&](auto forms) {
